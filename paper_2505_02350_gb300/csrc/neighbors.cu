@@ -13,8 +13,8 @@ using namespace serbf;
 
 namespace {
 
-// Per-kernel records.  kfwd: (c, r2), (Q11, Q22, Q33, a), (2Q12, 2Q13, 2Q23, 0)
-// with Q = log2(e) R^T D^2 R, so that exp(-||D R (v - c)||^2) = 2^(-dv^T Q dv);
+// Per-kernel records.  kfwd: (c, r2), (Q11, Q22, Q33, a), (2Q12, 2Q13, 2Q23, l)
+// with l the root of Q's largest eigenvalue and Q = log2(e) R^T D^2 R, so that exp(-||D R (v - c)||^2) = 2^(-dv^T Q dv);
 // kbwd: (c, r2) and the rows of R with e_k = log2(e) d_k^2 in .w.
 // R is the App. A matrix (entries r1..r9).
 __device__ __forceinline__ void prep_kernels(const float *p, int cap, int m, float nle, float4 *kfwd, float4 *kbwd,
@@ -46,7 +46,8 @@ __device__ __forceinline__ void prep_kernels(const float *p, int cap, int m, flo
         float aw = w * fabsf(w);
         kfwd[3 * j + 0] = make_float4(cx, cy, cz, r2);
         kfwd[3 * j + 1] = make_float4(Q[0][0], Q[1][1], Q[2][2], aw);
-        kfwd[3 * j + 2] = make_float4(2.f * Q[0][1], 2.f * Q[0][2], 2.f * Q[1][2], 0.f);
+        kfwd[3 * j + 2] = make_float4(2.f * Q[0][1], 2.f * Q[0][2], 2.f * Q[1][2],
+                                      sqrtf(fmaxf(e[0], fmaxf(e[1], e[2]))));
         kbwd[4 * j + 0] = make_float4(cx, cy, cz, r2);
         kbwd[4 * j + 1] = make_float4(R[0], R[1], R[2], e[0]);
         kbwd[4 * j + 2] = make_float4(R[3], R[4], R[5], e[1]);
