@@ -198,9 +198,9 @@ __device__ __forceinline__ bool in_support(float px, float py, float pz, float c
 // each argument), hence box_d2 < r2 is a superset of the membership test for
 // points in the box.
 __device__ __forceinline__ float box_d2(float cx, float cy, float cz, float4 lo, float4 hi) {
-    float ax = cx < lo.x ? __fsub_rn(lo.x, cx) : (cx > hi.x ? __fsub_rn(cx, hi.x) : 0.f);
-    float ay = cy < lo.y ? __fsub_rn(lo.y, cy) : (cy > hi.y ? __fsub_rn(cy, hi.y) : 0.f);
-    float az = cz < lo.z ? __fsub_rn(lo.z, cz) : (cz > hi.z ? __fsub_rn(cz, hi.z) : 0.f);
+    const float ax = fmaxf(fmaxf(__fsub_rn(lo.x, cx), __fsub_rn(cx, hi.x)), 0.f);
+    const float ay = fmaxf(fmaxf(__fsub_rn(lo.y, cy), __fsub_rn(cy, hi.y)), 0.f);
+    const float az = fmaxf(fmaxf(__fsub_rn(lo.z, cz), __fsub_rn(cz, hi.z)), 0.f);
     return support_d2(ax, ay, az);
 }
 
