@@ -185,6 +185,11 @@ __device__ __forceinline__ uint32_t redux_add(uint32_t v) {
     asm volatile("redux.sync.add.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
     return r;
 }
+__device__ __forceinline__ uint32_t redux_max_u32(uint32_t v) {
+    uint32_t r;
+    asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
+    return r;
+}
 __device__ __forceinline__ float redux_min(float v) {
     float r;
     asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
@@ -233,27 +238,25 @@ __device__ __forceinline__ FwdGPart reduce_parts(const P *p, uint32_t b, uint32_
 
 // Loss terms of one tile, stored as the tile's partial (lane order within the
 // tile).  The partials are reduced in tile order after the launch, so the
-// totals do not depend on which warp handled which tile.  Returns max|E|.
-__device__ __forceinline__ float finish_tile(const FwdArgs &a, uint32_t t, float l2, float mx_l, uint32_t cnt_l,
-                                             uint32_t pairs_l, int lane) {
+// totals do not depend on which warp handled which tile. 
+__device__ __forceinline__ void finish_tile(const FwdArgs &a, uint32_t t, float l2, float mx_l, uint32_t cnt_l,
+                                            uint32_t pairs_l, int lane) {
     const ff l2s = warp_sum_ff(ff{l2, 0.f});
     const float mx = redux_max(mx_l);
     const uint32_t cnt = redux_add(cnt_l), pr = redux_add(pairs_l);
     if (lane == 0) a.part[t] = FwdPart{l2s.hi, l2s.lo, mx, cnt, (unsigned long long)pr};
-    return mx;
 }
 
 // Loss terms of both tiles of an item in one reduction (a lane's two squares
 // are added exactly first), stored as the first tile's partial; the second
 // tile's is zero.
-__device__ __forceinline__ float finish_item(const FwdArgs &a, uint32_t t, bool two, ff l2, float mx_l, uint32_t cnt_l,
-                                             uint32_t pairs_l, int lane) {
+__device__ __forceinline__ void finish_item(const FwdArgs &a, uint32_t t, bool two, ff l2, float mx_l, uint32_t cnt_l,
+                                            uint32_t pairs_l, int lane) {
     const ff l2s = warp_sum_ff(l2);
     const float mx = redux_max(mx_l);
     const uint32_t cnt = redux_add(cnt_l), pr = redux_add(pairs_l);
     if (lane == 0) a.part[t] = FwdPart{l2s.hi, l2s.lo, mx, cnt, (unsigned long long)pr};
     if (lane == 1 && two) a.part[t + 1] = FwdPart{0.f, 0.f, 0.f, 0u, 0ull};
-    return mx;
 }
 
 // Eq. 3-18 filter and residual of one point; returns its loss contributions.
@@ -613,7 +616,9 @@ __device__ __forceinline__ float form_floor(float4 k0, float4 k1, float4 k2, flo
 // Power of two above which a kernel's form makes all its moments over the
 // item's cnt residual points round to zero: |moment| <= cnt max|E| 2^-q
 // max(1, r2) (phi <= 2^-q, and |Delta| <= sqrt(r2) in the support) is below
-// 2^-38 for q - log2(max(1, r2)) > this.  Infinite when a residual is not finite.
+// 2^-38 for q - log2(max(1, r2)) > this.  Infinite when a residual is not
+// finite (emax is the largest of the residuals' absolute bits, where a NaN
+// lies above everything).
 __device__ __forceinline__ float form_limit(float emax, int cnt) {
     const int e = (int)(__float_as_uint(emax) >> 23);  // emax < 2^(e - 126)
     return e >= 255 ? INFINITY : (float)(38 + (e - 126) + (32 - __clz(cnt)));
@@ -892,8 +897,8 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             uint32_t cnt[2], pr[2];
             const float e0 = point_out(a, it.i0, it.v0, tv[0], l0 + h0, n[0], l2[0], mx[0], cnt[0], pr[0]);
             const float e1 = point_out(a, it.i1, it.v1, tv[1], l1 + h1, n[1], l2[1], mx[1], cnt[1], pr[1]);
-            const float emax = finish_item(a, it.t0, it.two, two_sum(l2[0], l2[1]), fmaxf(mx[0], mx[1]), cnt[0] + cnt[1],
-                                           pr[0] + pr[1], lane);
+            finish_item(a, it.t0, it.two, two_sum(l2[0], l2[1]), fmaxf(mx[0], mx[1]), cnt[0] + cnt[1],
+                        pr[0] + pr[1], lane);
             if (ADJ) {
                 // adjoint pairs: every support pair of a point with E != 0
                 // (the adjoint takes exactly these)
@@ -905,6 +910,8 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
                 const int nc1 = nz_tile(nzs, kTile, e1 != 0.f, a.x[it.v1 ? it.i1 : 0], a.y[it.v1 ? it.i1 : 0],
                                         a.z[it.v1 ? it.i1 : 0], e1, lane, lo1, hi1);
                 __syncwarp();
+                const float emax = __uint_as_float(
+                    redux_max_u32(max(__float_as_uint(fabsf(e0)), __float_as_uint(fabsf(e1)))));
                 if (nc0 + nc1 > 0)
                     adjoint_share<1, (ADJ > 1)>(a, it, 0, nzs, nc0, nc1, box_min(lo0, lo1), box_max(hi0, hi1), touch[0],
                                                 ntouch, kTouchW, emax, adjq, lane, cost);
@@ -943,8 +950,9 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             const int64_t i = warp ? it.i1 : it.i0;
             const bool v = warp ? it.v1 : it.v0;
             const float e = point_out(a, i, v, warp ? tv[1] : tv[0], ps, np, l2, mx, cnt, pr);
-            const float emax = finish_tile(a, it.t0 + warp, l2, mx, cnt, pr, lane);
+            finish_tile(a, it.t0 + warp, l2, mx, cnt, pr, lane);
             if (ADJ) {
+                const float emax = __uint_as_float(redux_max_u32(__float_as_uint(fabsf(e))));
                 // adjoint pairs: every support pair of a point with E != 0
                 const uint32_t pb = redux_add(e != 0.f ? np : 0u);
                 if (lane == 0 && pb) atomicAdd(a.adj_pairs, (unsigned long long)pb);
@@ -977,7 +985,8 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
                 const float4 lo = nc1 ? (nc0 ? box_min(s_box[0][0], s_box[1][0]) : s_box[1][0]) : s_box[0][0];
                 const float4 hi = nc1 ? (nc0 ? box_max(s_box[0][1], s_box[1][1]) : s_box[1][1]) : s_box[0][1];
                 uint32_t c = 0;
-                const float emax = fmaxf(nc0 ? s_box[0][0].w : 0.f, nc1 ? s_box[1][0].w : 0.f);
+                const float emax = __uint_as_float(
+                    max(nc0 ? __float_as_uint(s_box[0][0].w) : 0u, nc1 ? __float_as_uint(s_box[1][0].w) : 0u));
                 adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, nc0, nc1, lo, hi, touch[warp], ntouch, kTouchW, emax,
                                             adjq, lane, c);
                 if (lane == 0) red_cost[warp] += c;
@@ -1042,19 +1051,6 @@ int launch_forward(const FwdArgs &a, int64_t nitems, int sm_count, cudaStream_t 
     launch_pdl(k_forward<G, ADJ>, dim3((unsigned)blocks), dim3(G * 32), 0, s, a);
     SERBF_CHECK_LAUNCH();
     return SERBF_OK;
-}
-
-template <int G>
-int64_t forward_groups(int sm_count) {
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_forward<G, 0>, G * 32, 0) != cudaSuccess ||
-            nb < 1)
-            nb = 1;
-        per_sm = nb;
-    }
-    return (int64_t)sm_count * per_sm;
 }
 
 // After the forward: the Eq. 3-19 loss terms from the tile partials in tile
@@ -1249,11 +1245,19 @@ bool make_args(const serbf_points *pts, const serbf_params *prm, const serbf_con
     return true;
 }
 
-// Warps per item: the fewest that still leave about four items per group of
-// warps for the heavy-first balancing, unless the configuration fixes it.
+// Warps per item, unless the configuration fixes it.  Items differ in cost
+// (an item in the middle of the kernels whose points all carry residuals costs
+// five times the mean and more), so a launch with few items per warp waits for
+// its heaviest ones; more warps per item shorten that tail and cost issue slots
+// for barriers and short batches.  Measured crossings on a 152-SM part, fused
+// call in us with 1 / 2 / 4 warps: 8.0 k items (80^3) 149 / 106 / 93, 14.6 k
+// (97^3, compensated) 251 / 181 / 172, 20.8 k (110^3) 243 / 194 / 226, 32.8 k
+// (128^3) 318 / 292 / 364, 147 k (9.4 M points) 2118 / 2280 / 2801; 8 warps were
+// within 3 % of 4 below 2 k items and slower above.
 int pick_warps(int64_t nitems, int sm_count, int fixed) {
     if (fixed == 1 || fixed == 2 || fixed == 4 || fixed == 8) return fixed;
-    return nitems >= 4 * forward_groups<1>(sm_count) ? 1 : (nitems >= 4 * forward_groups<2>(sm_count) ? 2 : 4);
+    const int64_t resident = 20 * (int64_t)sm_count;  // warps in flight
+    return nitems >= 16 * resident ? 1 : (nitems >= 6 * resident ? 2 : 4);
 }
 
 int forward_impl(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg, float *psi, float *err,
