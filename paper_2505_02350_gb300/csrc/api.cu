@@ -50,7 +50,7 @@ void carve(Carver &c, serbf_workspace *w, const serbf_ws_sizes *s) {
     w->keys1 = c.take<uint32_t>(N);
     w->vals0 = c.take<uint32_t>(N);
     w->vals1 = c.take<uint32_t>(N);
-    w->hist = c.take<uint32_t>(256 * SB + 1);
+    w->hist = c.take<uint32_t>(256 * (SB > kDirectBlocks ? SB : kDirectBlocks) + 256);
     w->cell_start = c.take<uint32_t>(S * cps + 1);
     w->super_tile0 = c.take<uint32_t>(S + 1);
     w->tile_super = c.take<uint32_t>(T);
@@ -97,22 +97,6 @@ void carve(Carver &c, serbf_workspace *w, const serbf_ws_sizes *s) {
     w->dtmp = c.take<double>(16);
     w->cell_max = c.take<uint32_t>(4);
     w->field_box = c.take<float4>(2);
-}
-
-__global__ void k_exscan_u32(uint32_t *a, int64_t n) {
-    __shared__ uint32_t tmp[33];
-    int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    int64_t b = per * threadIdx.x, e = b + per < n ? b + per : n;
-    uint32_t s = 0;
-    for (int64_t i = b; i < e; ++i) s += a[i];
-    uint32_t total;
-    uint32_t off = block_exscan(s, tmp, &total);
-    for (int64_t i = b; i < e; ++i) {
-        uint32_t v = a[i];
-        a[i] = off;
-        off += v;
-    }
-    if (threadIdx.x == 0) a[n] = total;
 }
 
 __global__ void k_exscan_i64(int64_t *a, int64_t n) {
@@ -208,11 +192,6 @@ int grid_for(int64_t n, int threads) {
 }  // namespace
 
 namespace serbf {
-int launch_exscan_u32(uint32_t *a, int64_t n, cudaStream_t s) {
-    k_exscan_u32<<<1, 1024, 0, s>>>(a, n);
-    SERBF_CHECK_LAUNCH();
-    return SERBF_OK;
-}
 int launch_exscan_i64(int64_t *a, int64_t n, cudaStream_t s) {
     k_exscan_i64<<<1, 1024, 0, s>>>(a, n);
     SERBF_CHECK_LAUNCH();

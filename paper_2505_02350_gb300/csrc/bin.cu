@@ -5,7 +5,15 @@
 // every super cell -- and every cell -- is a contiguous range of binned
 // points.  Each super cell's range is cut into 32-point tiles (one warp each);
 // tiles never straddle a super cell, so they are full except the last one of
-// each super cell, and a tile's bounding box is tight.  Also the Sec. 3.4.2
+// each super cell, and a tile's bounding box is tight.
+//
+// Eight to ten short launches, each started early behind its predecessor: keys
+// with the first digit's histogram, a histogram and a scatter per 8-bit digit
+// (and a row scan above 32 sort blocks), the last scatter moving the points;
+// then cells, super cells and tiles.  What bounds it is memory for large sets
+// and launches for small ones.  It replaced scans by a single block and a
+// serial walk per super cell: 2.1 M points took 576 us of kernels, now about
+// 130; 10 000 points 130 us, now about 45.  Also the Sec. 3.4.2
 // refinement entry point, which re-bins the grown training set.
 #include <math.h>
 
@@ -17,137 +25,237 @@ using namespace serbf;
 
 namespace {
 
-__global__ void k_keys(const float *x, const float *y, const float *z, int64_t n, serbf_grid g, int sf, int nsx,
-                       int nsy, uint32_t *keys, uint32_t *vals) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int kx = cell_axis(x[i], g.origin[0], g.h, g.n[0]);
-        int ky = cell_axis(y[i], g.origin[1], g.h, g.n[1]);
-        int kz = cell_axis(z[i], g.origin[2], g.h, g.n[2]);
-        keys[i] = cell_key(kx, ky, kz, sf, nsx, nsy);
-        vals[i] = (uint32_t)i;
-    }
+constexpr int kSortThreads = 512;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortRounds = kSortTile / kSortThreads;        // elements per thread
+constexpr int kSmallRounds = kSmallSortTile / kSortThreads;  // ... of a small set
+
+// Histogram of one 8-bit digit of a block's tile, stored digit-major.
+__device__ __forceinline__ void store_hist(const uint32_t *h, uint32_t *hist, int64_t nblk) {
+    if (threadIdx.x < 256) hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(256) k_radix_hist(const uint32_t *keys, int64_t n, int shift, uint32_t *hist,
-                                                    int64_t nblk) {
+// Cell keys of a tile of points and the histogram of their lowest digit (the
+// first radix pass takes the point's index as its value).
+template <int ROUNDS>
+__global__ void __launch_bounds__(kSortThreads) k_keys(const float *x, const float *y, const float *z, int64_t n,
+                                                       serbf_grid g, int sf, int nsx, int nsy, uint32_t *keys,
+                                                       uint32_t *hist, int64_t nblk, uint32_t *cell_max) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
+    if (threadIdx.x < 256) h[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) cell_max[0] = 0u;
     __syncthreads();
-    int64_t start = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortTile / 256; ++r) {
-        int64_t e = start + r * 256 + threadIdx.x;
+    const int64_t start = (int64_t)blockIdx.x * (ROUNDS * kSortThreads);
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int64_t i = start + r * kSortThreads + threadIdx.x;
+        if (i < n) {
+            const int kx = cell_axis(x[i], g.origin[0], g.h, g.n[0]);
+            const int ky = cell_axis(y[i], g.origin[1], g.h, g.n[1]);
+            const int kz = cell_axis(z[i], g.origin[2], g.h, g.n[2]);
+            const uint32_t key = cell_key(kx, ky, kz, sf, nsx, nsy);
+            keys[i] = key;
+            atomicAdd(&h[key & 255u], 1u);
+        }
+    }
+    __syncthreads();
+    store_hist(h, hist, nblk);
+}
+
+template <int ROUNDS>
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *keys, int64_t n, int shift, uint32_t *hist,
+                                                             int64_t nblk) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t h[256];
+    if (threadIdx.x < 256) h[threadIdx.x] = 0u;
+    __syncthreads();
+    const int64_t start = (int64_t)blockIdx.x * (ROUNDS * kSortThreads);
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int64_t e = start + r * kSortThreads + threadIdx.x;
         if (e < n) atomicAdd(&h[(keys[e] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
+    store_hist(h, hist, nblk);
 }
 
-// Stable scatter: within a block, elements keep their order per digit; blocks
-// are placed in order by the digit-major exclusive scan of the histograms.
-__global__ void __launch_bounds__(256) k_radix_scatter(const uint32_t *kin, const uint32_t *vin, uint32_t *kout,
-                                                       uint32_t *vout, int64_t n, int shift,
-                                                       const uint32_t *hist, int64_t nblk) {
-    __shared__ uint32_t wcnt[8][257];
-    __shared__ uint32_t run[256];
-    __shared__ uint32_t base[256];
-    int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = hist[(int64_t)tid * nblk + blockIdx.x];
-    run[tid] = 0;
-    for (int k = tid; k < 8 * 257; k += 256) (&wcnt[0][0])[k] = 0;
-    __syncthreads();
-    int64_t start = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortTile / 256; ++r) {
-        int64_t e = start + r * 256 + tid;
-        bool valid = e < n;
-        uint32_t key = valid ? kin[e] : 0u, val = valid ? vin[e] : 0u;
-        uint32_t d = valid ? (key >> shift) & 255u : 256u;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & ((1u << lane) - 1u));
-        if (rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        uint32_t acc = run[tid];
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            uint32_t c = wcnt[w][tid];
-            wcnt[w][tid] = acc;
-            acc += c;
-        }
-        run[tid] = acc;
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = base[d] + wcnt[warp][d] + rank;
-            kout[pos] = key;
-            vout[pos] = val;
-        }
-        __syncthreads();
-        for (int k = tid; k < 8 * 257; k += 256) (&wcnt[0][0])[k] = 0;
-        __syncthreads();
+// One block per digit: its counts become exclusive prefixes over the sort
+// blocks, its total goes to tot[digit].
+__global__ void __launch_bounds__(256) k_radix_rows(uint32_t *hist, int64_t nblk, uint32_t *tot) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t tmp[33];
+    uint32_t *row = hist + (int64_t)blockIdx.x * nblk;
+    uint32_t carry = 0;
+    for (int64_t b0 = 0; b0 < nblk; b0 += 256) {
+        const int64_t b = b0 + threadIdx.x;
+        uint32_t sum;
+        const uint32_t off = block_exscan(b < nblk ? row[b] : 0u, tmp, &sum);
+        if (b < nblk) row[b] = carry + off;
+        carry += sum;
     }
+    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
 }
 
-__global__ void k_apply_perm(const uint32_t *sorted_vals, const float *x, const float *y, const float *z,
-                             int64_t n, uint32_t *perm, float *xb, float *yb, float *zb) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t i = sorted_vals[k];
-        perm[k] = i;
-        xb[k] = x[i];
-        yb[k] = y[i];
-        zb[k] = z[i];
-    }
-}
+// Where the last radix pass puts the sorted points instead of the values.
+struct PermOut {
+    const float *x, *y, *z;
+    uint32_t *perm;
+    float *xb, *yb, *zb;
+};
 
-__global__ void k_zero_u32(uint32_t *a, int64_t n) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        a[k] = 0u;
-}
-
-__global__ void k_count_cells(const uint32_t *keys, int64_t n, uint32_t *cnt) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[keys[k]], 1u);
-}
-
-// tiles and forward work items per super cell (for the scans that number them)
-__global__ void k_super_tiles(const uint32_t *cell_start, int nsuper, int cps, uint32_t *stile, uint32_t *sitem,
-                              uint32_t *maxt, uint32_t *maxc) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsuper; s += gridDim.x * blockDim.x) {
-        uint32_t b = cell_start[(int64_t)s * cps], e = cell_start[(int64_t)(s + 1) * cps];
-        const uint32_t nt = (e - b + kTile - 1) / kTile;
-        stile[s] = nt;
-        sitem[s] = (nt + 1) / 2;
-        atomicMax(maxt, nt);
-        // most points in one cell of this super cell (bounds the points in a ball)
-        uint32_t mc = 0, prev = b;
-        for (int c = 1; c <= cps; ++c) {
-            const uint32_t q = cell_start[(int64_t)s * cps + c];
-            mc = max(mc, q - prev);
-            prev = q;
-        }
-        atomicMax(maxc, mc);
-    }
-}
-
-// Tiles of each super cell, and its work items: the tiles at even offsets
-// (with the following tile, if any, as the item's second tile).  The first
-// forward takes them in this order.
-__global__ void k_fill_tiles(const uint32_t *cell_start, const uint32_t *stile0, const uint32_t *sitem0, int nsuper,
-                             int cps, uint32_t *tile_super, uint32_t *tile_start, uint4 *item_rec,
-                             uint4 *order_rec, uint8_t *item_class) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsuper; s += gridDim.x * blockDim.x) {
-        const uint32_t t0 = stile0[s], t1 = stile0[s + 1], i0 = sitem0[s];
-        const uint32_t p0 = cell_start[(int64_t)s * cps], pe = cell_start[(int64_t)(s + 1) * cps];
-        for (uint32_t t = t0; t < t1; ++t) {
-            const uint32_t ps = p0 + (t - t0) * kTile;
-            tile_super[t] = (uint32_t)s;
-            tile_start[t] = ps;
-            if (((t - t0) & 1u) == 0) {
-                const uint32_t it = i0 + (t - t0) / 2;
-                const uint32_t np = min(pe - ps, 2u * kTile);
-                const uint4 r = make_uint4(t, (uint32_t)s, ps, np | (it << 7));
-                item_rec[it] = r;
-                order_rec[it] = r;
-                item_class[it] = 3;  // one class for all until a forward has measured them
+// Stable scatter of one tile by one digit.  A warp owns 256 consecutive
+// elements, so ranks come from ballots and the warp's own running digit
+// counts, without a block barrier per round; one scan over the warps then
+// places them (a barrier for each of 16 rounds of 256 elements took 18 us for
+// 10 000 points, this takes about 6).  vin == nullptr: the values are the
+// indices.  tot == nullptr: few blocks, each sums the histograms itself.
+template <bool LAST, int ROUNDS>
+__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const uint32_t *kin, const uint32_t *vin, uint32_t *kout,
+                                                                uint32_t *vout, int64_t n, int shift,
+                                                                const uint32_t *hist, int64_t nblk, const uint32_t *tot,
+                                                                PermOut o) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t wcnt[kSortWarps][256];
+    __shared__ uint32_t tmp[33];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = tid; k < kSortWarps * 256; k += kSortThreads) (&wcnt[0][0])[k] = 0u;
+    uint32_t total = 0, before = 0;
+    if (tid < 256) {
+        const uint32_t *row = hist + (int64_t)tid * nblk;
+        if (tot) {
+            total = tot[tid];
+            before = row[blockIdx.x];
+        } else {
+            for (int b = 0; b < (int)nblk; ++b) {
+                const uint32_t v = row[b];
+                total += v;
+                before += b < (int)blockIdx.x ? v : 0u;
             }
         }
+    }
+    const uint32_t base = block_exscan(total, tmp, nullptr) + before;  // barriers: wcnt is clear
+    const int64_t e0 = (int64_t)blockIdx.x * (ROUNDS * kSortThreads) + warp * (ROUNDS * 32) + lane;
+    uint32_t key[ROUNDS], rank[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) key[r] = e0 + 32 * r < n ? kin[e0 + 32 * r] : 0u;
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const uint32_t d = e0 + 32 * r < n ? (key[r] >> shift) & 255u : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t ahead = __popc(peers & ((1u << lane) - 1u));
+        const uint32_t c = d < 256u ? wcnt[warp][d] : 0u;
+        __syncwarp();
+        if (ahead == 0 && d < 256u) wcnt[warp][d] = c + __popc(peers);
+        __syncwarp();
+        rank[r] = c + ahead;
+    }
+    __syncthreads();
+    if (tid < 256) {
+        uint32_t run = base;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const uint32_t c = wcnt[w][tid];
+            wcnt[w][tid] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int64_t e = e0 + 32 * r;
+        if (e < n) {
+            const uint32_t val = vin ? vin[e] : (uint32_t)e;
+            const uint32_t pos = wcnt[warp][(key[r] >> shift) & 255u] + rank[r];
+            kout[pos] = key[r];
+            if (LAST) {
+                o.perm[pos] = val;
+                o.xb[pos] = o.x[val];
+                o.yb[pos] = o.y[val];
+                o.zb[pos] = o.z[val];
+            } else {
+                vout[pos] = val;
+            }
+        }
+    }
+}
+
+// First binned point of every cell (a binary search of the sorted keys per
+// cell: no counting atomics, no scan), and the most points in one cell (bounds
+// the points in a ball).
+__global__ void __launch_bounds__(256) k_cells(const uint32_t *keys, int64_t n, int64_t ncp, uint32_t *cell_start,
+                                               uint32_t *cell_max) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t first[257];
+    const int64_t c = blockIdx.x * (int64_t)256 + threadIdx.x;
+    auto search = [&](int64_t k) {
+        int64_t lo = 0, hi = n;  // first position with a key >= k
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int64_t)keys[mid] < k) lo = mid + 1; else hi = mid;
+        }
+        return (uint32_t)lo;
+    };
+    if (c <= ncp) {
+        const uint32_t f = search(c);
+        first[threadIdx.x] = f;
+        cell_start[c] = f;
+        if (threadIdx.x == 255 && c < ncp) first[256] = search(c + 1);
+    }
+    __syncthreads();
+    uint32_t cnt = c < ncp ? first[threadIdx.x + 1] - first[threadIdx.x] : 0u;
+    cnt = __reduce_max_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0 && cnt) atomicMax(cell_max, cnt);
+}
+
+// One block: tiles and forward work items of every super cell, numbered in
+// super-cell order; out = {tiles, items, most tiles in one super cell}.  Also
+// clears the forward's scheduling state (no mean cost yet: the first forward
+// files every item in the same class).
+__global__ void __launch_bounds__(1024) k_supers(const uint32_t *cell_start, int nsuper, int cps, uint32_t *stile,
+                                                 uint32_t *sitem, uint32_t *sched, unsigned long long *sched_total,
+                                                 uint32_t *out) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t tmp[33];
+    __shared__ uint32_t s_max;
+    if (threadIdx.x == 0) s_max = 0u;
+    if (threadIdx.x < 4) sched[threadIdx.x] = 0u;
+    if (threadIdx.x < 2) sched_total[threadIdx.x] = 0ull;
+    __syncthreads();
+    uint32_t t0 = 0, i0 = 0, mx = 0;
+    for (int s0 = 0; s0 < nsuper; s0 += blockDim.x) {
+        const int s = s0 + threadIdx.x;
+        uint32_t nt = 0;
+        if (s < nsuper) {
+            const uint32_t b = cell_start[(int64_t)s * cps], e = cell_start[(int64_t)(s + 1) * cps];
+            nt = (e - b + kTile - 1) / kTile;
+        }
+        mx = max(mx, nt);
+        uint32_t ts, is;
+        const uint32_t to = block_exscan(nt, tmp, &ts), io = block_exscan((nt + 1) / 2, tmp, &is);
+        if (s < nsuper) {
+            stile[s] = t0 + to;
+            sitem[s] = i0 + io;
+        }
+        t0 += ts;
+        i0 += is;
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, mx);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        stile[nsuper] = t0;
+        sitem[nsuper] = i0;
+        out[0] = t0;
+        out[1] = i0;
+        out[2] = s_max;
+        out[3] = 0u;  // arrival counter of k_tiles
     }
 }
 
@@ -167,82 +275,96 @@ __device__ __forceinline__ void warp_box(float x, float y, float z, bool v, floa
     hi = make_float4(mxx, mxy, mxz, 0.f);
 }
 
-// One warp per tile: the bounding box of its points.
-__global__ void k_tile_boxes(const uint32_t *tile_super, const uint32_t *tile_start, const uint32_t *cell_start,
-                             int cps, int64_t ntiles, const float *xb, const float *yb, const float *zb, float4 *lo,
-                             float4 *hi) {
-    int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (t >= ntiles) return;
-    uint32_t s = tile_super[t], p0 = tile_start[t], pe = cell_start[(int64_t)(s + 1) * cps];
-    uint32_t i = p0 + lane;
-    bool v = i < pe;
-    float4 a, b;
-    warp_box(v ? xb[i] : 0.f, v ? yb[i] : 0.f, v ? zb[i] : 0.f, v, a, b);
-    if (lane == 0) {
-        lo[t] = a;
-        hi[t] = b;
-    }
+struct TilesArgs {
+    const uint32_t *cell_start, *stile0, *sitem0;
+    int nsuper, cps;
+    uint32_t *tile_super, *tile_start;
+    uint4 *item_rec, *order_rec;
+    uint8_t *item_class;
+    const float *xb, *yb, *zb;
+    float4 *tlo, *thi, *slo, *shi, *box;
+    uint32_t *arrived;
+};
+
+__device__ __forceinline__ void grow(float4 &lo, float4 &hi, float4 a, float4 b) {
+    lo = make_float4(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z), 0.f);
+    hi = make_float4(fmaxf(hi.x, b.x), fmaxf(hi.y, b.y), fmaxf(hi.z, b.z), 0.f);
 }
 
-// One block: the union of the super-cell boxes (the box of every binned point).
-__global__ void k_field_box(const float4 *slo, const float4 *shi, int nsuper, float4 *box) {
-    __shared__ float red[6][32];
-    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    for (int s = threadIdx.x; s < nsuper; s += blockDim.x) {
-        const float4 a = slo[s], b = shi[s];
-        v[0] = fminf(v[0], a.x);
-        v[1] = fminf(v[1], a.y);
-        v[2] = fminf(v[2], a.z);
-        v[3] = fmaxf(v[3], b.x);
-        v[4] = fmaxf(v[4], b.y);
-        v[5] = fmaxf(v[5], b.z);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const float w = __shfl_xor_sync(0xffffffffu, v[k], o);
-            v[k] = k < 3 ? fminf(v[k], w) : fmaxf(v[k], w);
+constexpr int kTilesThreads = 512;
+
+// One block per super cell, a warp per tile: the tile's start and bounding
+// box, the work items (the tiles at even offsets, with the following tile, if
+// any, as the item's second; the first forward takes them in this order), the
+// super cell's box (empty: +inf / -inf).  The last block unites the super
+// cells' boxes (the box of every binned point).
+__global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    constexpr int NW = kTilesThreads / 32;
+    __shared__ float4 wlo[NW], whi[NW];
+    __shared__ bool s_last;
+    const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t t0 = a.stile0[s], t1 = a.stile0[s + 1], i0 = a.sitem0[s];
+    const uint32_t p0 = a.cell_start[(int64_t)s * a.cps], pe = a.cell_start[(int64_t)(s + 1) * a.cps];
+    const float4 none_lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    const float4 none_hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+    float4 lo = none_lo, hi = none_hi;
+    for (uint32_t t = t0 + warp; t < t1; t += NW) {
+        const uint32_t ps = p0 + (t - t0) * kTile, i = ps + lane;
+        const bool v = i < pe;
+        float4 tl, th;
+        warp_box(v ? a.xb[i] : 0.f, v ? a.yb[i] : 0.f, v ? a.zb[i] : 0.f, v, tl, th);
+        grow(lo, hi, tl, th);
+        if (lane == 0) {
+            a.tlo[t] = tl;
+            a.thi[t] = th;
+            a.tile_super[t] = (uint32_t)s;
+            a.tile_start[t] = ps;
+            if (((t - t0) & 1u) == 0) {
+                const uint32_t it = i0 + (t - t0) / 2;
+                const uint32_t np = min(pe - ps, 2u * kTile);
+                const uint4 r = make_uint4(t, (uint32_t)s, ps, np | (it << 7));
+                a.item_rec[it] = r;
+                a.order_rec[it] = r;
+                a.item_class[it] = 3;  // one class for all until a forward has measured them
+            }
         }
-        if (lane == 0) red[k][warp] = v[k];
+    }
+    if (lane == 0) {
+        wlo[warp] = lo;
+        whi[warp] = hi;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            for (int k = 0; k < 6; ++k) v[k] = k < 3 ? fminf(v[k], red[k][w]) : fmaxf(v[k], red[k][w]);
-        box[0] = make_float4(v[0], v[1], v[2], 0.f);
-        box[1] = make_float4(v[3], v[4], v[5], 0.f);
+        for (int w = 1; w < NW; ++w) grow(lo, hi, wlo[w], whi[w]);
+        a.slo[s] = lo;
+        a.shi[s] = hi;
+        __threadfence();
+        s_last = atomicAdd(a.arrived, 1u) == gridDim.x - 1;
     }
-}
-
-// One warp per super cell: union of its tile boxes (empty: +inf / -inf).
-__global__ void k_super_boxes(const uint32_t *stile0, int nsuper, const float4 *tlo, const float4 *thi, float4 *slo,
-                              float4 *shi) {
-    int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (s >= nsuper) return;
-    float mnx = INFINITY, mny = INFINITY, mnz = INFINITY, mxx = -INFINITY, mxy = -INFINITY, mxz = -INFINITY;
-    for (uint32_t t = stile0[s] + lane; t < stile0[s + 1]; t += 32) {
-        float4 a = tlo[t], b = thi[t];
-        mnx = fminf(mnx, a.x);
-        mny = fminf(mny, a.y);
-        mnz = fminf(mnz, a.z);
-        mxx = fmaxf(mxx, b.x);
-        mxy = fmaxf(mxy, b.y);
-        mxz = fmaxf(mxz, b.z);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mnx = fminf(mnx, __shfl_xor_sync(0xffffffffu, mnx, o));
-        mny = fminf(mny, __shfl_xor_sync(0xffffffffu, mny, o));
-        mnz = fminf(mnz, __shfl_xor_sync(0xffffffffu, mnz, o));
-        mxx = fmaxf(mxx, __shfl_xor_sync(0xffffffffu, mxx, o));
-        mxy = fmaxf(mxy, __shfl_xor_sync(0xffffffffu, mxy, o));
-        mxz = fmaxf(mxz, __shfl_xor_sync(0xffffffffu, mxz, o));
-    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    lo = none_lo;
+    hi = none_hi;
+    for (int q = threadIdx.x; q < a.nsuper; q += kTilesThreads) grow(lo, hi, __ldcg(a.slo + q), __ldcg(a.shi + q));
+    float4 l, h;
+    const float4 b = hi;
+    warp_box(lo.x, lo.y, lo.z, true, l, h);
+    lo = l;
+    warp_box(b.x, b.y, b.z, true, l, h);
     if (lane == 0) {
-        slo[s] = make_float4(mnx, mny, mnz, 0.f);
-        shi[s] = make_float4(mxx, mxy, mxz, 0.f);
+        wlo[warp] = lo;
+        whi[warp] = h;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        lo = none_lo;
+        hi = none_hi;
+        for (int w = 0; w < NW; ++w) grow(lo, hi, wlo[w], whi[w]);
+        a.box[0] = lo;
+        a.box[1] = hi;
     }
 }
 
@@ -262,19 +384,53 @@ int gsz(int64_t n, int t) {
 
 namespace serbf {
 
-int radix_sort_pairs(uint32_t **k, uint32_t **v, uint32_t **ktmp, uint32_t **vtmp, int64_t n, int bits,
-                     uint32_t *hist, cudaStream_t s) {
-    const int64_t nblk = (n + kSortTile - 1) / kSortTile;
+// Small sets are cut into more, smaller sort tiles (10 000 points are three
+// tiles of 4096: too few blocks to hide anything); up to kDirectBlocks of them
+// every block sums the histograms itself instead of a launch for it.
+struct SortPlan {
+    int64_t nblk;
+    bool small;
+};
+static SortPlan sort_plan(int64_t n) {
+    const bool small = n <= (int64_t)kDirectBlocks * kSmallSortTile;
+    const int64_t tile = small ? kSmallSortTile : kSortTile;
+    return {(n + tile - 1) / tile, small};
+}
+
+template <int ROUNDS>
+static void sort_pass(uint32_t *k, uint32_t *v, uint32_t *ko, uint32_t *vo, int64_t n, int shift, uint32_t *hist,
+                      int64_t nblk, bool hist_done, const PermOut *out, cudaStream_t s) {
+    const dim3 grid((unsigned)nblk), block(kSortThreads);
+    if (!hist_done) launch_pdl(k_radix_hist<ROUNDS>, grid, block, 0, s, k, n, shift, hist, nblk);
+    uint32_t *tot = nblk > kDirectBlocks ? hist + 256 * nblk : nullptr;
+    if (tot) launch_pdl(k_radix_rows, dim3(256), dim3(256), 0, s, hist, nblk, tot);
+    if (out)
+        launch_pdl(k_radix_scatter<true, ROUNDS>, grid, block, 0, s, k, v, ko, vo, n, shift, hist, nblk, tot, *out);
+    else
+        launch_pdl(k_radix_scatter<false, ROUNDS>, grid, block, 0, s, k, v, ko, vo, n, shift, hist, nblk, tot, PermOut{});
+}
+
+// The passes of a sort.  keyed: the first digit's histogram is there already
+// and the values are the indices.  With a PermOut the last pass writes it
+// instead of the values.
+static int sort_passes(uint32_t **k, uint32_t **v, uint32_t **ktmp, uint32_t **vtmp, int64_t n, int bits, uint32_t *hist,
+                       bool keyed, const PermOut *out, cudaStream_t s) {
+    const SortPlan p = sort_plan(n);
     for (int shift = 0; shift < bits; shift += 8) {
-        k_radix_hist<<<(unsigned)nblk, 256, 0, s>>>(*k, n, shift, hist, nblk);
-        int rc = launch_exscan_u32(hist, 256 * nblk, s);
-        if (rc) return rc;
-        k_radix_scatter<<<(unsigned)nblk, 256, 0, s>>>(*k, *v, *ktmp, *vtmp, n, shift, hist, nblk);
+        const bool done = keyed && shift == 0;
+        const PermOut *o = shift + 8 >= bits ? out : nullptr;
+        (p.small ? sort_pass<kSmallRounds> : sort_pass<kSortRounds>)(*k, done ? nullptr : *v, *ktmp, *vtmp, n, shift, hist,
+                                                                     p.nblk, done, o, s);
         std::swap(*k, *ktmp);
         std::swap(*v, *vtmp);
     }
     SERBF_CHECK_LAUNCH();
     return SERBF_OK;
+}
+
+int radix_sort_pairs(uint32_t **k, uint32_t **v, uint32_t **ktmp, uint32_t **vtmp, int64_t n, int bits,
+                     uint32_t *hist, cudaStream_t s) {
+    return sort_passes(k, v, ktmp, vtmp, n, bits, hist, false, nullptr, s);
 }
 
 }  // namespace serbf
@@ -306,53 +462,33 @@ extern "C" int serbf_bin_points(const float *x, const float *y, const float *z, 
 
     uint32_t *kin = ws->keys0, *vin = ws->vals0, *kout = ws->keys1, *vout = ws->vals1;
     if (n > 0) {
-        k_keys<<<gsz(n, 256), 256, 0, s>>>(x, y, z, n, *grid, sf, nsx, nsy, kin, vin);
+        const SortPlan p = sort_plan(n);
+        launch_pdl(p.small ? k_keys<kSmallRounds> : k_keys<kSortRounds>, dim3((unsigned)p.nblk), dim3(kSortThreads), 0, s, x,
+                   y, z, n, *grid, sf, nsx, nsy, kin, ws->hist, p.nblk, ws->cell_max);
         int nbits = 1;
         while (nbits < 32 && (1ll << nbits) < ncp) ++nbits;
-        int rc = radix_sort_pairs(&kin, &vin, &kout, &vout, n, nbits, ws->hist, s);
+        const PermOut out{x, y, z, perm, xb, yb, zb};
+        const int rc = sort_passes(&kin, &vin, &kout, &vout, n, nbits, ws->hist, true, &out, s);
         if (rc) return rc;
-        k_apply_perm<<<gsz(n, 256), 256, 0, s>>>(vin, x, y, z, n, perm, xb, yb, zb);
+    } else if (cudaMemsetAsync(ws->cell_max, 0, sizeof(uint32_t), s) != cudaSuccess) {
+        return SERBF_ECUDA;
     }
-    k_zero_u32<<<gsz(ncp + 1, 256), 256, 0, s>>>(ws->cell_start, ncp + 1);
-    if (n > 0) k_count_cells<<<gsz(n, 256), 256, 0, s>>>(kin, n, ws->cell_start);
-    int rc = launch_exscan_u32(ws->cell_start, ncp, s);
-    if (rc) return rc;
-    uint32_t *maxt = ws->counters + 8;
-    cudaMemsetAsync(maxt, 0, sizeof(uint32_t), s);
-    cudaMemsetAsync(ws->cell_max, 0, sizeof(uint32_t), s);
-    k_super_tiles<<<gsz(nsuper, 256), 256, 0, s>>>(ws->cell_start, (int)nsuper, cps, ws->super_tile0,
-                                                   ws->super_item0, maxt, ws->cell_max);
-    rc = launch_exscan_u32(ws->super_tile0, nsuper, s);
-    if (rc) return rc;
-    rc = launch_exscan_u32(ws->super_item0, nsuper, s);
-    if (rc) return rc;
-    k_fill_tiles<<<gsz(nsuper, 256), 256, 0, s>>>(ws->cell_start, ws->super_tile0, ws->super_item0, (int)nsuper, cps,
-                                                  ws->tile_super, ws->tile_start, ws->item_rec, ws->order_rec,
-                                                  ws->item_class);
+    launch_pdl(k_cells, dim3((unsigned)((ncp + 256) / 256)), dim3(256), 0, s, kin, n, ncp, ws->cell_start, ws->cell_max);
+    uint32_t *out = ws->counters + 12;
+    launch_pdl(k_supers, dim3(1), dim3(1024), 0, s, ws->cell_start, (int)nsuper, cps, ws->super_tile0, ws->super_item0,
+               ws->sched, ws->sched_total, out);
+    launch_pdl(k_tiles, dim3((unsigned)nsuper), dim3(kTilesThreads), 0, s,
+               TilesArgs{ws->cell_start, ws->super_tile0, ws->super_item0, (int)nsuper, cps, ws->tile_super,
+                         ws->tile_start, ws->item_rec, ws->order_rec, ws->item_class, xb, yb, zb, ws->tile_lo,
+                         ws->tile_hi, ws->sup_lo, ws->sup_hi, ws->field_box, out + 3});
     SERBF_CHECK_LAUNCH();
-    uint32_t nt = 0, mt = 0, ni = 0;
-    if (cudaMemcpyAsync(&nt, ws->super_tile0 + nsuper, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return SERBF_ECUDA;
-    if (cudaMemcpyAsync(&ni, ws->super_item0 + nsuper, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return SERBF_ECUDA;
-    if (cudaMemcpyAsync(&mt, maxt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
+    uint32_t got[3];  // tiles, items, most tiles in a super cell
+    if (cudaMemcpyAsync(got, out, sizeof(got), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
-    if ((int64_t)nt > ws->max_tiles || ni >= (1u << 25)) return SERBF_ECAPACITY;  // item ids have 25 bits
-    ws->nitems = ni;
-    // scheduling state: no mean cost yet (the first forward files every item
-    // in the same class), no counts
-    if (cudaMemsetAsync(ws->sched, 0, 4 * sizeof(uint32_t), s) != cudaSuccess) return SERBF_ECUDA;
-    if (cudaMemsetAsync(ws->sched_total, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess) return SERBF_ECUDA;
-
-    ws->ntiles = nt;
-    ws->max_chunks = (int32_t)((mt + kTile - 1) / kTile);
-    if (nt > 0)
-        k_tile_boxes<<<(unsigned)((nt * 32 + 255) / 256), 256, 0, s>>>(ws->tile_super, ws->tile_start, ws->cell_start,
-                                                                        cps, nt, xb, yb, zb, ws->tile_lo, ws->tile_hi);
-    k_super_boxes<<<(unsigned)((nsuper * 32 + 255) / 256), 256, 0, s>>>(ws->super_tile0, (int)nsuper, ws->tile_lo,
-                                                                        ws->tile_hi, ws->sup_lo, ws->sup_hi);
-    k_field_box<<<1, 256, 0, s>>>(ws->sup_lo, ws->sup_hi, (int)nsuper, ws->field_box);
-    SERBF_CHECK_LAUNCH();
+    if ((int64_t)got[0] > ws->max_tiles || got[1] >= (1u << 25)) return SERBF_ECAPACITY;  // item ids have 25 bits
+    ws->ntiles = got[0];
+    ws->nitems = got[1];
+    ws->max_chunks = (int32_t)((got[2] + kTile - 1) / kTile);
     ws->binned = 1;
     return SERBF_OK;
 }

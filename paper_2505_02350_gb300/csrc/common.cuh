@@ -22,6 +22,8 @@ struct TraceRange {
 constexpr uint64_t kMagic = 0x53455242465753ull;  // "SERBFWS"
 constexpr int kTile = 32;                         // points per forward/backward tile (one warp)
 constexpr int kSortTile = 4096;                   // elements per radix-sort block
+constexpr int kSmallSortTile = 1024;              // ... while these give at most kDirectBlocks blocks
+constexpr int kDirectBlocks = 32;
 constexpr int kQueue = 64;                        // per-warp ring of staged candidates
 constexpr int kFwdGroup = 64;                     // tiles per first-level forward reduction group
 constexpr double kFixUnit = 1.0 / 68719476736.0;  // 2^-36: fixed-point unit of the fused adjoint's moments
@@ -46,8 +48,8 @@ struct FwdPart {
 };
 
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the
-// keys (8 bits per pass, kSortTile elements per block; hist holds
-// 256 x blocks + 1 words).  On return *k and *v point to whichever of the two
+// keys (8 bits per pass; hist holds 256 x (max(kSortTile blocks, kDirectBlocks)
+// + 1) words).  On return *k and *v point to whichever of the two
 // buffer pairs holds the result.  Defined in bin.cu.
 int radix_sort_pairs(uint32_t **k, uint32_t **v, uint32_t **ktmp, uint32_t **vtmp, int64_t n, int bits,
                      uint32_t *hist, cudaStream_t s);
@@ -524,6 +526,5 @@ __device__ __forceinline__ KBox kernel_box(float cx, float cy, float cz, float r
 
 // ---------------------------------------------------------------- cross-unit launchers
 namespace serbf {
-int launch_exscan_u32(uint32_t *a, int64_t n, cudaStream_t s);  // in place, a[n] = total
 int launch_exscan_i64(int64_t *a, int64_t n, cudaStream_t s);   // in place, a[n] = total
 }  // namespace serbf
