@@ -4,12 +4,18 @@
 //
 // The interior points (1 < t < 2, Eq. 3-10) are sorted by d_in = |S|
 // descending (stable, so equal values keep the binned order: the first
-// maximum is taken, as an argmax does).  One block then walks that order:
-// the first point not yet removed is the next centre; every interior point
-// within its sphere -- found through the binning cells of the sphere's box --
-// is removed.  The removal test is the float squared distance in the support
-// predicate's operation order against fl(r r), so the decisions are exact
-// and reproducible.
+// maximum is taken, as an argmax does).  The greedy walk of that order is done
+// in rounds: one block takes the next kBatch points that are still there and
+// settles them among themselves in order (k_settle), then all blocks remove
+// the later points that the new centres' spheres cover (k_cover).  That is the
+// same walk: a point's fate depends only on earlier centres, all of which are
+// known when it is settled.  The removal test is the float squared distance in
+// the support predicate's operation order against fl(r r), so the decisions
+// are exact and reproducible.
+//
+// One block walking point by point took 100 ms for 23 k interior points and
+// 6457 centres (64^3, 15 us a centre, nearly all of it barriers and dependent
+// loads); ten rounds take under 1 ms.
 #include <math.h>
 
 #include "common.cuh"
@@ -18,7 +24,17 @@ using namespace serbf;
 
 namespace {
 
-constexpr int kInitThreads = 1024;
+constexpr int kBatch = 1024;      // points settled per round, one per thread
+constexpr int kRounds = 8;        // rounds between two looks at the state
+constexpr uint32_t kSparse = 384; // new centres in a round after which the next one looks for conflicts first
+
+// Where the walk stands (device; ws->counters + 8).
+struct Walk {
+    uint32_t next;     // first sorted position not settled yet
+    uint32_t fresh;    // centres of the last round
+    uint32_t count;    // interior points
+    uint32_t centres;  // centres so far
+};
 
 // Sort keys: interior points by |S| descending (inverted float bits of a
 // positive value), everything else last.
@@ -33,111 +49,155 @@ __global__ void k_init_keys(const float *t, const float *S, int64_t n, uint32_t 
     }
 }
 
-// rank[binned index] = position in the sorted interior order, or ~0u.
-__global__ void k_init_rank(const uint32_t *sorted_vals, int64_t n, const uint32_t *count, uint32_t *rank) {
-    const int64_t nin = *count;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        rank[sorted_vals[k]] = k < nin ? (uint32_t)k : 0xffffffffu;
+// Interior points in sorted order as (x, y, z, fl(r r)).
+__global__ void k_init_points(const float *x, const float *y, const float *z, const float *S, const uint32_t *order,
+                              const Walk *w, float4 *pts) {
+    const int64_t nin = w->count;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nin; q += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = order[q];
+        const float r = fabsf(S[i]);
+        pts[q] = make_float4(x[i], y[i], z[i], __fmul_rn(r, r));
+    }
 }
 
-struct InitArgs {
-    const float *x, *y, *z, *S;
+// Whether the sphere of c (centre, r r) holds p.
+__device__ __forceinline__ bool covered(float4 p, float4 c) {
+    return !(support_d2(__fsub_rn(p.x, c.x), __fsub_rn(p.y, c.y), __fsub_rn(p.z, c.z)) > c.w);
+}
+
+static_assert(kBatch * 16 <= 256 * (kDirectBlocks + 1) * 4, "the fresh centres fit the sort's histograms");
+
+struct WalkArgs {
+    Walk *w;
+    const float4 *pts;
     const uint32_t *order;  // binned indices of the interior points, |S| descending
-    const uint32_t *count;  // number of interior points
-    const uint32_t *rank;
     uint8_t *removed;       // per sorted position
-    const uint32_t *cell_start;
-    serbf_grid g;
-    int sf, nsx, nsy;
     uint32_t *centres;      // binned indices of the centres, in selection order
+    float4 *fresh;          // the last round's centres
     int32_t cap;
-    uint32_t *ncentres;
 };
 
-// Algorithm 1, one block.  Terminates: every round removes at least its own
-// centre and the scan pointer only moves forward.
-__global__ void __launch_bounds__(kInitThreads) k_inscribed(InitArgs a) {
-    __shared__ int64_t s_first;
-    __shared__ int s_found;
-    const int64_t nin = *a.count;
-    for (int64_t q = threadIdx.x; q < nin; q += blockDim.x) a.removed[q] = 0;
+// One block: the next kBatch points still there, settled in order.  Thread c
+// holds the c-th of them.  Each step takes the first one left that may cover
+// another and lets every later thread test its point, one barrier a step.
+// After a round with many centres the spheres are small and most points cover
+// none of the batch, so all pairs are tested first and only the points that do
+// cover a later one are stepped through.
+__global__ void __launch_bounds__(kBatch) k_settle(WalkArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float4 s_pt[kBatch];
+    __shared__ uint32_t s_pos[kBatch];
+    __shared__ uint32_t s_word[2][kBatch / 32];
+    __shared__ uint8_t s_covers[kBatch];
+    __shared__ uint32_t tmp[33];
+    __shared__ uint32_t s_next;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t nin = a.w->count, first = a.w->next, last = a.w->fresh, before = a.w->centres;
+    if (first >= nin) {
+        if (tid == 0) a.w->fresh = 0u;
+        return;
+    }
+    if (tid == 0) s_next = nin;
     __syncthreads();
-    int64_t ptr = 0;
-    uint32_t cnt = 0;
-    for (;;) {
-        // the first position >= ptr not yet removed
-        if (threadIdx.x == 0) {
-            s_first = -1;
-            s_found = 0;
+    uint32_t n = 0;
+    for (uint64_t b = first; b < nin && n < kBatch; b += 4 * kBatch) {
+        const uint64_t q0 = b + 4 * tid;
+        uint32_t here = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) here |= (q0 + k < nin && !a.removed[q0 + k] ? 1u : 0u) << k;
+        uint32_t tot, o = block_exscan(__popc(here), tmp, &tot) + n;
+        for (; here && o < kBatch; here &= here - 1, ++o) {
+            const uint32_t q = (uint32_t)q0 + __ffs(here) - 1;
+            s_pos[o] = q;
+            if (o == kBatch - 1) s_next = q + 1;
         }
-        __syncthreads();
-        while (ptr < nin) {
-            const int64_t q = ptr + threadIdx.x;
-            const bool ok = q < nin && !a.removed[q];
-            if (ok) atomicOr(&s_found, 1);
-            __syncthreads();
-            if (s_found) {
-                // lowest candidate: warp minima, then a shared minimum
-                if (ok) atomicMin(reinterpret_cast<unsigned long long *>(&s_first), (unsigned long long)q);
-                break;
-            }
-            ptr += blockDim.x;
-            __syncthreads();
-        }
-        __syncthreads();
-        if (!s_found) break;
-        const int64_t p = s_first;
-        const uint32_t i = a.order[p];
-        const float cx = a.x[i], cy = a.y[i], cz = a.z[i];
-        const float r = fabsf(a.S[i]);
-        const float r2 = __fmul_rn(r, r);
-        if (threadIdx.x == 0) {
-            if ((int32_t)cnt < a.cap) a.centres[cnt] = i;
-            a.removed[p] = 1;
-        }
-        ++cnt;
-        // remove the interior points within the sphere (cells of its box)
-        const KBox b = kernel_box(cx, cy, cz, r2, a.g);
-        const int nx = b.kx1 - b.kx0 + 1;
-        const int64_t ncells = (int64_t)nx * b.nrows;
-        for (int64_t c = threadIdx.x; c < ncells; c += blockDim.x) {
-            const int kx = b.kx0 + (int)(c % nx);
-            const int row = (int)(c / nx);
-            const int ky = b.ky0 + row % b.nyr, kz = b.kz0 + row / b.nyr;
-            const uint32_t key = cell_key(kx, ky, kz, a.sf, a.nsx, a.nsy);
-            for (uint32_t k = a.cell_start[key]; k < a.cell_start[key + 1]; ++k) {
-                const uint32_t rk = a.rank[k];
-                if (rk == 0xffffffffu || a.removed[rk]) continue;
-                const float dx = __fsub_rn(a.x[k], cx), dy = __fsub_rn(a.y[k], cy), dz = __fsub_rn(a.z[k], cz);
-                const float d2 = support_d2(dx, dy, dz);
-                if (!(d2 > r2)) a.removed[rk] = 1;
-            }
-        }
-        ptr = p + 1;
+        n += tot;
+    }
+    n = min(n, (uint32_t)kBatch);
+    __syncthreads();
+    const bool mine = tid < (int)n;
+    const float4 p = mine ? a.pts[s_pos[tid]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    s_pt[tid] = p;
+    const bool sparse = last >= kSparse;
+    s_covers[tid] = !sparse;
+    __syncthreads();
+    if (sparse) {
+        if (mine)
+            for (int i = 0; i < tid; ++i)
+                if (covered(p, s_pt[i])) s_covers[i] = 1;
         __syncthreads();
     }
-    if (threadIdx.x == 0) *a.ncentres = cnt;
+    const bool covers = s_covers[tid];
+    bool left = mine;
+    for (int cur = -1, buf = 0;; buf ^= 1) {
+        const unsigned bal = __ballot_sync(0xffffffffu, left && covers && tid > cur);
+        if (lane == 0) s_word[buf][warp] = bal;
+        __syncthreads();
+        const uint32_t word = s_word[buf][lane];
+        const unsigned some = __ballot_sync(0xffffffffu, word != 0u);
+        if (!some) break;
+        const int w = __ffs(some) - 1;
+        cur = 32 * w + __ffs(__shfl_sync(0xffffffffu, word, w)) - 1;
+        if (left && tid > cur && covered(p, s_pt[cur])) left = false;
+    }
+    uint32_t tot;
+    const uint32_t o = block_exscan(left, tmp, &tot);
+    if (left) {
+        if (before + o < (uint32_t)a.cap) a.centres[before + o] = a.order[s_pos[tid]];
+        a.fresh[o] = p;
+    }
+    if (tid == 0) {
+        a.w->next = s_next;
+        a.w->fresh = tot;
+        a.w->centres = before + tot;
+    }
 }
 
-// Eq. 3-12 for the selected centres (thread per centre): dhat = distance to
+// The points from the next position on that a new centre covers are removed.
+__global__ void __launch_bounds__(256) k_cover(WalkArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float4 c[256];
+    const uint32_t nin = a.w->count, k = a.w->fresh, next = a.w->next;
+    for (uint64_t q0 = (uint64_t)next + blockIdx.x * 256ull; q0 < nin; q0 += gridDim.x * 256ull) {
+        const uint64_t q = q0 + threadIdx.x;
+        bool here = q < nin && !a.removed[q];
+        const float4 p = here ? a.pts[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        bool gone = false;
+        for (uint32_t c0 = 0; c0 < k; c0 += 256) {
+            __syncthreads();
+            if (c0 + threadIdx.x < k) c[threadIdx.x] = a.fresh[c0 + threadIdx.x];
+            __syncthreads();
+            const int m = (int)min(256u, k - c0);
+            if (here && !gone)
+                for (int i = 0; i < m && !gone; ++i) gone = covered(p, c[i]);
+        }
+        if (gone) a.removed[q] = 1;
+    }
+}
+
+// Eq. 3-12 for the selected centres (a warp per centre): dhat = distance to
 // the nearest other centre (a single centre: twice its radius), then
 // d = 2 sqrt(-ln(gamma / w^2)) / dhat on all axes, angles 0, w = t.
 __global__ void k_init_params(const float *x, const float *y, const float *z, const float *t, const float *S,
                               const uint32_t *centres, const uint32_t *ncentres, int32_t cap, float gamma, float *p,
                               int32_t *m_dev) {
     const int M = (int)min(*ncentres, (uint32_t)cap);
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j == 0) *m_dev = M;
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (j == 0 && lane == 0) *m_dev = M;
     if (j >= M) return;
     const uint32_t cj = centres[j];
     const float px = x[cj], py = y[cj], pz = z[cj];
     float best = INFINITY;
-    for (int i = 0; i < M; ++i) {
+    for (int i = lane; i < M; i += 32) {
         if (i == j) continue;
         const uint32_t ci = centres[i];
         const float dx = x[ci] - px, dy = y[ci] - py, dz = z[ci] - pz;
         best = fminf(best, dx * dx + dy * dy + dz * dz);
     }
+    best = -warp_max(-best);
+    if (lane != 0) return;
     const float dhat = M > 1 ? sqrtf(best) : 2.f * fabsf(S[cj]);
     const float w = t[cj];
     const float d = 2.f * sqrtf(-logf(gamma / (w * w))) / dhat;
@@ -164,42 +224,40 @@ extern "C" int serbf_init_kernels(const serbf_points *pts, const float *S_raw, d
     const int64_t n = pts->n;
     if (n > 0 && (!pts->x || !pts->y || !pts->z || !pts->t || !S_raw)) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    uint32_t *count = ws->counters + 10, *ncent = ws->counters + 11;
-    if (cudaMemsetAsync(count, 0, 2 * sizeof(uint32_t), s) != cudaSuccess) return SERBF_ECUDA;
+    Walk *w = reinterpret_cast<Walk *>(ws->counters + 8);
+    if (cudaMemsetAsync(w, 0, sizeof(Walk), s) != cudaSuccess) return SERBF_ECUDA;
     uint32_t *k = ws->keys0, *v = ws->vals0, *kt = ws->keys1, *vt = ws->vals1;
     const int grid = (int)((n + 255) / 256 < 152 * 64 ? (n + 255) / 256 : 152 * 64);
+    uint32_t found = 0;
     if (n > 0) {
-        k_init_keys<<<grid > 0 ? grid : 1, 256, 0, s>>>(pts->t, S_raw, n, k, v, count);
+        k_init_keys<<<grid, 256, 0, s>>>(pts->t, S_raw, n, k, v, &w->count);
         int rc = radix_sort_pairs(&k, &v, &kt, &vt, n, 32, ws->hist, s);
         if (rc) return rc;
-        // kt now holds scratch: the rank of each binned point
-        k_init_rank<<<grid > 0 ? grid : 1, 256, 0, s>>>(v, n, count, kt);
-        InitArgs a;
-        a.x = pts->x;
-        a.y = pts->y;
-        a.z = pts->z;
-        a.S = S_raw;
-        a.order = v;
-        a.count = count;
-        a.rank = kt;
-        a.removed = reinterpret_cast<uint8_t *>(ws->nz);  // >= 16 bytes per point, free between epochs
-        a.cell_start = ws->cell_start;
-        a.g = ws->grid;
-        a.sf = ws->sf;
-        a.nsx = ws->ns[0];
-        a.nsy = ws->ns[1];
-        a.centres = vt;  // the sort's other value buffer is free now
-        a.cap = prm->cap;
-        a.ncentres = ncent;
-        k_inscribed<<<1, kInitThreads, 0, s>>>(a);
-        k_init_params<<<(prm->cap + 255) / 256, 256, 0, s>>>(pts->x, pts->y, pts->z, pts->t, S_raw, vt, ncent,
-                                                             prm->cap, (float)gamma, prm->p, prm->m);
+        // kt now holds the removal flags, the sort's other value buffer the
+        // centres, its histograms the last round's centres; the points lie in
+        // the adjoint's compaction buffer (16 bytes per point, idle here)
+        WalkArgs a{w, ws->nz, v, reinterpret_cast<uint8_t *>(kt), vt, reinterpret_cast<float4 *>(ws->hist), prm->cap};
+        k_init_points<<<grid, 256, 0, s>>>(pts->x, pts->y, pts->z, S_raw, v, w, ws->nz);
+        if (cudaMemsetAsync(kt, 0, (size_t)n, s) != cudaSuccess) return SERBF_ECUDA;
+        const int64_t cover = (n + 255) / 256, most = 8 * (int64_t)ws->sm_count;
+        Walk now;
+        do {
+            // ends: every round settles at least one point
+            for (int q = 0; q < kRounds; ++q) {
+                launch_pdl(k_settle, dim3(1), dim3(kBatch), 0, s, a);
+                launch_pdl(k_cover, dim3((unsigned)(cover < most ? cover : most)), dim3(256), 0, s, a);
+            }
+            SERBF_CHECK_LAUNCH();
+            if (cudaMemcpyAsync(&now, w, sizeof(Walk), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
+            if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
+        } while (now.next < now.count);
+        found = now.centres;
+        k_init_params<<<(unsigned)((prm->cap + 7) / 8), 256, 0, s>>>(pts->x, pts->y, pts->z, pts->t, S_raw, vt, &w->centres,
+                                                                     prm->cap, (float)gamma, prm->p, prm->m);
     } else {
         if (cudaMemsetAsync(prm->m, 0, sizeof(int32_t), s) != cudaSuccess) return SERBF_ECUDA;
     }
     SERBF_CHECK_LAUNCH();
-    uint32_t found = 0;
-    if (cudaMemcpyAsync(&found, ncent, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
     if (m_out) *m_out = (int32_t)found;
     return (int64_t)found > prm->cap ? SERBF_ECAPACITY : SERBF_OK;
