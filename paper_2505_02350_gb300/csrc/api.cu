@@ -99,40 +99,73 @@ void carve(Carver &c, serbf_workspace *w, const serbf_ws_sizes *s) {
     w->field_box = c.take<float4>(2);
 }
 
-__global__ void k_exscan_i64(int64_t *a, int64_t n) {
-    __shared__ unsigned long long ws[32];
-    __shared__ unsigned long long tot;
-    int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    int64_t b = per * threadIdx.x, e = b + per < n ? b + per : n;
-    unsigned long long s = 0;
-    for (int64_t i = b; i < e; ++i) s += (unsigned long long)a[i];
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    unsigned long long inc = s;
+// Exclusive scan in three launches: sums of tiles of kScanTile elements, a scan
+// of those by one block, then every tile with its base.  (One block over all
+// elements: 216 us for 262 144.)
+constexpr int kScanThreads = 512;
+constexpr int kScanPer = 8;
+
+__device__ __forceinline__ int64_t block_iscan_i64(int64_t v, long long *tmp, int64_t *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    long long inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+        const long long t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
-    if (lane == 31) ws[warp] = inc;
+    if (lane == 31) tmp[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        unsigned long long v = lane < nw ? ws[lane] : 0ull, vi = v;
+        long long w = lane < nw ? tmp[lane] : 0ll;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long t = __shfl_up_sync(0xffffffffu, vi, o);
-            if (lane >= o) vi += t;
+            const long long t = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += t;
         }
-        if (lane < nw) ws[lane] = vi - v;
-        if (lane == 31) tot = vi;
+        tmp[lane] = w;
     }
     __syncthreads();
-    unsigned long long off = ws[warp] + inc - s;
-    for (int64_t i = b; i < e; ++i) {
-        unsigned long long v = (unsigned long long)a[i];
-        a[i] = (int64_t)off;
-        off += v;
+    *total = tmp[nw - 1];
+    inc += warp ? tmp[warp - 1] : 0ll;
+    __syncthreads();
+    return inc;
+}
+
+// SUMS: the tile's sum to tiles[b]; otherwise the exclusive scan of the tile
+// from tiles[b] on (the last tile also writes a[n]).
+template <bool SUMS>
+__global__ void __launch_bounds__(kScanThreads) k_scan_tile(int64_t *a, int64_t n, int64_t *tiles) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ long long tmp[32];
+    const int64_t base = blockIdx.x * (int64_t)kScanTile;
+    int64_t carry = SUMS ? 0 : tiles[blockIdx.x];
+    for (int r = 0; r < kScanPer; ++r) {
+        const int64_t i = base + r * kScanThreads + threadIdx.x;
+        const int64_t v = i < n ? a[i] : 0;
+        int64_t total;
+        const int64_t inc = block_iscan_i64(v, tmp, &total);
+        if (!SUMS && i < n) a[i] = carry + inc - v;
+        carry += total;
     }
-    if (threadIdx.x == 0) a[n] = (int64_t)tot;
+    if (threadIdx.x == 0) {
+        if (SUMS) tiles[blockIdx.x] = carry;
+        else if (blockIdx.x == gridDim.x - 1) a[n] = carry;
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_scan_sums(int64_t *tiles, int64_t nt) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ long long tmp[32];
+    int64_t carry = 0;
+    for (int64_t t0 = 0; t0 < nt; t0 += blockDim.x) {
+        const int64_t t = t0 + threadIdx.x, v = t < nt ? tiles[t] : 0;
+        int64_t total;
+        const int64_t inc = block_iscan_i64(v, tmp, &total);
+        if (t < nt) tiles[t] = carry + inc - v;
+        carry += total;
+    }
 }
 
 __global__ void k_gather(const float *src, const uint32_t *perm, float *dst, int64_t n) {
@@ -192,8 +225,12 @@ int grid_for(int64_t n, int threads) {
 }  // namespace
 
 namespace serbf {
-int launch_exscan_i64(int64_t *a, int64_t n, cudaStream_t s) {
-    k_exscan_i64<<<1, 1024, 0, s>>>(a, n);
+int launch_exscan_i64(int64_t *a, int64_t n, int64_t *tiles, cudaStream_t s) {
+    static_assert(kScanThreads * kScanPer == kScanTile, "elements per block");
+    const int64_t nt = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
+    launch_pdl(k_scan_tile<true>, dim3((unsigned)nt), dim3(kScanThreads), 0, s, a, n, tiles);
+    launch_pdl(k_scan_sums, dim3(1), dim3(1024), 0, s, tiles, nt);
+    launch_pdl(k_scan_tile<false>, dim3((unsigned)nt), dim3(kScanThreads), 0, s, a, n, tiles);
     SERBF_CHECK_LAUNCH();
     return SERBF_OK;
 }

@@ -526,6 +526,7 @@ __device__ __forceinline__ KBox kernel_box(float cx, float cy, float cz, float r
 
 // ---------------------------------------------------------------- cross-unit launchers
 namespace serbf {
-constexpr int kScanTile = 4096;  // elements of a scan tile
-int launch_exscan_i64(int64_t *a, int64_t n, cudaStream_t s);   // in place, a[n] = total
+constexpr int kScanTile = 4096;  // elements of a tile of launch_exscan_i64
+// Exclusive scan in place, a[n] = total; tiles: n / kScanTile + 1 words of scratch.
+int launch_exscan_i64(int64_t *a, int64_t n, int64_t *tiles, cudaStream_t s);
 }  // namespace serbf

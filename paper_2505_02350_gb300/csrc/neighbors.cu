@@ -454,74 +454,132 @@ __global__ void __launch_bounds__(256) k_fine_lists_batch(const RebuildArgs *ra)
 
 // ---------------------------------------------------------------- point-major CSR
 // One warp per tile; lanes are points.  The super cell's list is walked in
-// ascending kernel order (entries whose support misses the tile box are
-// skipped), so each row comes out sorted.
+// ascending kernel order, 32 candidates filtered against the tile box at a
+// time (one per lane), the kernels that reach it handed round by shuffles, so
+// each row comes out sorted.
 template <bool FILL>
-__global__ void k_pmajor(const float *x, const float *y, const float *z, const uint32_t *tile_super,
-                         const uint32_t *tile_start, const float4 *tlo, const float4 *thi, const uint32_t *cell_start,
-                         int cps, int64_t ntiles, const uint32_t *slist, const uint32_t *scnt, int scap,
-                         const float4 *kfwd, int64_t *rowptr, uint32_t *col) {
-    int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) k_pmajor(const float *x, const float *y, const float *z, const uint32_t *tile_super,
+                                                const uint32_t *tile_start, const float4 *tlo, const float4 *thi,
+                                                const uint32_t *cell_start, int cps, int64_t ntiles,
+                                                const uint32_t *slist, const uint32_t *scnt, int scap,
+                                                const float4 *kfwd, int64_t *rowptr, uint32_t *col) {
+    pdl_wait();
+    pdl_trigger();
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (t >= ntiles) return;
-    uint32_t s = tile_super[t], p0 = tile_start[t], pe = cell_start[(int64_t)(s + 1) * cps];
-    int64_t i = (int64_t)p0 + lane;
-    bool valid = i < (int64_t)pe;
-    float px = valid ? x[i] : __int_as_float(0x7fc00000);
-    float py = valid ? y[i] : 0.f, pz = valid ? z[i] : 0.f;
-    float4 lo = tlo[t], hi = thi[t];
-    int L = min((int)scnt[s], scap);
+    const uint32_t s = tile_super[t], p0 = tile_start[t], pe = cell_start[(int64_t)(s + 1) * cps];
+    const int64_t i = (int64_t)p0 + lane;
+    const bool valid = i < (int64_t)pe;
+    const float px = valid ? x[i] : __int_as_float(0x7fc00000);
+    const float py = valid ? y[i] : 0.f, pz = valid ? z[i] : 0.f;
+    const float4 lo = tlo[t], hi = thi[t];
+    const int L = min((int)scnt[s], scap);
     const uint32_t *lst = slist + (size_t)s * scap;
-    int64_t o = FILL && valid ? rowptr[i] : 0;
-    int64_t n = 0;
-    for (int q = 0; q < L; ++q) {
-        uint32_t j = lst[q];
-        float4 k = kfwd[3 * j];
-        if (!(box_d2(k.x, k.y, k.z, lo, hi) < k.w)) continue;
-        if (in_support(px, py, pz, k.x, k.y, k.z, k.w)) {
-            if (FILL) col[o + n] = j;
-            ++n;
+    uint32_t *row = FILL && valid ? col + rowptr[i] : nullptr;
+    uint32_t n = 0;
+    for (int b = 0; b < L; b += 32) {
+        const bool live = b + lane < L;
+        const uint32_t j = live ? lst[b + lane] : 0u;
+        const float4 k = live ? kfwd[3 * (size_t)j] : make_float4(0.f, 0.f, 0.f, -1.f);
+        unsigned hits = __ballot_sync(0xffffffffu, live && box_d2(k.x, k.y, k.z, lo, hi) < k.w);
+        while (hits) {
+            const int q = __ffs(hits) - 1;
+            hits &= hits - 1;
+            const float cx = __shfl_sync(0xffffffffu, k.x, q), cy = __shfl_sync(0xffffffffu, k.y, q);
+            const float cz = __shfl_sync(0xffffffffu, k.z, q), r2 = __shfl_sync(0xffffffffu, k.w, q);
+            const uint32_t jq = __shfl_sync(0xffffffffu, j, q);
+            if (in_support(px, py, pz, cx, cy, cz, r2)) {
+                if (FILL) row[n] = jq;
+                ++n;
+            }
         }
     }
     if (!FILL && valid) rowptr[i] = n;
 }
 
 // ---------------------------------------------------------------- kernel-major CSR
-// One warp per kernel.  Super cells are visited in ascending id, their tiles in
+// kRowParts warps per kernel, each with an equal share of the super cells of
+// the support box.  Super cells are visited in ascending id, their tiles in
 // ascending order and each tile's points in order, which is ascending binned
-// index, so each CSR row comes out sorted.
+// index, so each CSR row comes out sorted: the shares' counts (part) give
+// every warp its place in the row.  One warp per kernel took 1.6 ms for 512
+// kernels on 64^3 (three warps per SM).
+constexpr int kRowParts = 32;
+static_assert(kRowParts == 32 && kRowParts + 4 <= kBwdWarpsPerKernel * 22, "a lane per share; the shares' counts fit the standalone adjoint's moments");
+
 template <bool FILL>
-__global__ void k_kmajor(const float *x, const float *y, const float *z, const float4 *kfwd, const int32_t *m_dev,
-                         serbf_grid g, int sf, int nsx, int nsy, const float4 *slo, const float4 *shi,
-                         const uint32_t *stile0, const uint32_t *tile_start, const float4 *tlo, const float4 *thi,
-                         const uint32_t *cell_start, int cps, int64_t *rowptr, uint32_t *col) {
-    int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) k_kmajor(const float *x, const float *y, const float *z, const float4 *kfwd,
+                                                const int32_t *m_dev, serbf_grid g, int sf, int nsx, int nsy,
+                                                const float4 *slo, const float4 *shi, const uint32_t *stile0,
+                                                const uint32_t *tile_start, const float4 *tlo, const float4 *thi,
+                                                const uint32_t *cell_start, int cps, uint32_t *part,
+                                                const int64_t *rowptr, uint32_t *col) {
+    pdl_wait();
+    pdl_trigger();
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, j = (int)(w / kRowParts), share = (int)(w % kRowParts);
     if (j >= *m_dev) return;
-    float4 k = kfwd[3 * j];
-    KBox b = kernel_box(k.x, k.y, k.z, k.w, g);
-    int64_t base = FILL ? rowptr[j] : 0;
+    const float4 k = kfwd[3 * (size_t)j];
+    const KBox b = kernel_box(k.x, k.y, k.z, k.w, g);
+    const int sx0 = b.kx0 / sf, sy0 = b.ky0 / sf, sz0 = b.kz0 / sf;
+    const int nx = b.kx1 / sf - sx0 + 1, ny = b.ky1 / sf - sy0 + 1, nz = b.kz1 / sf - sz0 + 1;
+    const int64_t all = (int64_t)nx * ny * nz;
+    const int64_t q0 = all * share / kRowParts, q1 = all * (share + 1) / kRowParts;
+    uint32_t *out = FILL ? col + rowptr[j] + part[w] : nullptr;
     uint32_t count = 0;
-    for (int sz = b.kz0 / sf; sz <= b.kz1 / sf; ++sz)
-        for (int sy = b.ky0 / sf; sy <= b.ky1 / sf; ++sy)
-            for (int sx = b.kx0 / sf; sx <= b.kx1 / sf; ++sx) {
-                int s = (sz * nsy + sy) * nsx + sx;
-                if (!(box_d2(k.x, k.y, k.z, slo[s], shi[s]) < k.w)) continue;
-                uint32_t pe_s = cell_start[(int64_t)(s + 1) * cps];
-                for (uint32_t t = stile0[s]; t < stile0[s + 1]; ++t) {
-                    if (!(box_d2(k.x, k.y, k.z, tlo[t], thi[t]) < k.w)) continue;
-                    uint32_t i = tile_start[t] + lane;
-                    bool hit = i < pe_s && in_support(x[i], y[i], z[i], k.x, k.y, k.z, k.w);
-                    unsigned bal = __ballot_sync(0xffffffffu, hit);
-                    if (FILL && hit) col[base + count + __popc(bal & ((1u << lane) - 1u))] = i;
-                    count += __popc(bal);
+    // 32 super cells at a time, one per lane, then 32 tiles of a reached one
+    for (int64_t qb = q0; qb < q1; qb += 32) {
+        const int64_t q = qb + lane;
+        uint32_t t0 = 0, t1 = 0, pe = 0;
+        if (q < q1) {
+            const int s = (int)(((sz0 + q / ((int64_t)nx * ny)) * nsy + sy0 + (q / nx) % ny) * nsx + sx0 + q % nx);
+            if (box_d2(k.x, k.y, k.z, slo[s], shi[s]) < k.w) {
+                t0 = stile0[s];
+                t1 = stile0[s + 1];
+                pe = cell_start[(int64_t)(s + 1) * cps];
+            }
+        }
+        unsigned sup = __ballot_sync(0xffffffffu, t1 > t0);
+        while (sup) {
+            const int src = __ffs(sup) - 1;
+            sup &= sup - 1;
+            const uint32_t a0 = __shfl_sync(0xffffffffu, t0, src), a1 = __shfl_sync(0xffffffffu, t1, src);
+            const uint32_t end = __shfl_sync(0xffffffffu, pe, src);
+            for (uint32_t tb = a0; tb < a1; tb += 32) {
+                const uint32_t t = tb + lane;
+                uint32_t start = 0;
+                bool hit = false;
+                if (t < a1) {
+                    hit = box_d2(k.x, k.y, k.z, tlo[t], thi[t]) < k.w;
+                    start = tile_start[t];
+                }
+                unsigned bal = __ballot_sync(0xffffffffu, hit);
+                while (bal) {
+                    const int ts = __ffs(bal) - 1;
+                    bal &= bal - 1;
+                    const uint32_t i = __shfl_sync(0xffffffffu, start, ts) + lane;
+                    const bool in = i < end && in_support(x[i], y[i], z[i], k.x, k.y, k.z, k.w);
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    if (FILL && in) out[count + __popc(m & ((1u << lane) - 1u))] = i;
+                    count += __popc(m);
                 }
             }
-    if (!FILL && lane == 0) rowptr[j] = count;
+        }
+    }
+    if (!FILL && lane == 0) part[w] = count;
 }
 
-__global__ void k_zero_i64(int64_t *a, int64_t n) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        a[k] = 0;
+// A warp per kernel: its shares' counts become places in the row, its total
+// goes to rowptr[j].
+__global__ void __launch_bounds__(256) k_row_parts(const int32_t *m_dev, uint32_t *part, int64_t *rowptr) {
+    pdl_wait();
+    pdl_trigger();
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (j >= *m_dev) return;
+    const uint32_t v = part[(size_t)j * kRowParts + lane], inc = warp_iscan(v);
+    part[(size_t)j * kRowParts + lane] = inc - v;
+    if (lane == 31) rowptr[j] = inc;
 }
 
 bool ws_ok(const serbf_workspace *ws) { return ws && ws->magic == kMagic && ws->binned; }
@@ -698,15 +756,17 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
     int64_t n = pts->n;
     int64_t total = -1;
     int result = SERBF_OK;
+    // scratch of the explicit lists, idle outside the standalone adjoint
+    uint32_t *part = reinterpret_cast<uint32_t *>(ws->moments);
     if (kmajor) {
-        unsigned blocks = (unsigned)(((int64_t)m * 32 + 255) / 256);
-        k_zero_i64<<<1, 256, 0, s>>>(kmajor->rowptr, (int64_t)m + 1);
-        if (m > 0)
-            k_kmajor<false><<<blocks, 256, 0, s>>>(pts->x, pts->y, pts->z, ws->kfwd, prm->m, ws->grid, ws->sf,
-                                                   ws->ns[0], ws->ns[1], ws->sup_lo, ws->sup_hi, ws->super_tile0,
-                                                   ws->tile_start, ws->tile_lo, ws->tile_hi, ws->cell_start, cps,
-                                                   kmajor->rowptr, nullptr);
-        rc = launch_exscan_i64(kmajor->rowptr, m, s);
+        const unsigned blocks = (unsigned)(((int64_t)m * kRowParts * 32 + 255) / 256);
+        if (m > 0) {
+            launch_pdl(k_kmajor<false>, dim3(blocks), dim3(256), 0, s, pts->x, pts->y, pts->z, ws->kfwd, prm->m, ws->grid,
+                       ws->sf, ws->ns[0], ws->ns[1], ws->sup_lo, ws->sup_hi, ws->super_tile0, ws->tile_start, ws->tile_lo,
+                       ws->tile_hi, ws->cell_start, cps, part, kmajor->rowptr, nullptr);
+            launch_pdl(k_row_parts, dim3((unsigned)((m + 7) / 8)), dim3(256), 0, s, prm->m, part, kmajor->rowptr);
+        }
+        rc = launch_exscan_i64(kmajor->rowptr, m, reinterpret_cast<int64_t *>(part + (size_t)m * kRowParts), s);
         if (rc) return rc;
         int64_t tot = 0;
         if (cudaMemcpyAsync(&tot, kmajor->rowptr + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -715,21 +775,19 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
         total = tot;
         if (tot > kmajor->cap) result = SERBF_ECAPACITY;
         else if (m > 0)
-            k_kmajor<true><<<blocks, 256, 0, s>>>(pts->x, pts->y, pts->z, ws->kfwd, prm->m, ws->grid, ws->sf,
-                                                  ws->ns[0], ws->ns[1], ws->sup_lo, ws->sup_hi, ws->super_tile0,
-                                                  ws->tile_start, ws->tile_lo, ws->tile_hi, ws->cell_start, cps,
-                                                  kmajor->rowptr, kmajor->col);
+            launch_pdl(k_kmajor<true>, dim3(blocks), dim3(256), 0, s, pts->x, pts->y, pts->z, ws->kfwd, prm->m, ws->grid,
+                       ws->sf, ws->ns[0], ws->ns[1], ws->sup_lo, ws->sup_hi, ws->super_tile0, ws->tile_start, ws->tile_lo,
+                       ws->tile_hi, ws->cell_start, cps, part, kmajor->rowptr, kmajor->col);
         SERBF_CHECK_LAUNCH();
     }
     if (pmajor) {
         int64_t nt = ws->ntiles;
-        unsigned blocks = (unsigned)((nt * 32 + 255) / 256);
-        k_zero_i64<<<64, 256, 0, s>>>(pmajor->rowptr, n + 1);
+        const unsigned blocks = (unsigned)((nt * 32 + 255) / 256);
         if (nt > 0)
-            k_pmajor<false><<<blocks, 256, 0, s>>>(pts->x, pts->y, pts->z, ws->tile_super, ws->tile_start,
+            launch_pdl(k_pmajor<false>, dim3(blocks), dim3(256), 0, s, pts->x, pts->y, pts->z, ws->tile_super, ws->tile_start,
                                                    ws->tile_lo, ws->tile_hi, ws->cell_start, cps, nt, ws->sup_list,
                                                    ws->sup_cnt, ws->sz.super_cap, ws->kfwd, pmajor->rowptr, nullptr);
-        rc = launch_exscan_i64(pmajor->rowptr, n, s);
+        rc = launch_exscan_i64(pmajor->rowptr, n, reinterpret_cast<int64_t *>(ws->nz), s);
         if (rc) return rc;
         int64_t tot = 0;
         if (cudaMemcpyAsync(&tot, pmajor->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -738,7 +796,7 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
         total = tot;
         if (tot > pmajor->cap) result = SERBF_ECAPACITY;
         else if (nt > 0)
-            k_pmajor<true><<<blocks, 256, 0, s>>>(pts->x, pts->y, pts->z, ws->tile_super, ws->tile_start,
+            launch_pdl(k_pmajor<true>, dim3(blocks), dim3(256), 0, s, pts->x, pts->y, pts->z, ws->tile_super, ws->tile_start,
                                                   ws->tile_lo, ws->tile_hi, ws->cell_start, cps, nt, ws->sup_list,
                                                   ws->sup_cnt, ws->sz.super_cap, ws->kfwd, pmajor->rowptr,
                                                   pmajor->col);
