@@ -23,9 +23,8 @@ int batch_forward_launch(const void *args, const void *fin, const uint32_t *item
                          int64_t total_items, int64_t finish_blocks, int G, int kahan, int sm_count, cudaStream_t s);
 size_t rebuild_args_size();
 int batch_rebuild_args(const serbf_points *, const serbf_params *, const serbf_config *, serbf_workspace *, void *,
-                       int *, int64_t *, int *, int *);
-int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int nsuper, int two_level,
-                         cudaStream_t s);
+                       int *, int64_t *, int *);
+int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, cudaStream_t s);
 size_t step_args_size();
 int batch_step_args(serbf_params *, const float *, float *, float *, serbf_state *, double *, const serbf_config *,
                     serbf_workspace *, void *, int *);
@@ -78,7 +77,7 @@ struct serbf_batch {
     char *base;
     Layout L;
     int64_t total_items, finish_blocks, chunks;
-    int32_t level1_blocks, nsuper, two_level, step_nb;
+    int32_t level1_blocks, parents, step_nb;
 };
 
 extern "C" {
@@ -100,7 +99,7 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     if (bytes < L.total) return SERBF_ENOMEM;
     std::vector<char> host(L.total, 0);
     int64_t total = 0, fin_blocks = 1, chunks = 0;
-    int lvl1 = 1, nsup = 1, two = 0, step_nb = 1, sm = 0;
+    int lvl1 = 1, parents = 0, step_nb = 1, sm = 0;
     const int kahan = fields[0].cfg ? fields[0].cfg->kahan : 0;
     uint32_t *off = reinterpret_cast<uint32_t *>(host.data() + L.off);
     for (int f = 0; f < nfields; ++f) {
@@ -108,12 +107,12 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
         if (!F.cfg || !F.ws || F.ws->magic != kMagic || !F.ws->binned || F.cfg->kahan != kahan) return SERBF_EINVAL;
         serbf_params prm = F.prm;
         int64_t fb = 1, ch = 0;
-        int l1 = 0, ns = 0, tw = 0, nb = 0;
+        int l1 = 0, pa = 0, nb = 0;
         int rc = batch_forward_args(&F.pts, &F.prm, F.cfg, F.psi, F.err, F.mask, F.grad, F.stats, F.ws,
                                     host.data() + L.fwd + (size_t)f * fwd_args_size(),
                                     host.data() + L.fin + (size_t)f * finish_args_size(), &fb);
         if (!rc) rc = batch_rebuild_args(&F.pts, &F.prm, F.cfg, F.ws, host.data() + L.reb + (size_t)f * rebuild_args_size(),
-                                         &l1, &ch, &ns, &tw);
+                                         &l1, &ch, &pa);
         if (!rc) rc = batch_step_args(&prm, F.grad, F.adam_m, F.adam_v, F.st, F.stats, F.cfg, F.ws,
                                       host.data() + L.step + (size_t)f * step_args_size(), &nb);
         if (!rc) rc = batch_add_args(&F.pts, F.S_raw, F.err, F.mask, &prm, F.adam_m, F.adam_v, F.st, F.stats, F.cfg,
@@ -126,8 +125,7 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
         fin_blocks = fb > fin_blocks ? fb : fin_blocks;
         chunks = ch > chunks ? ch : chunks;
         lvl1 = l1 > lvl1 ? l1 : lvl1;
-        nsup = ns > nsup ? ns : nsup;
-        two |= tw;
+        parents = pa > parents ? pa : parents;
         step_nb = nb > step_nb ? nb : step_nb;
         sm = F.ws->sm_count;
     }
@@ -147,8 +145,7 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     b->finish_blocks = fin_blocks;
     b->chunks = chunks;
     b->level1_blocks = lvl1;
-    b->nsuper = nsup;
-    b->two_level = two;
+    b->parents = parents;
     b->step_nb = step_nb;
     return SERBF_OK;
 }
@@ -160,7 +157,7 @@ int serbf_epoch_batched(serbf_batch *b, void *stream) {
     if (!b || b->magic != kBatchMagic) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     char *d = b->base;
-    int rc = batch_rebuild_launch(d + b->L.reb, b->nfields, b->level1_blocks, b->chunks, b->nsuper, b->two_level, s);
+    int rc = batch_rebuild_launch(d + b->L.reb, b->nfields, b->level1_blocks, b->chunks, b->parents, s);
     if (!rc)
         rc = batch_forward_launch(d + b->L.fwd, d + b->L.fin, reinterpret_cast<const uint32_t *>(d + b->L.off),
                                   b->nfields, reinterpret_cast<uint32_t *>(d + b->L.ctr), b->total_items,

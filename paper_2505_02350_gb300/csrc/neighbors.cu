@@ -140,15 +140,96 @@ __global__ void __launch_bounds__(kOrderChunk) k_order_items(const uint8_t *item
     order_items_body(item_class, hist, item_rec, order_rec, nitems, blockIdx.x);
 }
 
+// Ascending list of the kernels that pass `hit`, by one block of
+// kListThreads: a warp tests 128 consecutive candidates of each 1024 (four
+// ballots), the warps' counts meet in shared memory (double-buffered: one
+// barrier per 1024 candidates, where a block scan of every 256 took three: the
+// first level of 9.4 M points and 16384 kernels 71 -> 62 us).
+// Returns the count; entries beyond scap are not written.
+constexpr int kListThreads = 256;
+constexpr int kListWarps = kListThreads / 32;
+
+template <typename F>
+__device__ __forceinline__ uint32_t list_block(int m, uint32_t *out, int scap, F hit) {
+    __shared__ uint32_t s_cnt[2][kListWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t count = 0;
+    int buf = 0;
+    for (int j0 = 0; j0 < m; j0 += 4 * kListThreads, buf ^= 1) {
+        const int jw = j0 + 128 * warp + lane;
+        unsigned bal[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) bal[r] = __ballot_sync(0xffffffffu, jw + 32 * r < m && hit(jw + 32 * r));
+        if (lane == 0) s_cnt[buf][warp] = __popc(bal[0]) + __popc(bal[1]) + __popc(bal[2]) + __popc(bal[3]);
+        __syncthreads();
+        uint32_t at = count;
+#pragma unroll
+        for (int w = 0; w < kListWarps; ++w) {
+            const uint32_t c = s_cnt[buf][w];
+            at += w < warp ? c : 0u;
+            count += c;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const uint32_t o = at + __popc(bal[r] & lt);
+            if (((bal[r] >> lane) & 1u) && o < (uint32_t)scap) out[o] = (uint32_t)(jw + 32 * r);
+            at += __popc(bal[r]);
+        }
+    }
+    return count;
+}
+
+// Union of the boxes of the f x f x f super cells of block (cx, cy, cz).
+__device__ __forceinline__ void block_box(const float4 *slo, const float4 *shi, int nsx, int nsy, int nsz, int cx, int cy,
+                                          int cz, int f, float4 &lo, float4 &hi) {
+    lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+    for (int dz = 0; dz < f; ++dz)
+        for (int dy = 0; dy < f; ++dy)
+            for (int dx = 0; dx < f; ++dx) {
+                const int sx = f * cx + dx, sy = f * cy + dy, sz = f * cz + dz;
+                if (sx >= nsx || sy >= nsy || sz >= nsz) continue;
+                const int sc = (sz * nsy + sy) * nsx + sx;
+                const float4 a = slo[sc], b = shi[sc];
+                lo = make_float4(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z), 0.f);
+                hi = make_float4(fmaxf(hi.x, b.x), fmaxf(hi.y, b.y), fmaxf(hi.z, b.z), 0.f);
+            }
+}
+
+// The kernels of the parameter block whose support may reach a box (centre
+// and r2 by the same float operations as the records).
+__device__ __forceinline__ uint32_t list_params(const float *p, int cap, int m, float nle, float4 lo, float4 hi,
+                                                uint32_t *out, int scap) {
+    return list_block(m, out, scap, [&](int j) {
+        const float r2 = support_r2(p[PD1 * cap + j], p[PD2 * cap + j], p[PD3 * cap + j], nle);
+        return box_d2(p[PCX * cap + j], p[PCY * cap + j], p[PCZ * cap + j], lo, hi) < r2;
+    });
+}
+
+// The same for a list that is filtered again with the records: the test is
+// multiplied through by the least d^2 instead of dividing by it, with slack for
+// the rounding of either side, so it keeps every kernel of list_params and
+// perhaps one that just misses the box (that first level 62 -> 47 us).
+__device__ __forceinline__ uint32_t list_params_about(const float *p, int cap, int m, float nle, float4 lo, float4 hi,
+                                                      uint32_t *out, int scap) {
+    const float lim = 1.00001f * nle;
+    return list_block(m, out, scap, [&](int j) {
+        const float d1 = p[PD1 * cap + j], d2 = p[PD2 * cap + j], d3 = p[PD3 * cap + j];
+        float lam = d1 * d1;
+        if (d2 * d2 < lam) lam = d2 * d2;
+        if (d3 * d3 < lam) lam = d3 * d3;
+        return box_d2(p[PCX * cap + j], p[PCY * cap + j], p[PCZ * cap + j], lo, hi) * lam < lim;
+    });
+}
+
 // The per-step rebuild in one launch: blocks [0, nsuper) list, per super
-// cell, every kernel whose support may reach its box (centre and r2 taken
-// from the parameters with the same float operations as the records); the
-// remaining blocks write the per-kernel records.
+// cell, every kernel whose support may reach its box; the remaining blocks
+// write the per-kernel records.
 __device__ __forceinline__ void rebuild_body(const float *p, int cap, const int32_t *m_dev, float nle, float4 *kfwd,
                                              float4 *kbwd, const float4 *slo, const float4 *shi, int nsuper,
                                              uint32_t *list, uint32_t *cnt, int scap, int32_t *status,
                                              long long *needed, int bx, int nbx) {
-    __shared__ uint32_t tmp[33];
     const int m = *m_dev;
     const int s = bx;
     if (s >= nsuper) {
@@ -161,20 +242,7 @@ __device__ __forceinline__ void rebuild_body(const float *p, int cap, const int3
         if (threadIdx.x == 0) cnt[s] = 0;
         return;
     }
-    uint32_t count = 0;
-    uint32_t *out = list + (size_t)s * scap;
-    for (int j0 = 0; j0 < m; j0 += 256) {
-        const int j = j0 + threadIdx.x;
-        uint32_t hit = 0;
-        if (j < m) {
-            const float r2 = support_r2(p[PD1 * cap + j], p[PD2 * cap + j], p[PD3 * cap + j], nle);
-            hit = box_d2(p[PCX * cap + j], p[PCY * cap + j], p[PCZ * cap + j], lo, hi) < r2;
-        }
-        uint32_t tot;
-        const uint32_t off = block_exscan(hit, tmp, &tot);
-        if (hit && count + off < (uint32_t)scap) out[count + off] = (uint32_t)j;
-        count += tot;
-    }
+    const uint32_t count = list_params(p, cap, m, nle, lo, hi, list + (size_t)s * scap, scap);
     if (threadIdx.x == 0) {
         cnt[s] = count;
         if (count > (uint32_t)scap) {
@@ -184,17 +252,17 @@ __device__ __forceinline__ void rebuild_body(const float *p, int cap, const int3
     }
 }
 
-__global__ void __launch_bounds__(256) k_rebuild(const float *p, int cap, const int32_t *m_dev, float nle,
-                                                 float4 *kfwd, float4 *kbwd, const float4 *slo, const float4 *shi,
-                                                 int nsuper, uint32_t *list, uint32_t *cnt, int scap, int32_t *status,
-                                                 long long *needed) {
+__global__ void __launch_bounds__(kListThreads) k_rebuild(const float *p, int cap, const int32_t *m_dev, float nle,
+                                                          float4 *kfwd, float4 *kbwd, const float4 *slo, const float4 *shi,
+                                                          int nsuper, uint32_t *list, uint32_t *cnt, int scap,
+                                                          int32_t *status, long long *needed) {
     pdl_wait();
     pdl_trigger();
     rebuild_body(p, cap, m_dev, nle, kfwd, kbwd, slo, shi, nsuper, list, cnt, scap, status, needed, blockIdx.x,
                  gridDim.x);
 }
 
-// Two-level rebuild, for many super cells and kernels.  First launch: blocks
+// Rebuild in levels, for many super cells and kernels.  First launch: blocks
 // [0, ncoarse) list, per block of f x f x f super cells (f = 2; 4 for the
 // first of three levels), every kernel whose support may reach the union of
 // their boxes (as k_rebuild does per super cell); the remaining blocks write
@@ -203,7 +271,6 @@ __device__ __forceinline__ void coarse_lists_body(const float *p, int cap, const
                                                   float4 *kfwd, float4 *kbwd, const float4 *slo, const float4 *shi,
                                                   int nsx, int nsy, int nsz, int ncoarse, uint32_t *list,
                                                   uint32_t *cnt, int scap, int bx, int nbx, int f) {
-    __shared__ uint32_t tmp[33];
     __shared__ float4 s_lo, s_hi;
     const int m = *m_dev;
     const int c = bx;
@@ -214,20 +281,7 @@ __device__ __forceinline__ void coarse_lists_body(const float *p, int cap, const
     }
     if (threadIdx.x == 0) {
         const int ncx = (nsx + f - 1) / f, ncy = (nsy + f - 1) / f;
-        const int cx = c % ncx, cy = (c / ncx) % ncy, cz = c / (ncx * ncy);
-        float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f), hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
-        for (int dz = 0; dz < f; ++dz)
-            for (int dy = 0; dy < f; ++dy)
-                for (int dx = 0; dx < f; ++dx) {
-                    const int sx = f * cx + dx, sy = f * cy + dy, sz = f * cz + dz;
-                    if (sx >= nsx || sy >= nsy || sz >= nsz) continue;
-                    const int sc = (sz * nsy + sy) * nsx + sx;
-                    const float4 a = slo[sc], b = shi[sc];
-                    lo = make_float4(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z), 0.f);
-                    hi = make_float4(fmaxf(hi.x, b.x), fmaxf(hi.y, b.y), fmaxf(hi.z, b.z), 0.f);
-                }
-        s_lo = lo;
-        s_hi = hi;
+        block_box(slo, shi, nsx, nsy, nsz, c % ncx, (c / ncx) % ncy, c / (ncx * ncy), f, s_lo, s_hi);
     }
     __syncthreads();
     const float4 lo = s_lo, hi = s_hi;
@@ -235,159 +289,118 @@ __device__ __forceinline__ void coarse_lists_body(const float *p, int cap, const
         if (threadIdx.x == 0) cnt[c] = 0;
         return;
     }
-    uint32_t count = 0;
-    uint32_t *out = list + (size_t)c * scap;
-    for (int j0 = 0; j0 < m; j0 += 256) {
-        const int j = j0 + threadIdx.x;
-        uint32_t hit = 0;
-        if (j < m) {
-            const float r2 = support_r2(p[PD1 * cap + j], p[PD2 * cap + j], p[PD3 * cap + j], nle);
-            hit = box_d2(p[PCX * cap + j], p[PCY * cap + j], p[PCZ * cap + j], lo, hi) < r2;
-        }
-        uint32_t tot;
-        const uint32_t off = block_exscan(hit, tmp, &tot);
-        if (hit && count + off < (uint32_t)scap) out[count + off] = (uint32_t)j;
-        count += tot;
-    }
+    const uint32_t count = list_params_about(p, cap, m, nle, lo, hi, list + (size_t)c * scap, scap);
     if (threadIdx.x == 0) cnt[c] = count;
 }
 
-__global__ void __launch_bounds__(256) k_coarse_lists(const float *p, int cap, const int32_t *m_dev, float nle,
-                                                      float4 *kfwd, float4 *kbwd, const float4 *slo,
-                                                      const float4 *shi, int nsx, int nsy, int nsz, int ncoarse,
-                                                      uint32_t *list, uint32_t *cnt, int scap, int f) {
+__global__ void __launch_bounds__(kListThreads) k_coarse_lists(const float *p, int cap, const int32_t *m_dev, float nle,
+                                                               float4 *kfwd, float4 *kbwd, const float4 *slo,
+                                                               const float4 *shi, int nsx, int nsy, int nsz, int ncoarse,
+                                                               uint32_t *list, uint32_t *cnt, int scap, int f) {
     pdl_wait();
     pdl_trigger();
     coarse_lists_body(p, cap, m_dev, nle, kfwd, kbwd, slo, shi, nsx, nsy, nsz, ncoarse, list, cnt, scap, blockIdx.x,
                       gridDim.x, f);
 }
 
-// Middle of three levels: each block of 2 x 2 x 2 super cells keeps the
-// kernels of its parent's list (blocks of 4 x 4 x 4 super cells) that reach
-// its own box, tested with the records' centre and r2; a parent list that
-// overflowed is not used (every kernel is tested).  A kernel that reaches a
-// box reaches every box containing it, so the lists equal the one-level ones
-// filtered to these blocks.
-__device__ __forceinline__ void mid_lists_body(const int32_t *m_dev, const float4 *kfwd, const float4 *slo,
-                                               const float4 *shi, int nsx, int nsy, int nsz, int nmid,
-                                               const uint32_t *plist, const uint32_t *pcnt, uint32_t *list,
-                                               uint32_t *cnt, int scap, int bx) {
-    __shared__ uint32_t tmp[33];
-    __shared__ float4 s_lo, s_hi;
-    const int c = bx;
-    if (c >= nmid) return;
-    const int ncx = (nsx + 1) >> 1, ncy = (nsy + 1) >> 1;
-    const int cx = c % ncx, cy = (c / ncx) % ncy, cz = c / (ncx * ncy);
-    if (threadIdx.x == 0) {
-        float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f), hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
-        for (int dz = 0; dz < 2; ++dz)
-            for (int dy = 0; dy < 2; ++dy)
-                for (int dx = 0; dx < 2; ++dx) {
-                    const int sx = 2 * cx + dx, sy = 2 * cy + dy, sz = 2 * cz + dz;
-                    if (sx >= nsx || sy >= nsy || sz >= nsz) continue;
-                    const int sc = (sz * nsy + sy) * nsx + sx;
-                    const float4 a = slo[sc], b = shi[sc];
-                    lo = make_float4(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z), 0.f);
-                    hi = make_float4(fmaxf(hi.x, b.x), fmaxf(hi.y, b.y), fmaxf(hi.z, b.z), 0.f);
-                }
-        s_lo = lo;
-        s_hi = hi;
-    }
-    __syncthreads();
-    const float4 lo = s_lo, hi = s_hi;
-    if (!(lo.x <= hi.x)) {
-        if (threadIdx.x == 0) cnt[c] = 0;
-        return;
-    }
-    const int npx = (nsx + 3) >> 2, npy = (nsy + 3) >> 2;
-    const int pc = ((cz >> 1) * npy + (cy >> 1)) * npx + (cx >> 1);
-    const uint32_t pn = pcnt[pc];
-    const bool whole = pn > (uint32_t)scap;  // the parent's list overflowed
-    const int L = whole ? *m_dev : (int)pn;
-    const uint32_t *src = plist + (size_t)pc * scap;
-    uint32_t count = 0;
-    uint32_t *out = list + (size_t)c * scap;
-    for (int q0 = 0; q0 < L; q0 += 256) {
-        const int q = q0 + threadIdx.x;
-        uint32_t hit = 0, j = 0;
-        if (q < L) {
-            j = whole ? (uint32_t)q : src[q];
-            const float4 k = kfwd[3 * j];
-            hit = box_d2(k.x, k.y, k.z, lo, hi) < k.w;
+// Next levels: one block per parent (a block of super cells), one warp per
+// child (2 x 2 x 2 of them).  The parent's candidates are fetched once for all
+// eight children, 256 at a time, into shared memory; each warp keeps those
+// that reach its child's box, tested with the records' centre and r2 (the
+// values k_rebuild computes), 32 at a time and without a block scan.  A kernel
+// that reaches a box reaches every box containing it, so the lists equal the
+// one-level ones; a parent list that overflowed is not used (every kernel is
+// tested).  With a block per child and a scan per 256 candidates the last two
+// levels took 106 us of an epoch of 9.4 M points (32768 super cells), now 42.
+// FINE: children are super cells, and their overflow is reported; otherwise
+// they are blocks of 2 x 2 x 2 super cells.
+struct ChildArgs {
+    const int32_t *m_dev;
+    const float4 *kfwd, *slo, *shi;
+    int nsx, nsy, nsz;
+    const uint32_t *plist, *pcnt;
+    uint32_t *list, *cnt;
+    int scap;
+    int32_t *status;
+    long long *needed;
+};
+
+template <bool FINE>
+__device__ __forceinline__ void child_lists_body(const ChildArgs &a, int p) {
+    __shared__ float4 s_k[kListThreads];
+    __shared__ uint32_t s_j[kListThreads];
+    static_assert(kListWarps == 8, "a warp per child");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    // grid of the children and of their parents
+    const int nx = FINE ? a.nsx : (a.nsx + 1) >> 1, ny = FINE ? a.nsy : (a.nsy + 1) >> 1;
+    const int nz = FINE ? a.nsz : (a.nsz + 1) >> 1;
+    const int px = (nx + 1) >> 1, py = (ny + 1) >> 1;
+    const int cx = 2 * (p % px) + (warp & 1), cy = 2 * ((p / px) % py) + ((warp >> 1) & 1), cz = 2 * (p / (px * py)) + (warp >> 2);
+    const bool child = cx < nx && cy < ny && cz < nz;
+    const int c = child ? (cz * ny + cy) * nx + cx : 0;
+    float4 lo, hi;
+    if (FINE) {
+        lo = a.slo[c];
+        hi = a.shi[c];
+    } else {
+        // a lane per super cell of the child
+        const int sx = 2 * cx + (lane & 1), sy = 2 * cy + ((lane >> 1) & 1), sz = 2 * cz + ((lane >> 2) & 1);
+        const bool in = child && sx < a.nsx && sy < a.nsy && sz < a.nsz;
+        const int s = in ? (sz * a.nsy + sy) * a.nsx + sx : 0;
+        lo = in ? a.slo[s] : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+        hi = in ? a.shi[s] : make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+            lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+            lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+            hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+            hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+            hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
         }
-        uint32_t tot;
-        const uint32_t off = block_exscan(hit, tmp, &tot);
-        if (hit && count + off < (uint32_t)scap) out[count + off] = j;
-        count += tot;
     }
-    if (threadIdx.x == 0) cnt[c] = count;
+    const bool any = child && lo.x <= hi.x;  // the child holds points
+    const uint32_t pn = a.pcnt[p];
+    const bool whole = pn > (uint32_t)a.scap;
+    const int L = whole ? *a.m_dev : (int)pn;
+    const uint32_t *src = a.plist + (size_t)p * a.scap;
+    uint32_t *out = a.list + (size_t)c * a.scap;
+    uint32_t count = 0;
+    for (int q0 = 0; q0 < L; q0 += kListThreads) {
+        __syncthreads();
+        const int q = q0 + threadIdx.x;
+        if (q < L) {
+            const uint32_t j = whole ? (uint32_t)q : src[q];
+            s_j[threadIdx.x] = j;
+            s_k[threadIdx.x] = a.kfwd[3 * (size_t)j];
+        }
+        __syncthreads();
+        if (!any) continue;
+        const int n = min(kListThreads, L - q0);
+        for (int b = 0; b < n; b += 32) {
+            const float4 k = s_k[b + lane];
+            const bool hit = b + lane < n && box_d2(k.x, k.y, k.z, lo, hi) < k.w;
+            const unsigned bal = __ballot_sync(0xffffffffu, hit);
+            const uint32_t o = count + __popc(bal & lt);
+            if (hit && o < (uint32_t)a.scap) out[o] = s_j[b + lane];
+            count += __popc(bal);
+        }
+    }
+    if (child && lane == 0) {
+        a.cnt[c] = count;
+        if (FINE && count > (uint32_t)a.scap) {
+            atomicOr(a.status, SERBF_FLAG_SUPER_LIST);
+            atomicMax(a.needed + 0, (long long)count);
+        }
+    }
 }
 
-__global__ void __launch_bounds__(256) k_mid_lists(const int32_t *m_dev, const float4 *kfwd, const float4 *slo,
-                                                   const float4 *shi, int nsx, int nsy, int nsz, int nmid,
-                                                   const uint32_t *plist, const uint32_t *pcnt, uint32_t *list,
-                                                   uint32_t *cnt, int scap) {
+template <bool FINE>
+__global__ void __launch_bounds__(kListThreads) k_child_lists(ChildArgs a) {
     pdl_wait();
     pdl_trigger();
-    mid_lists_body(m_dev, kfwd, slo, shi, nsx, nsy, nsz, nmid, plist, pcnt, list, cnt, scap, blockIdx.x);
-}
-
-// Second launch: each super cell keeps the kernels of its block's list that
-// reach its own box, with the centre and r2 of the records (the values
-// k_rebuild computes), so the lists equal the one-level ones: a kernel that
-// reaches a super cell's box reaches the block's box, which contains it.  A
-// block list that overflowed is not used: its super cells test every kernel.
-__device__ __forceinline__ void fine_lists_body(const int32_t *m_dev, const float4 *kfwd, const float4 *slo,
-                                                const float4 *shi, int nsx, int nsy, int nsuper, const uint32_t *clist,
-                                                const uint32_t *ccnt, uint32_t *list, uint32_t *cnt, int scap,
-                                                int32_t *status, long long *needed, int bx) {
-    __shared__ uint32_t tmp[33];
-    const int s = bx;
-    if (s >= nsuper) return;
-    const float4 lo = slo[s], hi = shi[s];
-    if (!(lo.x <= hi.x)) {
-        if (threadIdx.x == 0) cnt[s] = 0;
-        return;
-    }
-    const int sx = s % nsx, sy = (s / nsx) % nsy, sz = s / (nsx * nsy);
-    const int ncx = (nsx + 1) >> 1, ncy = (nsy + 1) >> 1;
-    const int c = ((sz >> 1) * ncy + (sy >> 1)) * ncx + (sx >> 1);
-    const uint32_t cc = ccnt[c];
-    const bool whole = cc > (uint32_t)scap;  // the block's list overflowed
-    const int L = whole ? *m_dev : (int)cc;
-    const uint32_t *src = clist + (size_t)c * scap;
-    uint32_t count = 0;
-    uint32_t *out = list + (size_t)s * scap;
-    for (int q0 = 0; q0 < L; q0 += 256) {
-        const int q = q0 + threadIdx.x;
-        uint32_t hit = 0, j = 0;
-        if (q < L) {
-            j = whole ? (uint32_t)q : src[q];
-            const float4 k = kfwd[3 * j];
-            hit = box_d2(k.x, k.y, k.z, lo, hi) < k.w;
-        }
-        uint32_t tot;
-        const uint32_t off = block_exscan(hit, tmp, &tot);
-        if (hit && count + off < (uint32_t)scap) out[count + off] = j;
-        count += tot;
-    }
-    if (threadIdx.x == 0) {
-        cnt[s] = count;
-        if (count > (uint32_t)scap) {
-            atomicOr(status, SERBF_FLAG_SUPER_LIST);
-            atomicMax(needed + 0, (long long)count);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256) k_fine_lists(const int32_t *m_dev, const float4 *kfwd, const float4 *slo,
-                                                    const float4 *shi, int nsx, int nsy, int nsuper,
-                                                    const uint32_t *clist, const uint32_t *ccnt, uint32_t *list,
-                                                    uint32_t *cnt, int scap, int32_t *status, long long *needed) {
-    pdl_wait();
-    pdl_trigger();
-    fine_lists_body(m_dev, kfwd, slo, shi, nsx, nsy, nsuper, clist, ccnt, list, cnt, scap, status, needed,
-                    blockIdx.x);
+    child_lists_body<FINE>(a, blockIdx.x);
 }
 
 // ---------------------------------------------------------------- batches of fields
@@ -429,7 +442,7 @@ __global__ void __launch_bounds__(kOrderChunk) k_order_items_batch(const Rebuild
 
 // First rebuild launch: one-level fields rebuild, two-level fields list the
 // kernels of their blocks of 2 x 2 x 2 super cells; both write the records.
-__global__ void __launch_bounds__(256) k_rebuild_batch(const RebuildArgs *ra) {
+__global__ void __launch_bounds__(kListThreads) k_rebuild_batch(const RebuildArgs *ra) {
     pdl_wait();
     pdl_trigger();
     const RebuildArgs &r = ra[blockIdx.y];
@@ -443,13 +456,14 @@ __global__ void __launch_bounds__(256) k_rebuild_batch(const RebuildArgs *ra) {
 }
 
 // Second rebuild launch: the super-cell lists of two-level fields.
-__global__ void __launch_bounds__(256) k_fine_lists_batch(const RebuildArgs *ra) {
+__global__ void __launch_bounds__(kListThreads) k_fine_lists_batch(const RebuildArgs *ra) {
     pdl_wait();
     pdl_trigger();
     const RebuildArgs &r = ra[blockIdx.y];
-    if (!r.two_level || (int)blockIdx.x >= r.nsuper) return;
-    fine_lists_body(r.m_dev, r.kfwd, r.slo, r.shi, r.nsx, r.nsy, r.nsuper, r.clist, r.ccnt, r.list, r.cnt, r.scap,
-                    r.status, r.needed, blockIdx.x);
+    if (!r.two_level || (int)blockIdx.x >= r.ncoarse) return;
+    child_lists_body<true>(ChildArgs{r.m_dev, r.kfwd, r.slo, r.shi, r.nsx, r.nsy, r.nsz, r.clist, r.ccnt, r.list, r.cnt,
+                                     r.scap, r.status, r.needed},
+                           blockIdx.x);
 }
 
 // ---------------------------------------------------------------- point-major CSR
@@ -612,11 +626,10 @@ namespace serbf {
 size_t rebuild_args_size() { return sizeof(RebuildArgs); }
 
 // Host record of one field's neighbour rebuild for a batch (out:
-// sizeof(RebuildArgs) bytes); *level1_blocks, *chunks and *nsuper size the
-// batch's grids, *two_level says which form the field takes.
+// sizeof(RebuildArgs) bytes); *level1_blocks, *chunks and *parents (blocks of
+// super cells of a field that takes two levels, else 0) size the batch's grids.
 int batch_rebuild_args(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg,
-                       serbf_workspace *ws, void *out, int *level1_blocks, int64_t *chunks, int *nsuper,
-                       int *two_level) {
+                       serbf_workspace *ws, void *out, int *level1_blocks, int64_t *chunks, int *parents) {
     if (!pts || !prm || !cfg || !ws_ok(ws)) return SERBF_EINVAL;
     if (!prm->p || !prm->m || prm->cap < 1 || prm->cap > ws->sz.max_kernels) return SERBF_EINVAL;
     if (pts->n != ws->npoints) return SERBF_EINVAL;
@@ -656,22 +669,20 @@ int batch_rebuild_args(const serbf_points *pts, const serbf_params *prm, const s
     memcpy(out, &r, sizeof(r));
     *level1_blocks = r.level1_blocks;
     *chunks = (ws->nitems + kOrderChunk - 1) / kOrderChunk;
-    *nsuper = ws->nsuper;
-    *two_level = r.two_level;
+    *parents = r.two_level ? r.ncoarse : 0;
     return SERBF_OK;
 }
 
 // The batched rebuild: item order (two launches), then the lists and
 // records (one launch, two when some field takes two levels).
-int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int nsuper, int two_level,
-                         cudaStream_t s) {
+int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, cudaStream_t s) {
     const RebuildArgs *ra = static_cast<const RebuildArgs *>(args);
     if (chunks > 0) {
         k_class_count_batch<<<dim3((unsigned)chunks, (unsigned)nfields), kOrderChunk, 0, s>>>(ra);
         k_order_items_batch<<<dim3((unsigned)chunks, (unsigned)nfields), kOrderChunk, 0, s>>>(ra);
     }
-    launch_pdl(k_rebuild_batch, dim3((unsigned)level1_blocks, (unsigned)nfields), dim3(256), 0, s, ra);
-    if (two_level) launch_pdl(k_fine_lists_batch, dim3((unsigned)nsuper, (unsigned)nfields), dim3(256), 0, s, ra);
+    launch_pdl(k_rebuild_batch, dim3((unsigned)level1_blocks, (unsigned)nfields), dim3(kListThreads), 0, s, ra);
+    if (parents) launch_pdl(k_fine_lists_batch, dim3((unsigned)parents, (unsigned)nfields), dim3(kListThreads), 0, s, ra);
     SERBF_CHECK_LAUNCH();
     return SERBF_OK;
 }
@@ -713,26 +724,24 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
                 // blocks of 4 x 4 x 4 super cells against every kernel (their
                 // lists and counts held in the super cells' storage, which the
                 // last level rewrites), then blocks of 2 x 2 x 2
-                launch_pdl(k_coarse_lists, dim3((unsigned)(ntop + prep_blocks)), dim3(256), 0, s,
+                launch_pdl(k_coarse_lists, dim3((unsigned)(ntop + prep_blocks)), dim3(kListThreads), 0, s,
                            (const float *)prm->p, prm->cap, (const int32_t *)prm->m, nle, ws->kfwd, ws->kbwd,
                            (const float4 *)ws->sup_lo, (const float4 *)ws->sup_hi, nsx, nsy, nsz, (int)ntop,
                            ws->sup_list, ws->sup_cnt, ws->sz.super_cap, 4);
-                launch_pdl(k_mid_lists, dim3((unsigned)ncoarse), dim3(256), 0, s, (const int32_t *)prm->m,
-                           (const float4 *)ws->kfwd, (const float4 *)ws->sup_lo, (const float4 *)ws->sup_hi, nsx, nsy,
-                           nsz, (int)ncoarse, (const uint32_t *)ws->sup_list, (const uint32_t *)ws->sup_cnt,
-                           ws->crs_list, ws->crs_cnt, ws->sz.super_cap);
+                launch_pdl(k_child_lists<false>, dim3((unsigned)ntop), dim3(kListThreads), 0, s,
+                           ChildArgs{prm->m, ws->kfwd, ws->sup_lo, ws->sup_hi, nsx, nsy, nsz, ws->sup_list, ws->sup_cnt,
+                                     ws->crs_list, ws->crs_cnt, ws->sz.super_cap, ws->status, ws->needed});
             } else {
-                launch_pdl(k_coarse_lists, dim3((unsigned)(ncoarse + prep_blocks)), dim3(256), 0, s,
+                launch_pdl(k_coarse_lists, dim3((unsigned)(ncoarse + prep_blocks)), dim3(kListThreads), 0, s,
                            (const float *)prm->p, prm->cap, (const int32_t *)prm->m, nle, ws->kfwd, ws->kbwd,
                            (const float4 *)ws->sup_lo, (const float4 *)ws->sup_hi, nsx, nsy, nsz, (int)ncoarse,
                            ws->crs_list, ws->crs_cnt, ws->sz.super_cap, 2);
             }
-            launch_pdl(k_fine_lists, dim3(ws->nsuper), dim3(256), 0, s, (const int32_t *)prm->m,
-                       (const float4 *)ws->kfwd, (const float4 *)ws->sup_lo, (const float4 *)ws->sup_hi, nsx, nsy,
-                       ws->nsuper, (const uint32_t *)ws->crs_list, (const uint32_t *)ws->crs_cnt, ws->sup_list,
-                       ws->sup_cnt, ws->sz.super_cap, ws->status, ws->needed);
+            launch_pdl(k_child_lists<true>, dim3((unsigned)ncoarse), dim3(kListThreads), 0, s,
+                       ChildArgs{prm->m, ws->kfwd, ws->sup_lo, ws->sup_hi, nsx, nsy, nsz, ws->crs_list, ws->crs_cnt,
+                                 ws->sup_list, ws->sup_cnt, ws->sz.super_cap, ws->status, ws->needed});
         } else {
-            launch_pdl(k_rebuild, dim3(ws->nsuper + prep_blocks), dim3(256), 0, s, (const float *)prm->p, prm->cap,
+            launch_pdl(k_rebuild, dim3(ws->nsuper + prep_blocks), dim3(kListThreads), 0, s, (const float *)prm->p, prm->cap,
                        (const int32_t *)prm->m, nle, ws->kfwd, ws->kbwd, (const float4 *)ws->sup_lo,
                        (const float4 *)ws->sup_hi, ws->nsuper, ws->sup_list, ws->sup_cnt, ws->sz.super_cap,
                        ws->status, ws->needed);
