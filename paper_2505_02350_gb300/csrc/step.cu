@@ -15,23 +15,31 @@ namespace {
 
 constexpr int kStepThreads = 256;
 
-// Block sums of NV float values with float-float trees (FP64 is slow here).
+// Block sums of NV doubles, in a fixed order.
 template <int NV>
-__device__ void block_sums_ff(const float (&v)[NV], ff (*sh)[NV], ff (&out)[NV]) {
+__device__ void block_sums(const double (&v)[3], double (*sh)[3], double (&out)[3]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double t[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const ff s = warp_sum_ff(ff{v[k], 0.f});
-        if (lane == 0) sh[warp][k] = s;
-    }
+    for (int k = 0; k < NV; ++k) t[k] = v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        if (lane == 0) sh[warp][k] = t[k];
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            ff t = lane < nw ? sh[lane][k] : ff{0.f, 0.f};
-            t = warp_sum_ff(t);
-            if (lane == 0) sh[32][k] = t;
-        }
+        for (int k = 0; k < NV; ++k) t[k] = lane < nw ? sh[lane][k] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            if (lane == 0) sh[32][k] = t[k];
     }
     __syncthreads();
 #pragma unroll
@@ -39,27 +47,13 @@ __device__ void block_sums_ff(const float (&v)[NV], ff (*sh)[NV], ff (&out)[NV])
     __syncthreads();
 }
 
-// Block sums of three doubles, in a fixed order.
-__device__ void block_sums_d3(const double (&v)[3], double (*sh)[3], double (&out)[3]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const double s = warp_sum(v[k]);
-        if (lane == 0) sh[warp][k] = s;
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            double t = lane < nw ? sh[lane][k] : 0.0;
-            t = warp_sum(t);
-            if (lane == 0) sh[32][k] = t;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 3; ++k) out[k] = sh[32][k];
-    __syncthreads();
+// |w| alone while the L1 term is off (its two other sums are zero).
+__device__ __forceinline__ void block_sums_d3(bool use_l1, const double (&v)[3], double (*sh)[3], double (&out)[3]) {
+    out[1] = out[2] = 0.0;
+    if (use_l1)
+        block_sums<3>(v, sh, out);
+    else
+        block_sums<1>(v, sh, out);
 }
 
 __device__ __forceinline__ float sgnf(float v) { return (float)((v > 0.f) - (v < 0.f)); }
@@ -74,8 +68,9 @@ struct StepArgs {
     double *stats;
     serbf_config c;
     float *part;      // per block partial sums
-    double *scal;     // alpha, beta, bias corrections for the update kernel
-    uint32_t *counter;
+    double *scal;     // alpha, beta, bias corrections, learning rate for the update kernel
+    uint32_t *counter; // [0], [1]: blocks done in the two launches
+    uint32_t *bf;      // weights that stay, summed over the blocks (zero between launches)
 };
 
 constexpr int kStateWords = (int)(sizeof(serbf_state) / 4);
@@ -95,20 +90,25 @@ __device__ __forceinline__ void alpha_terms(const StepArgs &a, int j, bool use_l
     }
 }
 
+// The Adam bias corrections feed a float update: float powers (a double pow
+// costs microseconds on this part's FP64 unit).
+__device__ __forceinline__ void bias_corrections(const StepArgs &a, float &b1, float &b2) {
+    const float t = (float)(a.st->adam_t + 1);
+    b1 = 1.0f - powf((float)a.c.beta1, t);
+    b2 = 1.0f - powf((float)a.c.beta2, t);
+}
+
 // alpha of Eq. 3-21 in double (clamped to [0, 1]; 1 when the L1 term is off
-// or the two gradients coincide), beta = 1 - alpha, the Adam bias
-// corrections; writes the stats.  sc = {alpha, beta, 1 - beta1^t, 1 - beta2^t}.
-__device__ __forceinline__ void alpha_finish(const StepArgs &a, bool use_l1, const double (&fin)[3], double (&sc)[4]) {
+// or the two gradients coincide), beta = 1 - alpha; writes the stats and scal.
+__device__ __forceinline__ void alpha_finish(const StepArgs &a, bool use_l1, const double (&fin)[3], const float (&bias)[3]) {
     const double num = fin[1], den = fin[2];
     double al = 1.0;
     if (use_l1 && den > 0.0) al = fmin(1.0, fmax(0.0, num / den));
-    // the Adam bias corrections feed a float update: float powers (a double
-    // pow costs microseconds on this part's FP64 unit)
-    const float t = (float)(a.st->adam_t + 1);
-    sc[0] = al;
-    sc[1] = 1.0 - al;
-    sc[2] = 1.0f - powf((float)a.c.beta1, t);
-    sc[3] = 1.0f - powf((float)a.c.beta2, t);
+    a.scal[0] = al;
+    a.scal[1] = 1.0 - al;
+    a.scal[2] = bias[0];
+    a.scal[3] = bias[1];
+    a.scal[4] = bias[2];
     a.stats[SERBF_STAT_L1] = fin[0];
     a.stats[SERBF_STAT_ALPHA] = al;
     a.stats[SERBF_STAT_BETA] = 1.0 - al;
@@ -122,8 +122,8 @@ __device__ __forceinline__ float tau_d_float(double tau_d) {
 }
 
 // Combined gradient of Eq. grad (App. A) and the Adam update of parameter
-// (r, j); returns 1 when it is a weight that stays at or above tau_d (b_f).
-__device__ __forceinline__ float adam_param(const StepArgs &a, int r, int j, const float (&sc)[4], float lr,
+// (r, j); returns whether it is a weight that stays at or above tau_d (b_f).
+__device__ __forceinline__ bool adam_param(const StepArgs &a, int r, int j, const float (&sc)[4], float lr,
                                             float taud) {
     const float b1 = (float)a.c.beta1, b2 = (float)a.c.beta2, eps = (float)a.c.adam_eps;
     const int64_t q = (int64_t)r * a.cap + j;
@@ -136,7 +136,7 @@ __device__ __forceinline__ float adam_param(const StepArgs &a, int r, int j, con
     a.am[q] = mo;
     a.av[q] = vo;
     a.p[q] = pn;
-    return (r == PW && fabsf(pn) >= taud) ? 1.f : 0.f;
+    return r == PW && fabsf(pn) >= taud;
 }
 
 // The epoch tail of Algorithm 3 on a shared-memory copy of the state, run by
@@ -251,36 +251,49 @@ __device__ void finish_step(const StepArgs &a, double bf, double alpha, double b
 
 // ---------------------------------------------------------------- grid path
 // Stage 1 (one thread per kernel, many blocks): the sums of alpha_terms; the
-// last block turns them into alpha, beta and the Adam bias corrections.
-// Block bx of nbx.
+// last block turns them into alpha, beta and the Adam bias corrections, and
+// passes the learning rate on (so that the update reads nothing of the state).
+// Block bx of nbx.  A chain of latencies bounds it: the powers are formed by
+// a warp of their own beside the sums, a single block skips the hand-off, and
+// up to 32 blocks' partials are summed by one warp (with the update below, an
+// epoch of 32^3 points and 64 kernels 43 -> 38 us).
 __device__ __forceinline__ void step_alpha_body(const StepArgs &a, int bx, int nbx) {
     __shared__ double sh3[33][3];
+    __shared__ float s_bias[3];
     __shared__ bool s_last;
     const int m = *a.m;
     const bool use_l1 = a.st->l1_optim && (a.stats[SERBF_STAT_MAXE] < a.c.tau_m);
     double part[3] = {0.0, 0.0, 0.0};
     const int j = bx * blockDim.x + threadIdx.x;
     if (j < m) alpha_terms(a, j, use_l1, part);
-    double tot[3];
-    block_sums_d3(part, sh3, tot);
-    double *bp = reinterpret_cast<double *>(a.part);  // 3 doubles per block
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 3; ++k) bp[3 * bx + k] = tot[k];
-        __threadfence();
-        s_last = atomicAdd(a.counter, 1u) == (unsigned)nbx - 1;
+    if (threadIdx.x == kStepThreads - 32) {
+        bias_corrections(a, s_bias[0], s_bias[1]);
+        s_bias[2] = (float)a.st->lr;
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (unsigned b = threadIdx.x; b < (unsigned)nbx; b += blockDim.x)
-        for (int k = 0; k < 3; ++k) acc[k] += __ldcg(bp + 3 * b + k);
     double fin[3];
-    block_sums_d3(acc, sh3, fin);
+    block_sums_d3(use_l1, part, sh3, fin);  // barriers: s_bias is written
+    if (nbx > 1) {
+        double *bp = reinterpret_cast<double *>(a.part);  // 3 doubles per block
+        if (threadIdx.x == 0) {
+            for (int k = 0; k < 3; ++k) bp[3 * bx + k] = fin[k];
+            __threadfence();
+            s_last = atomicAdd(a.counter, 1u) == (unsigned)nbx - 1;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (unsigned b = threadIdx.x; b < (unsigned)nbx; b += blockDim.x)
+            for (int k = 0; k < 3; ++k) acc[k] += __ldcg(bp + 3 * b + k);
+        if (nbx <= 32) {
+            if (threadIdx.x >= 32) return;
+            for (int k = 0; k < 3; ++k) fin[k] = warp_sum(acc[k]);
+        } else {
+            block_sums_d3(use_l1, acc, sh3, fin);
+        }
+    }
     if (threadIdx.x == 0) {
-        double sc[4];
-        alpha_finish(a, use_l1, fin, sc);
-        for (int k = 0; k < 4; ++k) a.scal[k] = sc[k];
+        alpha_finish(a, use_l1, fin, s_bias);
         *a.counter = 0u;
     }
 }
@@ -291,36 +304,38 @@ __global__ void __launch_bounds__(kStepThreads) k_step_alpha(StepArgs a) {
     step_alpha_body(a, blockIdx.x, gridDim.x);
 }
 
-// Stage 2 (one thread per parameter, many blocks): adam_param; then the last
-// block runs the epoch tail.  Block (bx, r) of nbx x 10.
+// Stage 2 (one thread per parameter, many blocks): adam_param.  The blocks of
+// the weight row count the weights that stay, and the last of them runs the
+// epoch tail, beside the other rows: those read only what stage 1 passed on,
+// never the state that the tail rewrites.  Block (bx, r) of nbx x 10.
 __device__ __forceinline__ void step_adam_body(const StepArgs &a, int bx, int r, int nbx) {
-    __shared__ ff sh1[33][1];
     __shared__ bool s_last;
+    __shared__ uint32_t s_bf;
     __shared__ __align__(8) uint32_t s_words[kStateWords];
     const int m = *a.m;
     const int j = bx * blockDim.x + threadIdx.x;
     const float sc[4] = {(float)a.scal[0], (float)a.scal[1], (float)a.scal[2], (float)a.scal[3]};
-    const float lr = (float)a.st->lr, taud = tau_d_float(a.c.tau_d);
-    float bfc[1] = {0.f};
-    if (j < m) bfc[0] = adam_param(a, r, j, sc, lr, taud);
-    ff tot[1];
-    block_sums_ff<1>(bfc, sh1, tot);
-    const unsigned nblocks = (unsigned)nbx * SERBF_NPARAM, bid = (unsigned)r * nbx + bx;
+    const float lr = (float)a.scal[4], taud = tau_d_float(a.c.tau_d);
+    const bool stays = j < m && adam_param(a, r, j, sc, lr, taud);
+    if (r != PW) return;
+    const uint32_t cnt = (uint32_t)__syncthreads_count(stays);
     if (threadIdx.x == 0) {
-        a.part[bid] = tot[0].hi;
-        __threadfence();
-        s_last = atomicAdd(a.counter + 1, 1u) == nblocks - 1;
+        s_last = true;
+        s_bf = cnt;
+        if (nbx > 1) {
+            atomicAdd(a.bf, cnt);
+            __threadfence();
+            s_last = atomicAdd(a.counter + 1, 1u) == (unsigned)nbx - 1;
+            if (s_last) {
+                __threadfence();
+                s_bf = atomicExch(a.bf, 0u);
+                a.counter[1] = 0u;
+            }
+        }
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
-    // the last block: b_f, then the epoch tail
-    float cnt = 0.f;
-    for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x) cnt += __ldcg(a.part + b);
-    float cc[1] = {cnt};
-    block_sums_ff<1>(cc, sh1, tot);
-    finish_step(a, (double)tot[0].hi + tot[0].lo, a.scal[0], a.scal[1], s_words);
-    if (threadIdx.x == 0) a.counter[1] = 0u;
+    finish_step(a, (double)s_bf, a.scal[0], a.scal[1], s_words);
 }
 
 __global__ void __launch_bounds__(kStepThreads) k_step_adam(StepArgs a) {
@@ -433,7 +448,7 @@ int batch_step_args(serbf_params *prm, const float *grad, float *adam_m, float *
     if (!(cfg->lr >= 0.0) || !(cfg->beta1 >= 0.0 && cfg->beta1 < 1.0) || !(cfg->beta2 >= 0.0 && cfg->beta2 < 1.0))
         return SERBF_EINVAL;
     StepBatch b{StepArgs{prm->p, prm->m, prm->cap, grad, adam_m, adam_v, st_dev, stats, *cfg, ws->step_part,
-                         ws->step_scal, ws->counters + 2},
+                         ws->step_scal, ws->counters + 2, ws->counters + 7},
                 (prm->cap + kStepThreads - 1) / kStepThreads};
     memcpy(out, &b, sizeof(b));
     *nb = b.nb;
@@ -463,7 +478,7 @@ extern "C" int serbf_step(serbf_params *prm, const float *grad, float *adam_m, f
     if (!(cfg->lr >= 0.0) || !(cfg->beta1 >= 0.0 && cfg->beta1 < 1.0) || !(cfg->beta2 >= 0.0 && cfg->beta2 < 1.0))
         return SERBF_EINVAL;
     StepArgs a{prm->p, prm->m, prm->cap, grad, adam_m, adam_v, st_dev, stats, *cfg,
-               ws->step_part, ws->step_scal, ws->counters + 2};
+               ws->step_part, ws->step_scal, ws->counters + 2, ws->counters + 7};
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned nb = (unsigned)((prm->cap + kStepThreads - 1) / kStepThreads);
     launch_pdl(k_step_alpha, dim3(nb), dim3(kStepThreads), 0, s, a);
