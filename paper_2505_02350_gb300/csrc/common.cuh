@@ -25,7 +25,7 @@ constexpr int kSortTile = 4096;                   // elements per radix-sort blo
 constexpr int kSmallSortTile = 1024;              // ... while these give at most kDirectBlocks blocks
 constexpr int kDirectBlocks = 32;
 constexpr int kQueue = 64;                        // per-warp ring of staged candidates
-constexpr int kFwdGroup = 64;                     // tiles per first-level forward reduction group
+constexpr int kFwdGroup = 128;                    // tiles per first-level forward reduction group
 constexpr double kFixUnit = 1.0 / 68719476736.0;  // 2^-36: fixed-point unit of the fused adjoint's moments
 constexpr int kCostClasses = 8;                   // cost classes of the forward's heavy-first schedule
 constexpr int kOrderChunk = 1024;                 // items per block of the class sort
