@@ -17,12 +17,11 @@ namespace serbf {
 size_t fwd_args_size();
 size_t finish_args_size();
 int batch_forward_args(const serbf_points *, const serbf_params *, const serbf_config *, float *, float *, uint8_t *,
-                       float *, double *, serbf_workspace *, void *, void *, int64_t *);
-int batch_pick_warps(int64_t nitems, int sm_count, int fixed);
+                       float *, double *, serbf_workspace *, int, void *, void *, int64_t *);
 int batch_forward_launch(const void *args, const void *fin, const uint32_t *item_off, int nfields, uint32_t *counters,
                          int64_t total_items, int64_t finish_blocks, int G, int kahan, int sm_count, cudaStream_t s);
 size_t rebuild_args_size();
-int batch_rebuild_args(const serbf_points *, const serbf_params *, const serbf_config *, serbf_workspace *, void *,
+int batch_rebuild_args(const serbf_points *, const serbf_params *, const serbf_config *, serbf_workspace *, int, void *,
                        int *, int64_t *, int *);
 int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, cudaStream_t s);
 size_t step_args_size();
@@ -102,16 +101,23 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     int lvl1 = 1, parents = 0, step_nb = 1, sm = 0;
     const int kahan = fields[0].cfg ? fields[0].cfg->kahan : 0;
     uint32_t *off = reinterpret_cast<uint32_t *>(host.data() + L.off);
+    int64_t items2 = 0;
     for (int f = 0; f < nfields; ++f) {
         const serbf_field &F = fields[f];
         if (!F.cfg || !F.ws || F.ws->magic != kMagic || !F.ws->binned || F.cfg->kahan != kahan) return SERBF_EINVAL;
+        items2 += F.ws->items[0].n;
+        sm = F.ws->sm_count;
+    }
+    const int G = forward_warps(items2, sm, fwd_warps);
+    for (int f = 0; f < nfields; ++f) {
+        const serbf_field &F = fields[f];
         serbf_params prm = F.prm;
         int64_t fb = 1, ch = 0;
         int l1 = 0, pa = 0, nb = 0;
-        int rc = batch_forward_args(&F.pts, &F.prm, F.cfg, F.psi, F.err, F.mask, F.grad, F.stats, F.ws,
+        int rc = batch_forward_args(&F.pts, &F.prm, F.cfg, F.psi, F.err, F.mask, F.grad, F.stats, F.ws, G,
                                     host.data() + L.fwd + (size_t)f * fwd_args_size(),
                                     host.data() + L.fin + (size_t)f * finish_args_size(), &fb);
-        if (!rc) rc = batch_rebuild_args(&F.pts, &F.prm, F.cfg, F.ws, host.data() + L.reb + (size_t)f * rebuild_args_size(),
+        if (!rc) rc = batch_rebuild_args(&F.pts, &F.prm, F.cfg, F.ws, G, host.data() + L.reb + (size_t)f * rebuild_args_size(),
                                          &l1, &ch, &pa);
         if (!rc) rc = batch_step_args(&prm, F.grad, F.adam_m, F.adam_v, F.st, F.stats, F.cfg, F.ws,
                                       host.data() + L.step + (size_t)f * step_args_size(), &nb);
@@ -120,14 +126,13 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
         if (rc) return rc;
         if (!F.grad) return SERBF_EINVAL;
         off[f] = (uint32_t)total;
-        total += F.ws->nitems;
+        total += items_of(F.ws, G).n;
         if (total >= (int64_t)1 << 32) return SERBF_ECAPACITY;
         fin_blocks = fb > fin_blocks ? fb : fin_blocks;
         chunks = ch > chunks ? ch : chunks;
         lvl1 = l1 > lvl1 ? l1 : lvl1;
         parents = pa > parents ? pa : parents;
         step_nb = nb > step_nb ? nb : step_nb;
-        sm = F.ws->sm_count;
     }
     off[nfields] = (uint32_t)total;
     cudaStream_t s = (cudaStream_t)stream;
@@ -136,7 +141,7 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     memset(b, 0, sizeof(*b));
     b->magic = kBatchMagic;
     b->nfields = nfields;
-    b->G = batch_pick_warps(total, sm, fwd_warps);
+    b->G = G;
     b->kahan = kahan;
     b->sm_count = sm;
     b->base = static_cast<char *>(dev);

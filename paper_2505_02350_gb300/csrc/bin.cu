@@ -213,22 +213,21 @@ __global__ void __launch_bounds__(256) k_cells(const uint32_t *keys, int64_t n, 
     if ((threadIdx.x & 31) == 0 && cnt) atomicMax(cell_max, cnt);
 }
 
-// One block: tiles and forward work items of every super cell, numbered in
-// super-cell order; out = {tiles, items, most tiles in one super cell}.  Also
-// clears the forward's scheduling state (no mean cost yet: the first forward
-// files every item in the same class).
+// One block: tiles and forward work items (both sets) of every super cell,
+// numbered in super-cell order; out = {tiles, items of set 0, of set 1, most
+// tiles in one super cell}.  Also clears the forward's scheduling state (no
+// mean cost yet: the first forward files every item in the same class).
 __global__ void __launch_bounds__(1024) k_supers(const uint32_t *cell_start, int nsuper, int cps, uint32_t *stile,
-                                                 uint32_t *sitem, uint32_t *sched, unsigned long long *sched_total,
-                                                 uint32_t *out) {
+                                                 ItemSet two, ItemSet four, uint32_t *out, uint32_t *arrived) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t tmp[33];
     __shared__ uint32_t s_max;
     if (threadIdx.x == 0) s_max = 0u;
-    if (threadIdx.x < 4) sched[threadIdx.x] = 0u;
-    if (threadIdx.x < 2) sched_total[threadIdx.x] = 0ull;
+    if (threadIdx.x < 4) two.sched[threadIdx.x] = four.sched[threadIdx.x] = 0u;
+    if (threadIdx.x < 2) two.total[threadIdx.x] = four.total[threadIdx.x] = 0ull;
     __syncthreads();
-    uint32_t t0 = 0, i0 = 0, mx = 0;
+    uint32_t t0 = 0, i0 = 0, q0 = 0, mx = 0;
     for (int s0 = 0; s0 < nsuper; s0 += blockDim.x) {
         const int s = s0 + threadIdx.x;
         uint32_t nt = 0;
@@ -237,25 +236,30 @@ __global__ void __launch_bounds__(1024) k_supers(const uint32_t *cell_start, int
             nt = (e - b + kTile - 1) / kTile;
         }
         mx = max(mx, nt);
-        uint32_t ts, is;
+        uint32_t ts, is, qs;
         const uint32_t to = block_exscan(nt, tmp, &ts), io = block_exscan((nt + 1) / 2, tmp, &is);
+        const uint32_t qo = block_exscan((nt + kMostTiles - 1) / kMostTiles, tmp, &qs);
         if (s < nsuper) {
             stile[s] = t0 + to;
-            sitem[s] = i0 + io;
+            two.super0[s] = i0 + io;
+            four.super0[s] = q0 + qo;
         }
         t0 += ts;
         i0 += is;
+        q0 += qs;
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_max, mx);
     __syncthreads();
     if (threadIdx.x == 0) {
         stile[nsuper] = t0;
-        sitem[nsuper] = i0;
+        two.super0[nsuper] = i0;
+        four.super0[nsuper] = q0;
         out[0] = t0;
         out[1] = i0;
-        out[2] = s_max;
-        out[3] = 0u;  // arrival counter of k_tiles
+        out[2] = q0;
+        out[3] = s_max;
+        *arrived = 0u;
     }
 }
 
@@ -276,11 +280,10 @@ __device__ __forceinline__ void warp_box(float x, float y, float z, bool v, floa
 }
 
 struct TilesArgs {
-    const uint32_t *cell_start, *stile0, *sitem0;
+    const uint32_t *cell_start, *stile0;
     int nsuper, cps;
     uint32_t *tile_super, *tile_start;
-    uint4 *item_rec, *order_rec;
-    uint8_t *item_class;
+    ItemSet two, four;
     const float *xb, *yb, *zb;
     float4 *tlo, *thi, *slo, *shi, *box;
     uint32_t *arrived;
@@ -294,10 +297,19 @@ __device__ __forceinline__ void grow(float4 &lo, float4 &hi, float4 a, float4 b)
 constexpr int kTilesThreads = 512;
 
 // One block per super cell, a warp per tile: the tile's start and bounding
-// box, the work items (the tiles at even offsets, with the following tile, if
-// any, as the item's second; the first forward takes them in this order), the
+// box, the work items (the first forward takes them in this order), the
 // super cell's box (empty: +inf / -inf).  The last block unites the super
 // cells' boxes (the box of every binned point).
+__device__ __forceinline__ void put_item(const ItemSet &set, int s, uint32_t t, uint32_t k, uint32_t ps, uint32_t left,
+                                         uint32_t tiles) {
+    if (k % tiles) return;
+    const uint32_t it = set.super0[s] + k / tiles;
+    const uint4 r = make_uint4(t, (uint32_t)s, ps, (min(left, tiles * kTile) - 1u) | (it << 7));
+    set.rec[it] = r;
+    set.order[it] = r;
+    set.cls[it] = 3;  // one class for all until a forward has measured them
+}
+
 __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
     pdl_wait();
     pdl_trigger();
@@ -305,7 +317,7 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
     __shared__ float4 wlo[NW], whi[NW];
     __shared__ bool s_last;
     const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t t0 = a.stile0[s], t1 = a.stile0[s + 1], i0 = a.sitem0[s];
+    const uint32_t t0 = a.stile0[s], t1 = a.stile0[s + 1];
     const uint32_t p0 = a.cell_start[(int64_t)s * a.cps], pe = a.cell_start[(int64_t)(s + 1) * a.cps];
     const float4 none_lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
     const float4 none_hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
@@ -321,14 +333,8 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
             a.thi[t] = th;
             a.tile_super[t] = (uint32_t)s;
             a.tile_start[t] = ps;
-            if (((t - t0) & 1u) == 0) {
-                const uint32_t it = i0 + (t - t0) / 2;
-                const uint32_t np = min(pe - ps, 2u * kTile);
-                const uint4 r = make_uint4(t, (uint32_t)s, ps, np | (it << 7));
-                a.item_rec[it] = r;
-                a.order_rec[it] = r;
-                a.item_class[it] = 3;  // one class for all until a forward has measured them
-            }
+            put_item(a.two, s, t, t - t0, ps, pe - ps, 2u);
+            put_item(a.four, s, t, t - t0, ps, pe - ps, (uint32_t)kMostTiles);
         }
     }
     if (lane == 0) {
@@ -475,20 +481,21 @@ extern "C" int serbf_bin_points(const float *x, const float *y, const float *z, 
     }
     launch_pdl(k_cells, dim3((unsigned)((ncp + 256) / 256)), dim3(256), 0, s, kin, n, ncp, ws->cell_start, ws->cell_max);
     uint32_t *out = ws->counters + 12;
-    launch_pdl(k_supers, dim3(1), dim3(1024), 0, s, ws->cell_start, (int)nsuper, cps, ws->super_tile0, ws->super_item0,
-               ws->sched, ws->sched_total, out);
+    launch_pdl(k_supers, dim3(1), dim3(1024), 0, s, ws->cell_start, (int)nsuper, cps, ws->super_tile0, ws->items[0],
+               ws->items[1], out, ws->counters);
     launch_pdl(k_tiles, dim3((unsigned)nsuper), dim3(kTilesThreads), 0, s,
-               TilesArgs{ws->cell_start, ws->super_tile0, ws->super_item0, (int)nsuper, cps, ws->tile_super,
-                         ws->tile_start, ws->item_rec, ws->order_rec, ws->item_class, xb, yb, zb, ws->tile_lo,
-                         ws->tile_hi, ws->sup_lo, ws->sup_hi, ws->field_box, out + 3});
+               TilesArgs{ws->cell_start, ws->super_tile0, (int)nsuper, cps, ws->tile_super, ws->tile_start, ws->items[0],
+                         ws->items[1], xb, yb, zb, ws->tile_lo, ws->tile_hi, ws->sup_lo, ws->sup_hi, ws->field_box,
+                         ws->counters});
     SERBF_CHECK_LAUNCH();
-    uint32_t got[3];  // tiles, items, most tiles in a super cell
+    uint32_t got[4];  // tiles, items of either set, most tiles in a super cell
     if (cudaMemcpyAsync(got, out, sizeof(got), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
     if ((int64_t)got[0] > ws->max_tiles || got[1] >= (1u << 25)) return SERBF_ECAPACITY;  // item ids have 25 bits
     ws->ntiles = got[0];
-    ws->nitems = got[1];
-    ws->max_chunks = (int32_t)((got[2] + kTile - 1) / kTile);
+    ws->items[0].n = got[1];
+    ws->items[1].n = got[2];
+    ws->max_chunks = (int32_t)((got[3] + kTile - 1) / kTile);
     ws->binned = 1;
     return SERBF_OK;
 }

@@ -24,6 +24,7 @@ constexpr int kTile = 32;                         // points per forward/backward
 constexpr int kSortTile = 4096;                   // elements per radix-sort block
 constexpr int kSmallSortTile = 1024;              // ... while these give at most kDirectBlocks blocks
 constexpr int kDirectBlocks = 32;
+constexpr int kMostTiles = 4;                      // most tiles of a forward work item
 constexpr int kQueue = 64;                        // per-warp ring of staged candidates
 constexpr int kFwdGroup = 128;                    // tiles per first-level forward reduction group
 constexpr double kFixUnit = 1.0 / 68719476736.0;  // 2^-36: fixed-point unit of the fused adjoint's moments
@@ -56,6 +57,22 @@ int radix_sort_pairs(uint32_t **k, uint32_t **v, uint32_t **ktmp, uint32_t **vtm
 
 }  // namespace serbf
 
+// Forward work items: runs of up to two tiles of one super cell (set 0) or of
+// up to four (set 1), from the super cell's first tile on.  A launch takes one
+// set: one warp per item takes set 1, several share an item of set 0.  Item
+// record: (first tile, super cell, first point, points - 1 | item << 7).
+// Heavy-first order: each launch files every item of its set into a cost class
+// (cls); a stable sort by class, descending, gives the set's next order.
+struct ItemSet {
+    int64_t n;
+    uint32_t *super0;          // nsuper + 1: first item of each super cell
+    uint4 *rec;                // in item order
+    uint4 *order;              // heaviest class first
+    uint8_t *cls;
+    uint32_t *sched;           // [0] mean cost of the last launch
+    unsigned long long *total; // cost sum of the running launch
+};
+
 // Host-side description of the caller's scratch buffer.
 struct serbf_workspace {
     uint64_t magic;
@@ -64,7 +81,6 @@ struct serbf_workspace {
     serbf_ws_sizes sz;
     int64_t max_tiles;
     int64_t max_supers;
-    int64_t max_items;
     int64_t sort_blocks;
     // grid recorded by serbf_bin_points
     serbf_grid grid;
@@ -74,7 +90,6 @@ struct serbf_workspace {
     int32_t binned;
     int64_t npoints;
     int64_t ntiles;
-    int64_t nitems;      // forward work items (one or two tiles of one super cell)
     int32_t sm_count;
     int32_t max_chunks;  // most 32-tile chunks in one super cell
     // side stream for work that overlaps the main stream inside one call
@@ -87,20 +102,8 @@ struct serbf_workspace {
     uint32_t *super_tile0;  // nsuper + 1: first tile of each super cell
     uint32_t *tile_super, *tile_start;
     float4 *tile_lo, *tile_hi;
-    // forward work items: tiles at even offsets within their super cell,
-    // taken together with the next tile of the same super cell if any.
-    // Item record: (first tile, super cell, first point, points | item << 7).
-    uint32_t *super_item0;  // nsuper + 1: first item of each super cell
-    uint4 *item_rec;        // record of each item, in item order
-    // heavy-first order of the forward: each launch files every item into a
-    // cost class (item_class); a stable sort by class, descending (class
-    // counts per chunk of kOrderChunk items in class_hist), gives the next
-    // launch's order (order_rec).
-    uint8_t *item_class;    // max_items
-    uint32_t *class_hist;   // chunks x kCostClasses
-    uint4 *order_rec;       // max_items
-    uint32_t *sched;        // [0] mean cost of the last launch
-    unsigned long long *sched_total;  // cost sum of the running launch
+    ItemSet items[2];
+    uint32_t *class_hist;   // order chunks x kCostClasses
     float4 *sup_lo, *sup_hi;
     // per-kernel records
     float4 *kfwd;  // 3 per kernel
@@ -526,6 +529,10 @@ __device__ __forceinline__ KBox kernel_box(float cx, float cy, float cz, float r
 
 // ---------------------------------------------------------------- cross-unit launchers
 namespace serbf {
+// Warps per forward work item for a field (or batch) of items2 items of two
+// tiles, unless fixed (1, 2, 4 or 8) says so; and the item set they take.
+int forward_warps(int64_t items2, int sm_count, int fixed);
+inline const ItemSet &items_of(const serbf_workspace *ws, int warps) { return ws->items[warps == 1 ? 1 : 0]; }
 constexpr int kScanTile = 4096;  // elements of a tile of launch_exscan_i64
 // Exclusive scan in place, a[n] = total; tiles: n / kScanTile + 1 words of scratch.
 int launch_exscan_i64(int64_t *a, int64_t n, int64_t *tiles, cudaStream_t s);

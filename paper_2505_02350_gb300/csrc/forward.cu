@@ -1,17 +1,26 @@
 // Point-major forward (Eq. 3-26) over the support pairs of Eq. 3-15-1, the
 // point filter of Eq. 3-18 and the loss terms of Eq. 3-19.
 //
-// Work item = up to two consecutive 32-point tiles of one super cell; each
-// lane holds one point of each tile.  The warp streams
+// Work item = up to two (several warps per item) or four (one warp per item)
+// consecutive 32-point tiles of one super cell; each lane holds one point of
+// each tile.  The warp streams
 // its super cell's candidate list (ascending kernel index), keeps the kernels
 // whose support reaches the item's bounding box (one candidate per lane,
 // ballot), and stages their records in a per-warp shared-memory ring, in
 // pairs.  Each batch of 32 staged kernels is then evaluated with broadcast
 // 16-byte loads and packed f32x2 arithmetic (two kernels per instruction,
-// two points per lane), so every shared-memory load serves four pairs.  A
-// kernel whose support covers the whole box skips the predicate; otherwise
-// every lane applies the exact support predicate to its own points, so the
-// pairs summed are exactly the point-major neighbour rows.
+// two or four points per lane), so every shared-memory load serves four or
+// eight pairs.  A kernel whose support covers the whole box skips the
+// predicate; otherwise every lane applies the exact support predicate to its
+// own points, so the pairs summed are exactly the point-major neighbour rows.
+//
+// What bounds it is the instructions issued: pair arithmetic is 40 % of them,
+// the rest scans, stages, filters and flushes per item.  Four tiles per item
+// halve that rest per point and widen the item box (a few more pairs outside
+// the support); with one warp per item that gains (9.4 M points 2118 -> 2070 us,
+// 16 fields 844 -> 704 us for the fused call), with several it does not (64^3 +
+// 32^3 points 59 -> 72 us with four), so they keep two.  The tiles follow from
+// the warps alone, so a field in a batch gets the bits it gets by itself.
 //
 // Persistent blocks take items heaviest first (order from the costs measured
 // by the previous launch) to keep the tail short; the warps of a block split
@@ -32,12 +41,10 @@ struct FwdArgs {
     const uint32_t *slist, *scnt;
     const float4 *kfwd;
     const float4 *kbwd;      // adjoint records (c, r2), rows of R with log2(e) d_k^2
-    const uint4 *item_rec;   // item records
     const uint4 *order_rec;  // item records, heaviest class first (stable)
     uint8_t *item_class;     // cost class of each item, for the next order
     uint32_t *sched;         // mean cost of the last launch
     unsigned long long *sched_total;
-    int64_t max_items;
     unsigned long long *adj_fix;    // fixed-point moments (fused adjoint)
     unsigned long long *adj_pairs;  // adjoint pair count (fused adjoint)
     int64_t ntiles, nitems;
@@ -52,7 +59,7 @@ struct FwdArgs {
 };
 
 constexpr int kTouch = 256;  // kernels an item's warps remember for its adjoint (more: re-scan the list)
-constexpr int kNz = 2 * kTile;
+constexpr int kNz = kMostTiles * kTile;
 
 // Two float32 lanes in one 64-bit register: the packed f32x2 arithmetic of
 // sm_100+ does two IEEE round-to-nearest operations per instruction, each
@@ -141,18 +148,19 @@ __device__ __forceinline__ void box_near_far_d2(float cx, float cy, float cz, fl
 }
 
 // npairs staged kernel pairs from pair index pb against the lane's two
-// points.  PARTIAL: the support only partly covers the item box, so each
+// points.  NP: the lane's points that take part, of NT (an item of a sparse
+// super cell may have fewer tiles).  PARTIAL: the support only partly covers the item box, so each
 // pair takes the exact Eq. 3-15-1 predicate (the operations of support_d2,
 // packed: fma(dz, dz, fma(dy, dy, fl(dx dx))) < r2).
-template <bool PARTIAL, int UNROLL>
-__device__ __forceinline__ void eval_pairs(const float *ring, int pb, int npairs, const f2 (&P)[2][3], f2 (&acc)[2],
-                                           uint32_t (&n)[2]) {
+template <bool PARTIAL, int UNROLL, int NP, int NT>
+__device__ __forceinline__ void eval_pairs(const float *ring, int pb, int npairs, const f2 (&P)[NT][3], f2 (&acc)[NT],
+                                           uint32_t (&n)[NT]) {
 #pragma unroll UNROLL
     for (int q = 0; q < npairs; ++q) {
         const ulonglong2 *r = reinterpret_cast<const ulonglong2 *>(ring + kPairFloats * (pb + q));
         const ulonglong2 F0 = r[0], F1 = r[1], F2 = r[2], F3 = r[3], F4 = r[4], F5 = r[5];
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
+        for (int p = 0; p < NP; ++p) {
             const f2 dx = f2_sub(P[p][0], F0.x), dy = f2_sub(P[p][1], F0.y), dz = f2_sub(P[p][2], F1.x);
             const f2 zz = f2_mul(dz, dz);
             // q = dv^T Q dv (log2 units): dx (Q11 dx + 2Q12 dy + 2Q13 dz) + dy (Q22 dy + 2Q23 dz) + Q33 dz^2
@@ -174,6 +182,19 @@ __device__ __forceinline__ void eval_pairs(const float *ring, int pb, int npairs
             }
             acc[p] = f2_fma(F3.y, f2_pack(e0, e1), acc[p]);
         }
+    }
+}
+
+template <bool PARTIAL, int UNROLL, int NT>
+__device__ __forceinline__ void eval_staged(int ntl, const float *ring, int pb, int npairs, const f2 (&P)[NT][3],
+                                            f2 (&acc)[NT], uint32_t (&n)[NT]) {
+    if constexpr (NT > 2) {
+        if (ntl > 2)
+            eval_pairs<PARTIAL, 1, NT>(ring, pb, npairs, P, acc, n);  // four points are enough independent chains
+        else
+            eval_pairs<PARTIAL, 1, 2>(ring, pb, npairs, P, acc, n);
+    } else {
+        eval_pairs<PARTIAL, UNROLL, 2>(ring, pb, npairs, P, acc, n);
     }
 }
 
@@ -247,16 +268,16 @@ __device__ __forceinline__ void finish_tile(const FwdArgs &a, uint32_t t, float 
     if (lane == 0) a.part[t] = FwdPart{l2s.hi, l2s.lo, mx, cnt, (unsigned long long)pr};
 }
 
-// Loss terms of both tiles of an item in one reduction (a lane's two squares
-// are added exactly first), stored as the first tile's partial; the second
-// tile's is zero.
-__device__ __forceinline__ void finish_item(const FwdArgs &a, uint32_t t, bool two, ff l2, float mx_l, uint32_t cnt_l,
+// Loss terms of an item's ntl tiles in one reduction (a lane's squares are
+// summed in float-float first), stored as the first tile's partial; the other
+// tiles' are zero.
+__device__ __forceinline__ void finish_item(const FwdArgs &a, uint32_t t, int ntl, ff l2, float mx_l, uint32_t cnt_l,
                                             uint32_t pairs_l, int lane) {
     const ff l2s = warp_sum_ff(l2);
     const float mx = redux_max(mx_l);
     const uint32_t cnt = redux_add(cnt_l), pr = redux_add(pairs_l);
     if (lane == 0) a.part[t] = FwdPart{l2s.hi, l2s.lo, mx, cnt, (unsigned long long)pr};
-    if (lane == 1 && two) a.part[t + 1] = FwdPart{0.f, 0.f, 0.f, 0u, 0ull};
+    if (lane > 0 && lane < ntl) a.part[t + lane] = FwdPart{0.f, 0.f, 0.f, 0u, 0ull};
 }
 
 // Eq. 3-18 filter and residual of one point; returns its loss contributions.
@@ -284,27 +305,30 @@ __device__ __forceinline__ float point_out(const FwdArgs &a, int64_t i, bool val
     return e;
 }
 
-// Item geometry shared by the warps of a block.
+// Item geometry shared by the warps of a block: tiles t0 .. t0 + ntl - 1 of
+// super cell sup, np points from i0 (a lane's points: i0 + lane + 32 k).
 struct ItemInfo {
-    uint32_t t0, sup, item;
-    int two;
-    int64_t i0, i1;
-    int v0, v1;
+    uint32_t t0, sup;
+    int ntl, np;
+    int64_t i0;
 };
 
-// Decode an item record (first tile, super cell, first point, points | item << 7).
-__device__ __forceinline__ ItemInfo item_info(uint4 r, int lane) {
+// Decode an item record (first tile, super cell, first point, points - 1 | item << 7).
+__device__ __forceinline__ ItemInfo item_info(uint4 r) {
     ItemInfo it;
-    const uint32_t np = r.w & 127u;
+    it.np = (int)(r.w & 127u) + 1;
     it.t0 = r.x;
     it.sup = r.y;
-    it.two = np > (uint32_t)kTile;
-    it.i0 = (int64_t)r.z + lane;
-    it.i1 = it.i0 + kTile;  // the second tile starts kTile points later
-    it.v0 = (uint32_t)lane < np;
-    it.v1 = (uint32_t)(lane + kTile) < np;
-    it.item = r.w >> 7;
+    it.ntl = (it.np + kTile - 1) / kTile;
+    it.i0 = (int64_t)r.z;
     return it;
+}
+
+__device__ __forceinline__ float4 box_min(float4 a, float4 b) {
+    return make_float4(fminf(a.x, b.x), fminf(a.y, b.y), fminf(a.z, b.z), 0.f);
+}
+__device__ __forceinline__ float4 box_max(float4 a, float4 b) {
+    return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), 0.f);
 }
 
 // One warp's share of a work item: candidate chunks w, w + W, w + 2W, ... of
@@ -312,42 +336,37 @@ __device__ __forceinline__ ItemInfo item_info(uint4 r, int lane) {
 // box, staged in pairs and evaluated against the lane's two points.
 // Returns the lane's partial sums and pair counts; *cost gets the warp's
 // measured work.
-template <int G, int ADJ>
+template <int G, int ADJ, int NT>
 __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &it, int w, float *ringP, float *ringF,
-                                              int lane, f2 (&acc)[2], uint32_t (&n)[2], uint32_t &cost,
-                                              uint32_t *touch, int tcap, int &ntouch, float (&tv)[2]) {
+                                              int lane, f2 (&acc)[NT], uint32_t (&n)[NT], uint32_t &cost,
+                                              uint32_t *touch, int tcap, int &ntouch) {
     const unsigned lt = (1u << lane) - 1u;
     // invalid lanes carry NaN so the support test fails for them
     const float qnan = __int_as_float(0x7fc00000);
-    f2 P[2][3];
-    {
-        const float x0 = it.v0 ? a.x[it.i0] : qnan, y0 = it.v0 ? a.y[it.i0] : 0.f, z0 = it.v0 ? a.z[it.i0] : 0.f;
-        const float x1 = it.v1 ? a.x[it.i1] : qnan, y1 = it.v1 ? a.y[it.i1] : 0.f, z1 = it.v1 ? a.z[it.i1] : 0.f;
-        P[0][0] = f2_pack(x0, x0);
-        P[0][1] = f2_pack(y0, y0);
-        P[0][2] = f2_pack(z0, z0);
-        P[1][0] = f2_pack(x1, x1);
-        P[1][1] = f2_pack(y1, y1);
-        P[1][2] = f2_pack(z1, z1);
-        // the targets, for the residuals after the sums (loaded early)
-        tv[0] = it.v0 ? a.t[it.i0] : 0.f;
-        tv[1] = it.v1 ? a.t[it.i1] : 0.f;
+    f2 P[NT][3];
+#pragma unroll
+    for (int p = 0; p < NT; ++p) {
+        const bool v = lane + p * kTile < it.np;
+        const int64_t i = it.i0 + lane + p * kTile;
+        const float x = v ? a.x[i] : qnan, y = v ? a.y[i] : 0.f, z = v ? a.z[i] : 0.f;
+        P[p][0] = f2_pack(x, x);
+        P[p][1] = f2_pack(y, y);
+        P[p][2] = f2_pack(z, z);
+        acc[p] = 0ull;
+        n[p] = 0u;
     }
     float4 lo = a.tile_lo[it.t0], hi = a.tile_hi[it.t0];
-    if (it.two) {
-        const float4 l1 = a.tile_lo[it.t0 + 1], h1 = a.tile_hi[it.t0 + 1];
-        lo = make_float4(fminf(lo.x, l1.x), fminf(lo.y, l1.y), fminf(lo.z, l1.z), 0.f);
-        hi = make_float4(fmaxf(hi.x, h1.x), fmaxf(hi.y, h1.y), fmaxf(hi.z, h1.z), 0.f);
-    }
+#pragma unroll
+    for (int p = 1; p < NT; ++p)
+        if (p < it.ntl) {
+            lo = box_min(lo, a.tile_lo[it.t0 + p]);
+            hi = box_max(hi, a.tile_hi[it.t0 + p]);
+        }
     const uint32_t *lst = a.slist + (size_t)it.sup * a.scap;
     const int L = min((int)a.scnt[it.sup], a.scap);
     constexpr int kStride = 32 * G;
     int hp = 0, qp = 0, hf = 0, qf = 0;
     uint32_t nfull = 0, npart = 0;
-    acc[0] = 0ull;
-    acc[1] = 0ull;
-    n[0] = 0u;
-    n[1] = 0u;
     // software pipeline: records of the next chunk and indices of the one
     // after it are in flight while a chunk is filtered
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -400,12 +419,12 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
         nfull += nf;
         __syncwarp();
         if (qp >= 32) {
-            eval_pairs<true, 2>(ringP, hp >> 1, 16, P, acc, n);
+            eval_staged<true, 2>(it.ntl, ringP, hp >> 1, 16, P, acc, n);
             hp ^= 32;
             qp -= 32;
         }
         if (qf >= 32) {
-            eval_pairs<false, 2>(ringF, hf >> 1, 16, P, acc, n);
+            eval_staged<false, 2>(it.ntl, ringF, hf >> 1, 16, P, acc, n);
             hf ^= 32;
             qf -= 32;
         }
@@ -421,11 +440,11 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
         if (lane == 0) stage_empty(ringF, hf + qf);
         __syncwarp();
     }
-    if (qp > 0) eval_pairs<true, 1>(ringP, hp >> 1, (qp + 1) >> 1, P, acc, n);
-    if (qf > 0) eval_pairs<false, 1>(ringF, hf >> 1, (qf + 1) >> 1, P, acc, n);
+    if (qp > 0) eval_staged<true, 1>(it.ntl, ringP, hp >> 1, (qp + 1) >> 1, P, acc, n);
+    if (qf > 0) eval_staged<false, 1>(it.ntl, ringF, hf >> 1, (qf + 1) >> 1, P, acc, n);
     __syncwarp();
-    n[0] += nfull;
-    n[1] += nfull;
+#pragma unroll
+    for (int p = 0; p < NT; ++p) n[p] += nfull;
     // about one unit per filtered candidate, ~6 per fully and ~9 per partly
     // covering kernel
     cost = 32u * (uint32_t)nchunks + 6u * nfull + 9u * npart;
@@ -490,14 +509,15 @@ __device__ __forceinline__ void f2_kadd(f2 &s, f2 &c, f2 v) {
 }
 
 // A batch of cnt <= 32 kernels from queue slot head: all nz points of the
-// item against each kernel.  A short batch spreads each kernel over
+// item against each kernel (segs: 8 bits for each run of points, runs from
+// slots 0, 32, ...).  A short batch spreads each kernel over
 // L = 2, 4 or 8 neighbouring lanes (cnt <= 16, 8, 4) that take every L-th
 // point pair; their moments are combined with xor shuffles within the group
 // (a fixed order for a given cnt) before the atomics, so short batches do
 // not leave most lanes idle.  KAHAN: compensated per-lane sums.
 template <bool KAHAN>
 __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *q, int head, int cnt,
-                                              const NzPoints &nz, int nc0, int nc1, int lane) {
+                                              const NzPoints &nz, uint32_t segs, int lane) {
     const int sh = cnt > 16 ? 0 : (cnt > 8 ? 1 : (cnt > 4 ? 2 : 3));
     const int L = 1 << sh, kl = lane >> sh, sub = lane & (L - 1);
     const bool act = kl < cnt;  // whole groups of L lanes are inactive together
@@ -512,8 +532,8 @@ __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *
 #pragma unroll
     for (int r = 0; r < (KAHAN ? 10 : 1); ++r) cmp[r] = 0ull;
 #pragma unroll 1
-    for (int seg = 0; seg < 2; ++seg) {
-        const int base = seg ? kTile : 0, cntp = act ? ((seg ? nc1 : nc0) + 1) >> 1 : 0;
+    for (int base = 0; segs != 0u; base += kTile, segs >>= 8) {
+        const int cntp = act ? (int)((segs & 255u) + 1u) >> 1 : 0;
 #pragma unroll 4
         for (int pp = sub; pp < cntp; pp += L) {
             const int i = base + 2 * pp;
@@ -636,7 +656,7 @@ __device__ __forceinline__ float form_limit(float emax, int cnt) {
 // it, 2462 us with it here, 2533 us with it there.
 template <int G, bool KAHAN>
 __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &it, int w, const NzPoints &nz,
-                                              int nc0, int nc1, float4 lo, float4 hi, const uint32_t *touch,
+                                              uint32_t segs, int nc, float4 lo, float4 hi, const uint32_t *touch,
                                               int ntouch, int tcap, float emax, uint32_t *q, int lane,
                                               uint32_t &cost) {
     const unsigned lt = (1u << lane) - 1u;
@@ -647,7 +667,7 @@ __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &
     const float4 mid = make_float4(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z), 0.f);
     const float ex = hi.x - lo.x, ey = hi.y - lo.y, ez = hi.z - lo.z;
     const float hd = 0.5001f * sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
-    const float qlim = form_limit(emax, nc0 + nc1);
+    const float qlim = form_limit(emax, nc);
     int head = 0, qn = 0, nk = 0;
     for (int b = b0; b < L; b += stride) {
         const bool live = b + lane < L;
@@ -663,25 +683,21 @@ __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &
         nk += __popc(bal);
         __syncwarp();
         if (qn >= 32) {
-            adjoint_batch<KAHAN>(a, q, head, 32, nz, nc0, nc1, lane);
+            adjoint_batch<KAHAN>(a, q, head, 32, nz, segs, lane);
             head = (head + 32) & (kQueue - 1);
             qn -= 32;
             __syncwarp();
         }
     }
-    if (qn > 0) adjoint_batch<KAHAN>(a, q, head, qn, nz, nc0, nc1, lane);
+    if (qn > 0) adjoint_batch<KAHAN>(a, q, head, qn, nz, segs, lane);
     __syncwarp();
-    cost += (uint32_t)(nk * (nc0 + nc1)) / 4u + 32u;
+    cost += (uint32_t)(nk * nc) / 4u + 32u;
 }
 
-// The nz points of one 32-point tile (lanes = points): compacted in lane
-// order from `base`, padded to an even count with a copy of the last point
-// with E = 0 (it adds zero and is not counted); returns their count and box
-// (empty: +inf / -inf).
-__device__ __forceinline__ int nz_tile(NzPoints &nzp, int base, bool nz, float x, float y, float z, float e, int lane,
-                                       float4 &lo, float4 &hi) {
+// The nz points of one 32-point tile (lanes = points), compacted in lane
+// order from slot `base`; returns their count.
+__device__ __forceinline__ int nz_tile(NzPoints &nzp, int base, bool nz, float x, float y, float z, float e, int lane) {
     const unsigned bal = __ballot_sync(0xffffffffu, nz);
-    const int cnt = __popc(bal);
     if (nz) {
         const int i = base + __popc(bal & ((1u << lane) - 1u));
         nzp.at(0, i) = x;
@@ -689,34 +705,30 @@ __device__ __forceinline__ int nz_tile(NzPoints &nzp, int base, bool nz, float x
         nzp.at(2, i) = z;
         nzp.at(3, i) = e;
     }
-    __syncwarp();
-    if ((cnt & 1) && lane == 0) {
-        // pad: a copy of the last point with E = 0 (finite, adds nothing)
-        nzp.at(0, base + cnt) = nzp.at(0, base + cnt - 1);
-        nzp.at(1, base + cnt) = nzp.at(1, base + cnt - 1);
-        nzp.at(2, base + cnt) = nzp.at(2, base + cnt - 1);
-        nzp.at(3, base + cnt) = 0.f;
-    }
-    float mnx = nz ? x : INFINITY, mny = nz ? y : INFINITY, mnz = nz ? z : INFINITY;
-    float mxx = nz ? x : -INFINITY, mxy = nz ? y : -INFINITY, mxz = nz ? z : -INFINITY;
-    if (bal) {
-        mnx = redux_min(mnx);
-        mny = redux_min(mny);
-        mnz = redux_min(mnz);
-        mxx = redux_max(mxx);
-        mxy = redux_max(mxy);
-        mxz = redux_max(mxz);
-    }
-    lo = make_float4(mnx, mny, mnz, 0.f);
-    hi = make_float4(mxx, mxy, mxz, 0.f);
-    return cnt;
+    return __popc(bal);
 }
 
-__device__ __forceinline__ float4 box_min(float4 a, float4 b) {
-    return make_float4(fminf(a.x, b.x), fminf(a.y, b.y), fminf(a.z, b.z), 0.f);
+// Pads a run of nz points that ends at slot `end` to an even count: a copy of
+// the last point with E = 0 (finite, adds zero, not counted).  One lane, after
+// a __syncwarp.
+__device__ __forceinline__ void nz_pad(NzPoints &nzp, int end) {
+    nzp.at(0, end) = nzp.at(0, end - 1);
+    nzp.at(1, end) = nzp.at(1, end - 1);
+    nzp.at(2, end) = nzp.at(2, end - 1);
+    nzp.at(3, end) = 0.f;
 }
-__device__ __forceinline__ float4 box_max(float4 a, float4 b) {
-    return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), 0.f);
+
+// A lane's share of the box of the nz points (empty: +inf / -inf), and the
+// warp's box of the lanes' shares.
+__device__ __forceinline__ void nz_grow(float4 &lo, float4 &hi, bool nz, float x, float y, float z) {
+    if (nz) {
+        lo = make_float4(fminf(lo.x, x), fminf(lo.y, y), fminf(lo.z, z), 0.f);
+        hi = make_float4(fmaxf(hi.x, x), fmaxf(hi.y, y), fmaxf(hi.z, z), 0.f);
+    }
+}
+__device__ __forceinline__ void nz_box(float4 &lo, float4 &hi) {
+    lo = make_float4(redux_min(lo.x), redux_min(lo.y), redux_min(lo.z), 0.f);
+    hi = make_float4(redux_max(hi.x), redux_max(hi.y), redux_max(hi.z), 0.f);
 }
 
 // ---------------------------------------------------------------- scheduling
@@ -727,7 +739,7 @@ __device__ __forceinline__ float4 box_max(float4 a, float4 b) {
 // whatever the order, and the loss partials are reduced by tile index, so
 // the order never changes a result.
 __device__ __forceinline__ uint4 resolve(const FwdArgs &a, uint32_t k) {
-    return (int64_t)k < a.nitems ? a.order_rec[k] : make_uint4(0u, 0u, 0u, 0u);  // w = 0: none left
+    return (int64_t)k < a.nitems ? a.order_rec[k] : make_uint4(~0u, 0u, 0u, 0u);  // x = ~0: none left
 }
 
 // Class of a measured cost: 0 below mean / 4, then about one class per half
@@ -779,11 +791,11 @@ struct FwdBatch {
 constexpr int kMaxBatchFields = 1024;
 
 // Item k of the batch: its field (binary search of the item offsets, read
-// through the read-only cache) and record; w = 0 when none is left.
+// through the read-only cache) and record; x = ~0 when none is left.
 __device__ __forceinline__ uint4 resolve_batch(const FwdBatch &b, uint32_t k, uint32_t &field) {
     const uint32_t *off = b.item_off;
     field = 0;
-    if (k >= __ldg(off + b.nfields)) return make_uint4(0u, 0u, 0u, 0u);
+    if (k >= __ldg(off + b.nfields)) return make_uint4(~0u, 0u, 0u, 0u);
     int lo = 0, hi = b.nfields - 1;  // largest f with off[f] <= k
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -828,6 +840,7 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     // gathers gets what the blocks leave of the SM's unified 256 KB.  The
     // rings are idle during the adjoint, so the nz points live in warp 0's
     // first ring and each warp's adjoint queue in its second.
+    constexpr int NT = G > 1 ? 2 : kMostTiles;  // tiles of an item (the points of a lane)
     constexpr int GR = G > 1 ? G : 1;    // the cross-warp sums exist only for G > 1
     constexpr int RL = G > 1 ? 32 : 1;
     constexpr int kTouchW = G > 1 ? kTouch / 2 : kTouch;  // kernels remembered per warp
@@ -859,11 +872,11 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
         }
     }
     __syncthreads();
-    uint4 rec = s_rec;  // the item's record; no points (w = 0) when done
+    uint4 rec = s_rec;  // the item's record; x = ~0 when done
     uint32_t field = BATCH ? s_field : 0u, loaded = ~0u;
     uint32_t mean = BATCH ? 0u : a1.sched[0];
     const FwdArgs &a = BATCH ? *reinterpret_cast<const FwdArgs *>(s_args) : a1;
-    while (rec.w != 0u) {
+    while (rec.x != ~0u) {
         if (BATCH && field != loaded) {
             // the block's threads copy the field's arguments (block-uniform
             // branch: every thread holds the same record and field)
@@ -875,46 +888,65 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             loaded = field;
             mean = a.sched[0];
         }
-        const ItemInfo it = item_info(rec, lane);
+        const ItemInfo it = item_info(rec);
         // the next claim is made now, its record is fetched after the sums
         // and used at the end, so neither round trip is on the item's path
         uint32_t knext = 0, fnext = 0;
         if (threadIdx.x == 0) knext = atomicAdd(BATCH ? b.next : a.item_next, 1u);
-        f2 acc[2];
-        uint32_t n[2], cost;
+        f2 acc[NT];
+        uint32_t n[NT], cost;
         int ntouch = 0;
-        float tv[2];
-        forward_share<G, ADJ>(a, it, warp, ringP[warp], ringF[warp], lane, acc, n, cost, touch[ADJ ? warp : 0],
-                              kTouchW, ntouch, tv);
-        uint4 rn = make_uint4(0u, 0u, 0u, 0u);
+        forward_share<G, ADJ>(a, it, warp, ringP[warp], ringF[warp], lane, acc, n, cost, touch[ADJ ? warp : 0], kTouchW,
+                              ntouch);
+        uint4 rn = make_uint4(~0u, 0u, 0u, 0u);
         if (threadIdx.x == 0) rn = BATCH ? resolve_batch(b, knext, fnext) : resolve(a, knext);
         if constexpr (G == 1) {
-            // one warp: finish both tiles directly
-            float l0, h0, l1, h1;
-            f2_unpack(acc[0], l0, h0);
-            f2_unpack(acc[1], l1, h1);
-            float l2[2], mx[2];
-            uint32_t cnt[2], pr[2];
-            const float e0 = point_out(a, it.i0, it.v0, tv[0], l0 + h0, n[0], l2[0], mx[0], cnt[0], pr[0]);
-            const float e1 = point_out(a, it.i1, it.v1, tv[1], l1 + h1, n[1], l2[1], mx[1], cnt[1], pr[1]);
-            finish_item(a, it.t0, it.two, two_sum(l2[0], l2[1]), fmaxf(mx[0], mx[1]), cnt[0] + cnt[1],
-                        pr[0] + pr[1], lane);
-            if (ADJ) {
+            // one warp: finish the tiles directly
+            float tv[NT], ev[NT];
+#pragma unroll
+            for (int p = 0; p < NT; ++p) tv[p] = lane + p * kTile < it.np ? a.t[it.i0 + lane + p * kTile] : 0.f;
+            ff l2 = {0.f, 0.f};
+            float mx = 0.f;
+            uint32_t cnt = 0u, pr = 0u, pb = 0u, ebits = 0u;
+#pragma unroll
+            for (int p = 0; p < NT; ++p) {
+                float l0, h0, l2p, mxp;
+                uint32_t cntp, prp;
+                f2_unpack(acc[p], l0, h0);
+                ev[p] = point_out(a, it.i0 + lane + p * kTile, lane + p * kTile < it.np, tv[p], l0 + h0, n[p], l2p, mxp,
+                                  cntp, prp);
+                l2 = ff_add(l2, l2p);
+                mx = fmaxf(mx, mxp);
+                cnt += cntp;
+                pr += prp;
                 // adjoint pairs: every support pair of a point with E != 0
                 // (the adjoint takes exactly these)
-                const uint32_t pb = redux_add((e0 != 0.f ? n[0] : 0u) + (e1 != 0.f ? n[1] : 0u));
+                pb += ev[p] != 0.f ? n[p] : 0u;
+                ebits = max(ebits, __float_as_uint(fabsf(ev[p])));
+            }
+            finish_item(a, it.t0, it.ntl, l2, mx, cnt, pr, lane);
+            if (ADJ) ebits = redux_max_u32(ebits);
+            if (ADJ && ebits != 0u) {
+                pb = redux_add(pb);
                 if (lane == 0 && pb) atomicAdd(a.adj_pairs, (unsigned long long)pb);
-                float4 lo0, hi0, lo1, hi1;
-                const int nc0 = nz_tile(nzs, 0, e0 != 0.f, a.x[it.v0 ? it.i0 : 0], a.y[it.v0 ? it.i0 : 0],
-                                        a.z[it.v0 ? it.i0 : 0], e0, lane, lo0, hi0);
-                const int nc1 = nz_tile(nzs, kTile, e1 != 0.f, a.x[it.v1 ? it.i1 : 0], a.y[it.v1 ? it.i1 : 0],
-                                        a.z[it.v1 ? it.i1 : 0], e1, lane, lo1, hi1);
+                float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+                float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+                int nc = 0;
+#pragma unroll
+                for (int p = 0; p < NT; ++p) {
+                    if (p < it.ntl) {
+                        const int64_t i = it.i0 + (lane + p * kTile < it.np ? lane + p * kTile : 0);
+                        const float x = a.x[i], y = a.y[i], z = a.z[i];
+                        nz_grow(lo, hi, ev[p] != 0.f, x, y, z);
+                        nc += nz_tile(nzs, nc, ev[p] != 0.f, x, y, z, ev[p], lane);
+                    }
+                }
+                nz_box(lo, hi);
                 __syncwarp();
-                const float emax = __uint_as_float(
-                    redux_max_u32(max(__float_as_uint(fabsf(e0)), __float_as_uint(fabsf(e1)))));
-                if (nc0 + nc1 > 0)
-                    adjoint_share<1, (ADJ > 1)>(a, it, 0, nzs, nc0, nc1, box_min(lo0, lo1), box_max(hi0, hi1), touch[0],
-                                                ntouch, kTouchW, emax, adjq, lane, cost);
+                if ((nc & 1) && lane == 0) nz_pad(nzs, nc);
+                __syncwarp();
+                adjoint_share<1, (ADJ > 1)>(a, it, 0, nzs, (uint32_t)nc, nc, lo, hi, touch[0], ntouch, kTouchW,
+                                            __uint_as_float(ebits), adjq, lane, cost);
                 __syncwarp();
             }
             if (lane == 0) note_cost(a, mean, rec, cost);
@@ -935,7 +967,7 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
         }
         __syncthreads();
         // warp 0 finishes the first tile, warp 1 the second (if any)
-        if (warp < 2 && (warp == 0 || it.two)) {
+        if (warp < it.ntl) {
             float ps = 0.f;
             uint32_t np = 0;
 #pragma unroll
@@ -947,24 +979,30 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             }
             float l2, mx;
             uint32_t cnt, pr;
-            const int64_t i = warp ? it.i1 : it.i0;
-            const bool v = warp ? it.v1 : it.v0;
-            const float e = point_out(a, i, v, warp ? tv[1] : tv[0], ps, np, l2, mx, cnt, pr);
+            const int64_t i = it.i0 + lane + warp * kTile;
+            const bool v = lane + warp * kTile < it.np;
+            const float e = point_out(a, i, v, v ? a.t[i] : 0.f, ps, np, l2, mx, cnt, pr);
             finish_tile(a, it.t0 + warp, l2, mx, cnt, pr, lane);
             if (ADJ) {
                 const float emax = __uint_as_float(redux_max_u32(__float_as_uint(fabsf(e))));
                 // adjoint pairs: every support pair of a point with E != 0
                 const uint32_t pb = redux_add(e != 0.f ? np : 0u);
                 if (lane == 0 && pb) atomicAdd(a.adj_pairs, (unsigned long long)pb);
-                float4 lo, hi;
-                const int nc = nz_tile(nzs, kTile * warp, e != 0.f, a.x[v ? i : 0], a.y[v ? i : 0],
-                                       a.z[v ? i : 0], e, lane, lo, hi);
+                float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+                float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+                const int64_t iv = v ? i : it.i0;
+                const float x = a.x[iv], y = a.y[iv], z = a.z[iv];
+                const int nc = nz_tile(nzs, kTile * warp, e != 0.f, x, y, z, e, lane);
+                nz_grow(lo, hi, e != 0.f, x, y, z);
+                nz_box(lo, hi);
+                __syncwarp();
+                if ((nc & 1) && lane == 0) nz_pad(nzs, kTile * warp + nc);
                 if (lane == 0) {
                     s_nc[warp] = nc;
                     lo.w = emax;
                     s_box[warp][0] = lo;
                     s_box[warp][1] = hi;
-                    if (warp == 0 && !it.two) s_nc[1] = 0;
+                    if (warp == 0 && it.ntl < 2) s_nc[1] = 0;
                 }
             }
             if (warp == 0 && lane == 0) {
@@ -987,8 +1025,8 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
                 uint32_t c = 0;
                 const float emax = __uint_as_float(
                     max(nc0 ? __float_as_uint(s_box[0][0].w) : 0u, nc1 ? __float_as_uint(s_box[1][0].w) : 0u));
-                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, nc0, nc1, lo, hi, touch[warp], ntouch, kTouchW, emax,
-                                            adjq, lane, c);
+                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, (uint32_t)(nc0 | nc1 << 8), nc0 + nc1, lo, hi, touch[warp],
+                                            ntouch, kTouchW, emax, adjq, lane, c);
                 if (lane == 0) red_cost[warp] += c;
             }
             __syncthreads();
@@ -1014,11 +1052,12 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     }
 }
 
-// Resident warps per SM (the register budget): 20 for the fused variants
-// with 1 or 2 warps per item and 16 with 4, 24 for eight warps and for the
-// forward alone (20 with one warp); measured on the 128^3 and 256^3 fields,
-// other bounds were slower.
-#define SERBF_FWD_BOUNDS(G, ADJ) __launch_bounds__(G * 32, (G == 8 ? 24 : (ADJ ? (G == 4 ? 16 : 20) : (G == 1 ? 20 : 24))) / G)
+// Resident warps per SM (the register budget): 16 with one warp per item (four
+// points per lane: 126 registers; 20 warps spill 80 bytes and took 2158 us
+// instead of 2085 for 9.4 M points) and with four, 20 for the fused variant
+// with two, 24 with eight and for the forward alone with two or four; measured
+// on the 128^3 and 256^3 fields, other bounds were slower.
+#define SERBF_FWD_BOUNDS(G, ADJ) __launch_bounds__(G * 32, (G == 1 ? 16 : (G == 8 ? 24 : (ADJ ? (G == 4 ? 16 : 20) : 24))) / G)
 
 template <int G, int ADJ>
 __global__ void SERBF_FWD_BOUNDS(G, ADJ) k_forward(FwdArgs a) {
@@ -1188,9 +1227,10 @@ __global__ void __launch_bounds__(kFinishThreads) k_fwd_finish_batch(const Finis
     fwd_finish_body<ADJ>(f, blockIdx.x, gridDim.x);
 }
 
-// The arguments of one forward (+ adjoint) call; false on bad arguments.
+// The arguments of one forward (+ adjoint) call with G warps per item; false
+// on bad arguments.
 bool make_args(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg, float *psi, float *err,
-               uint8_t *mask, float *grad, double *stats, serbf_workspace *ws, FwdArgs &a, FinishArgs &f,
+               uint8_t *mask, float *grad, double *stats, serbf_workspace *ws, int G, FwdArgs &a, FinishArgs &f,
                int64_t &finish_blocks) {
     if (!pts || !prm || !cfg || !ws || ws->magic != kMagic || !ws->binned) return false;
     if (pts->n != ws->npoints || !prm->m || !prm->p) return false;
@@ -1206,13 +1246,12 @@ bool make_args(const serbf_points *pts, const serbf_params *prm, const serbf_con
     a.t = pts->t;
     a.tile_super = ws->tile_super;
     a.stile0 = ws->super_tile0;
-    a.item_rec = ws->item_rec;
-    a.order_rec = ws->order_rec;
-    a.item_class = ws->item_class;
-    a.sched = ws->sched;
-    a.sched_total = ws->sched_total;
-    a.max_items = ws->max_items;
-    a.nitems = ws->nitems;
+    const ItemSet &items = items_of(ws, G);
+    a.order_rec = items.order;
+    a.item_class = items.cls;
+    a.sched = items.sched;
+    a.sched_total = items.total;
+    a.nitems = items.n;
     a.tile_start = ws->tile_start;
     a.cell_start = ws->cell_start;
     a.tile_lo = ws->tile_lo;
@@ -1263,33 +1302,19 @@ bool make_args(const serbf_points *pts, const serbf_params *prm, const serbf_con
     return true;
 }
 
-// Warps per item, unless the configuration fixes it.  Items differ in cost
-// (an item in the middle of the kernels whose points all carry residuals costs
-// five times the mean and more), so a launch with few items per warp waits for
-// its heaviest ones; more warps per item shorten that tail and cost issue slots
-// for barriers and short batches.  Measured crossings on a 152-SM part, fused
-// call in us with 1 / 2 / 4 warps: 8.0 k items (80^3) 149 / 106 / 93, 14.6 k
-// (97^3, compensated) 251 / 181 / 172, 20.8 k (110^3) 243 / 194 / 226, 32.8 k
-// (128^3) 318 / 292 / 364, 147 k (9.4 M points) 2118 / 2280 / 2801; 8 warps were
-// within 3 % of 4 below 2 k items and slower above.
-int pick_warps(int64_t nitems, int sm_count, int fixed) {
-    if (fixed == 1 || fixed == 2 || fixed == 4 || fixed == 8) return fixed;
-    const int64_t resident = 20 * (int64_t)sm_count;  // warps in flight
-    return nitems >= 16 * resident ? 1 : (nitems >= 6 * resident ? 2 : 4);
-}
-
 int forward_impl(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg, float *psi, float *err,
                  uint8_t *mask, float *grad, double *stats, serbf_workspace *ws, void *stream) {
     FwdArgs a;
     FinishArgs f;
     int64_t nb = 1;
-    if (!make_args(pts, prm, cfg, psi, err, mask, grad, stats, ws, a, f, nb)) return SERBF_EINVAL;
+    if (!cfg || !ws || ws->magic != kMagic) return SERBF_EINVAL;
+    const int G = forward_warps(ws->items[0].n, ws->sm_count, cfg->fwd_warps);
+    if (!make_args(pts, prm, cfg, psi, err, mask, grad, stats, ws, G, a, f, nb)) return SERBF_EINVAL;
     const bool adj = grad != nullptr;
     cudaStream_t s = (cudaStream_t)stream;
     int rc = SERBF_OK;
     if (ws->ntiles > 0) {
-        const int64_t ni = ws->nitems;
-        const int G = pick_warps(ni, ws->sm_count, cfg->fwd_warps);
+        const int64_t ni = a.nitems;
         const int mode = adj ? (cfg->kahan ? 2 : 1) : 0;
         switch (G * 4 + mode) {
             case 4: rc = launch_forward<1, 0>(a, ni, ws->sm_count, s); break;
@@ -1338,23 +1363,36 @@ int launch_forward_batch(const FwdBatch &b, int64_t nitems, int sm_count, cudaSt
 
 namespace serbf {
 
+// Warps per item, unless the configuration fixes it.  Items differ in cost
+// (an item in the middle of the kernels whose points all carry residuals costs
+// five times the mean and more), so a launch with few items per warp waits for
+// its heaviest ones; more warps per item shorten that tail and cost issue slots
+// for barriers and short batches.  Measured crossings on a 152-SM part, fused
+// call in us with 1 / 2 / 4 warps: 8.0 k items (80^3) 149 / 106 / 93, 14.6 k
+// (97^3, compensated) 251 / 181 / 172, 20.8 k (110^3) 243 / 194 / 226, 32.8 k
+// (128^3) 318 / 292 / 364, 147 k (9.4 M points) 2118 / 2280 / 2801; 8 warps were
+// within 3 % of 4 below 2 k items and slower above.
+int forward_warps(int64_t items2, int sm_count, int fixed) {
+    if (fixed == 1 || fixed == 2 || fixed == 4 || fixed == 8) return fixed;
+    const int64_t resident = 20 * (int64_t)sm_count;  // warps in flight
+    return items2 >= 16 * resident ? 1 : (items2 >= 6 * resident ? 2 : 4);
+}
+
 size_t fwd_args_size() { return sizeof(FwdArgs); }
 size_t finish_args_size() { return sizeof(FinishArgs); }
 
 // Host records of one field's fused forward + adjoint (out: sizeof(FwdArgs)
 // and sizeof(FinishArgs) bytes) and the finishing kernel's block count.
 int batch_forward_args(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg, float *psi,
-                       float *err, uint8_t *mask, float *grad, double *stats, serbf_workspace *ws, void *fwd_out,
+                       float *err, uint8_t *mask, float *grad, double *stats, serbf_workspace *ws, int G, void *fwd_out,
                        void *fin_out, int64_t *finish_blocks) {
     FwdArgs a;
     FinishArgs f;
-    if (!make_args(pts, prm, cfg, psi, err, mask, grad, stats, ws, a, f, *finish_blocks)) return SERBF_EINVAL;
+    if (!make_args(pts, prm, cfg, psi, err, mask, grad, stats, ws, G, a, f, *finish_blocks)) return SERBF_EINVAL;
     memcpy(fwd_out, &a, sizeof(a));
     memcpy(fin_out, &f, sizeof(f));
     return SERBF_OK;
 }
-
-int batch_pick_warps(int64_t nitems, int sm_count, int fixed) { return pick_warps(nitems, sm_count, fixed); }
 
 // One persistent launch over the items of every field, then the finishing
 // kernel of every field (grid.y = field).  args / fin / item_off / counters

@@ -629,7 +629,7 @@ size_t rebuild_args_size() { return sizeof(RebuildArgs); }
 // sizeof(RebuildArgs) bytes); *level1_blocks, *chunks and *parents (blocks of
 // super cells of a field that takes two levels, else 0) size the batch's grids.
 int batch_rebuild_args(const serbf_points *pts, const serbf_params *prm, const serbf_config *cfg,
-                       serbf_workspace *ws, void *out, int *level1_blocks, int64_t *chunks, int *parents) {
+                       serbf_workspace *ws, int warps, void *out, int *level1_blocks, int64_t *chunks, int *parents) {
     if (!pts || !prm || !cfg || !ws_ok(ws)) return SERBF_EINVAL;
     if (!prm->p || !prm->m || prm->cap < 1 || prm->cap > ws->sz.max_kernels) return SERBF_EINVAL;
     if (pts->n != ws->npoints) return SERBF_EINVAL;
@@ -661,14 +661,15 @@ int batch_rebuild_args(const serbf_points *pts, const serbf_params *prm, const s
     r.status = ws->status;
     r.needed = ws->needed;
     r.level1_blocks = (r.two_level ? (int)ncoarse : ws->nsuper) + prep_blocks;
-    r.item_class = ws->item_class;
+    const ItemSet &items = items_of(ws, warps);
+    r.item_class = items.cls;
     r.class_hist = ws->class_hist;
-    r.item_rec = ws->item_rec;
-    r.order_rec = ws->order_rec;
-    r.nitems = ws->nitems;
+    r.item_rec = items.rec;
+    r.order_rec = items.order;
+    r.nitems = items.n;
     memcpy(out, &r, sizeof(r));
     *level1_blocks = r.level1_blocks;
-    *chunks = (ws->nitems + kOrderChunk - 1) / kOrderChunk;
+    *chunks = (items.n + kOrderChunk - 1) / kOrderChunk;
     *parents = r.two_level ? r.ncoarse : 0;
     return SERBF_OK;
 }
@@ -702,14 +703,14 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
     if (pmajor && (!pmajor->rowptr || (pmajor->cap > 0 && !pmajor->col))) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     // fork: the item order for the next forward overlaps the rebuild
-    const bool fork = ws->nitems > 0 && ws->aux;
+    const ItemSet &items = items_of(ws, forward_warps(ws->items[0].n, ws->sm_count, cfg->fwd_warps));
+    const bool fork = items.n > 0 && ws->aux;
     if (fork) {
         if (cudaEventRecord(ws->ev_fork, s) != cudaSuccess) return SERBF_ECUDA;
         if (cudaStreamWaitEvent(ws->aux, ws->ev_fork, 0) != cudaSuccess) return SERBF_ECUDA;
-        const unsigned nchunks = (unsigned)((ws->nitems + kOrderChunk - 1) / kOrderChunk);
-        k_class_count<<<nchunks, kOrderChunk, 0, ws->aux>>>(ws->item_class, ws->nitems, ws->class_hist);
-        k_order_items<<<nchunks, kOrderChunk, 0, ws->aux>>>(ws->item_class, ws->class_hist, ws->item_rec,
-                                                            ws->order_rec, ws->nitems);
+        const unsigned nchunks = (unsigned)((items.n + kOrderChunk - 1) / kOrderChunk);
+        k_class_count<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, items.n, ws->class_hist);
+        k_order_items<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, ws->class_hist, items.rec, items.order, items.n);
         SERBF_CHECK_LAUNCH();
         if (cudaEventRecord(ws->ev_join, ws->aux) != cudaSuccess) return SERBF_ECUDA;
     }
