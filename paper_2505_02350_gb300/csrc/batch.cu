@@ -18,12 +18,13 @@ size_t fwd_args_size();
 size_t finish_args_size();
 int batch_forward_args(const serbf_points *, const serbf_params *, const serbf_config *, float *, float *, uint8_t *,
                        float *, double *, serbf_workspace *, int, void *, void *, int64_t *);
-int batch_forward_launch(const void *args, const void *fin, const uint32_t *item_off, int nfields, uint32_t *counters,
+int batch_forward_launch(const void *args, const void *fin, const uint32_t *table, int nfields, uint32_t *counters,
                          int64_t total_items, int64_t finish_blocks, int G, int kahan, int sm_count, cudaStream_t s);
 size_t rebuild_args_size();
 int batch_rebuild_args(const serbf_points *, const serbf_params *, const serbf_config *, serbf_workspace *, int, void *,
                        int *, int64_t *, int *);
-int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, cudaStream_t s);
+int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, uint32_t *table,
+                         cudaStream_t s);
 size_t step_args_size();
 int batch_step_args(serbf_params *, const float *, float *, float *, serbf_state *, double *, const serbf_config *,
                     serbf_workspace *, void *, int *);
@@ -44,7 +45,7 @@ size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
 // Device layout of the batch tables, in this order, each 256-byte aligned.
 struct Layout {
-    size_t fwd, fin, reb, step, add, off, ctr, total;
+    size_t fwd, fin, reb, step, add, table, ctr, total;
 };
 
 Layout layout(int n) {
@@ -60,8 +61,8 @@ Layout layout(int n) {
     o = up256(o + (size_t)n * step_args_size());
     L.add = o;
     o = up256(o + (size_t)n * add_args_size());
-    L.off = o;
-    o = up256(o + (size_t)(n + 1) * sizeof(uint32_t));
+    L.table = o;  // the order over all fields' items: positions and places by class and field
+    o = up256(o + (size_t)(2 * kCostClasses * n + 1) * sizeof(uint32_t));
     L.ctr = o;
     o = up256(o + 16 * sizeof(uint32_t));
     L.total = o;
@@ -100,7 +101,6 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     int64_t total = 0, fin_blocks = 1, chunks = 0;
     int lvl1 = 1, parents = 0, step_nb = 1, sm = 0;
     const int kahan = fields[0].cfg ? fields[0].cfg->kahan : 0;
-    uint32_t *off = reinterpret_cast<uint32_t *>(host.data() + L.off);
     int64_t items2 = 0;
     for (int f = 0; f < nfields; ++f) {
         const serbf_field &F = fields[f];
@@ -125,7 +125,6 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
                                      F.ws, host.data() + L.add + (size_t)f * add_args_size());
         if (rc) return rc;
         if (!F.grad) return SERBF_EINVAL;
-        off[f] = (uint32_t)total;
         total += items_of(F.ws, G).n;
         if (total >= (int64_t)1 << 32) return SERBF_ECAPACITY;
         fin_blocks = fb > fin_blocks ? fb : fin_blocks;
@@ -134,7 +133,6 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
         parents = pa > parents ? pa : parents;
         step_nb = nb > step_nb ? nb : step_nb;
     }
-    off[nfields] = (uint32_t)total;
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaMemcpyAsync(dev, host.data(), L.total, cudaMemcpyHostToDevice, s) != cudaSuccess) return SERBF_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
@@ -162,9 +160,10 @@ int serbf_epoch_batched(serbf_batch *b, void *stream) {
     if (!b || b->magic != kBatchMagic) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     char *d = b->base;
-    int rc = batch_rebuild_launch(d + b->L.reb, b->nfields, b->level1_blocks, b->chunks, b->parents, s);
+    int rc = batch_rebuild_launch(d + b->L.reb, b->nfields, b->level1_blocks, b->chunks, b->parents,
+                                  reinterpret_cast<uint32_t *>(d + b->L.table), s);
     if (!rc)
-        rc = batch_forward_launch(d + b->L.fwd, d + b->L.fin, reinterpret_cast<const uint32_t *>(d + b->L.off),
+        rc = batch_forward_launch(d + b->L.fwd, d + b->L.fin, reinterpret_cast<const uint32_t *>(d + b->L.table),
                                   b->nfields, reinterpret_cast<uint32_t *>(d + b->L.ctr), b->total_items,
                                   b->finish_blocks, b->G, b->kahan, b->sm_count, s);
     if (!rc) rc = batch_step_launch(d + b->L.step, b->nfields, b->step_nb, s);

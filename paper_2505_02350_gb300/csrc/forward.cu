@@ -446,8 +446,8 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
 #pragma unroll
     for (int p = 0; p < NT; ++p) n[p] += nfull;
     // about one unit per filtered candidate, ~6 per fully and ~9 per partly
-    // covering kernel
-    cost = 32u * (uint32_t)nchunks + 6u * nfull + 9u * npart;
+    // covering kernel and two points of a lane
+    cost = 32u * (uint32_t)nchunks + (6u * nfull + 9u * npart) * (NT / 2);
 }
 
 // ---------------------------------------------------------------- fused adjoint
@@ -780,46 +780,63 @@ __device__ __forceinline__ void sched_finish(const FwdArgs &a) {
 }
 
 // A batch of fields advanced by one launch: the fields' arguments in device
-// memory and their work items concatenated in field order (item_off: prefix
-// sums of the item counts).  Blocks claim from one counter over all items.
+// memory and one order over all their work items, heaviest class first and by
+// field within a class (classes are relative to the mean cost of all items, so
+// they compare across fields).  Blocks claim positions of that order from one
+// counter.  Entry e = (7 - class) nfields + field of the table: its first
+// position in the order, and its first place in the field's own order.  (Taken
+// field after field, the last field's heavy items came last and the SMs were
+// busy 73 % of the launch for 16 fields.)
 struct FwdBatch {
     const FwdArgs *args;
-    const uint32_t *item_off;  // nfields + 1
+    const uint32_t *pos;    // kCostClasses x nfields + 1
+    const uint32_t *place;  // kCostClasses x nfields
     int nfields;
-    uint32_t *next, *exit;     // claim and exit counters (zero between launches)
+    uint32_t *next, *exit;  // claim and exit counters (zero between launches)
 };
 constexpr int kMaxBatchFields = 1024;
 
-// Item k of the batch: its field (binary search of the item offsets, read
+// Item k of the batch: its field (binary search of the positions, read
 // through the read-only cache) and record; x = ~0 when none is left.
 __device__ __forceinline__ uint4 resolve_batch(const FwdBatch &b, uint32_t k, uint32_t &field) {
-    const uint32_t *off = b.item_off;
+    const int n = kCostClasses * b.nfields;
     field = 0;
-    if (k >= __ldg(off + b.nfields)) return make_uint4(~0u, 0u, 0u, 0u);
-    int lo = 0, hi = b.nfields - 1;  // largest f with off[f] <= k
+    if (k >= __ldg(b.pos + n)) return make_uint4(~0u, 0u, 0u, 0u);
+    int lo = 0, hi = n - 1;  // largest e with pos[e] <= k
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(off + mid) <= k) lo = mid; else hi = mid - 1;
+        if (__ldg(b.pos + mid) <= k) lo = mid; else hi = mid - 1;
     }
-    field = (uint32_t)lo;
-    return b.args[lo].order_rec[k - off[lo]];
+    field = (uint32_t)(lo % b.nfields);
+    return b.args[field].order_rec[__ldg(b.place + lo) + (k - __ldg(b.pos + lo))];
 }
 
-// Last block out of a batch launch: every field's mean cost, and the batch
-// counters reset.
-__device__ __forceinline__ void sched_finish_batch(const FwdBatch &b) {
-    __threadfence();
-    if (atomicAdd(b.exit, 1u) != gridDim.x - 1) return;
-    __threadfence();
-    for (int f = 0; f < b.nfields; ++f) {
-        const FwdArgs &a = b.args[f];
-        const unsigned long long tot = __ldcg(a.sched_total);
-        const unsigned long long mean = a.nitems > 0 ? tot / (unsigned long long)a.nitems : 0ull;
-        a.sched[0] = (uint32_t)min(mean, 0xffffffffull);
-        *a.sched_total = 0ull;
+// Last block out of a batch launch (one warp): the mean cost of all fields'
+// items, and the batch counters reset.
+__device__ __forceinline__ void sched_finish_batch(const FwdBatch &b, int lane) {
+    int last = 0;
+    if (lane == 0) {
+        __threadfence();
+        last = atomicAdd(b.exit, 1u) == gridDim.x - 1;
     }
-    *b.next = 0u;
-    *b.exit = 0u;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    unsigned long long tot = 0ull, items = 0ull;
+    for (int f = lane; f < b.nfields; f += 32) {
+        tot += __ldcg(b.args[f].sched_total);
+        items += (unsigned long long)b.args[f].nitems;
+    }
+    tot = warp_sum(tot);
+    items = warp_sum(items);
+    const uint32_t mean = (uint32_t)min(items ? tot / items : 0ull, 0xffffffffull);
+    for (int f = lane; f < b.nfields; f += 32) {
+        b.args[f].sched[0] = mean;
+        *b.args[f].sched_total = 0ull;
+    }
+    if (lane == 0) {
+        *b.next = 0u;
+        *b.exit = 0u;
+    }
 }
 
 // Persistent blocks take work items, heaviest first, from a global counter.
@@ -1044,11 +1061,10 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     }
     // the last block out prepares the next launch: every block has made its
     // last claim and recorded its costs before it counts itself out
-    if (threadIdx.x == 0) {
-        if (BATCH)
-            sched_finish_batch(b);
-        else
-            sched_finish(a1);
+    if (BATCH) {
+        if (warp == 0) sched_finish_batch(b, lane);
+    } else if (threadIdx.x == 0) {
+        sched_finish(a1);
     }
 }
 
@@ -1395,12 +1411,12 @@ int batch_forward_args(const serbf_points *pts, const serbf_params *prm, const s
 }
 
 // One persistent launch over the items of every field, then the finishing
-// kernel of every field (grid.y = field).  args / fin / item_off / counters
-// are device arrays written by the batch set-up.
-int batch_forward_launch(const void *args, const void *fin, const uint32_t *item_off, int nfields, uint32_t *counters,
+// kernel of every field (grid.y = field).  args / fin / counters are device
+// arrays written by the batch set-up, table by the batched rebuild.
+int batch_forward_launch(const void *args, const void *fin, const uint32_t *table, int nfields, uint32_t *counters,
                          int64_t total_items, int64_t finish_blocks, int G, int kahan, int sm_count, cudaStream_t s) {
     if (nfields < 1 || nfields > kMaxBatchFields) return SERBF_EINVAL;
-    FwdBatch b{static_cast<const FwdArgs *>(args), item_off, nfields, counters, counters + 1};
+    FwdBatch b{static_cast<const FwdArgs *>(args), table, table + kCostClasses * nfields + 1, nfields, counters, counters + 1};
     int rc = SERBF_OK;
     if (total_items > 0) {
         switch (G * 2 + (kahan ? 1 : 0)) {

@@ -434,7 +434,41 @@ __global__ void __launch_bounds__(kOrderChunk) k_class_count_batch(const Rebuild
     class_count_body(r.item_class, r.nitems, r.class_hist, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kOrderChunk) k_order_items_batch(const RebuildArgs *ra) {
+// The batch's table of its order over all fields' items (see FwdBatch): pos,
+// then place.  One block; a thread per (class, field) sums the chunks' counts.
+__device__ __forceinline__ void order_table_body(const RebuildArgs *ra, int nfields, uint32_t *table) {
+    __shared__ uint32_t tmp[33];
+    const int n = kCostClasses * nfields;
+    uint32_t *pos = table, *place = table + n + 1;
+    uint32_t carry = 0;
+    for (int e0 = 0; e0 < n; e0 += blockDim.x) {
+        const int e = e0 + threadIdx.x, f = e % nfields, c = kCostClasses - 1 - e / nfields;
+        uint32_t count = 0, heavier = 0;
+        if (e < n) {
+            const RebuildArgs &r = ra[f];
+            const int64_t chunks = (r.nitems + kOrderChunk - 1) / kOrderChunk;
+            for (int64_t q = 0; q < chunks; ++q) {
+                count += r.class_hist[q * kCostClasses + c];
+                for (int h = c + 1; h < kCostClasses; ++h) heavier += r.class_hist[q * kCostClasses + h];
+            }
+        }
+        uint32_t total;
+        const uint32_t o = block_exscan(count, tmp, &total);
+        if (e < n) {
+            pos[e] = carry + o;
+            place[e] = heavier;
+        }
+        carry += total;
+    }
+    if (threadIdx.x == 0) pos[n] = carry;
+}
+
+// The row of blocks past the longest field's chunks makes the table.
+__global__ void __launch_bounds__(kOrderChunk) k_order_items_batch(const RebuildArgs *ra, int nfields, uint32_t *table) {
+    if (blockIdx.x == gridDim.x - 1) {
+        if (blockIdx.y == 0) order_table_body(ra, nfields, table);
+        return;
+    }
     const RebuildArgs &r = ra[blockIdx.y];
     if ((int64_t)blockIdx.x * kOrderChunk >= r.nitems) return;
     order_items_body(r.item_class, r.class_hist, r.item_rec, r.order_rec, r.nitems, blockIdx.x);
@@ -676,11 +710,12 @@ int batch_rebuild_args(const serbf_points *pts, const serbf_params *prm, const s
 
 // The batched rebuild: item order (two launches), then the lists and
 // records (one launch, two when some field takes two levels).
-int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, cudaStream_t s) {
+int batch_rebuild_launch(const void *args, int nfields, int level1_blocks, int64_t chunks, int parents, uint32_t *table,
+                         cudaStream_t s) {
     const RebuildArgs *ra = static_cast<const RebuildArgs *>(args);
     if (chunks > 0) {
         k_class_count_batch<<<dim3((unsigned)chunks, (unsigned)nfields), kOrderChunk, 0, s>>>(ra);
-        k_order_items_batch<<<dim3((unsigned)chunks, (unsigned)nfields), kOrderChunk, 0, s>>>(ra);
+        k_order_items_batch<<<dim3((unsigned)chunks + 1, (unsigned)nfields), kOrderChunk, 0, s>>>(ra, nfields, table);
     }
     launch_pdl(k_rebuild_batch, dim3((unsigned)level1_blocks, (unsigned)nfields), dim3(kListThreads), 0, s, ra);
     if (parents) launch_pdl(k_fine_lists_batch, dim3((unsigned)parents, (unsigned)nfields), dim3(kListThreads), 0, s, ra);
