@@ -331,9 +331,19 @@ __device__ __forceinline__ float4 box_max(float4 a, float4 b) {
     return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), 0.f);
 }
 
-// One warp's share of a work item: candidate chunks w, w + W, w + 2W, ... of
-// the super cell's list (32 candidates each) are filtered against the item
-// box, staged in pairs and evaluated against the lane's two points.
+// Warp w's share [b0, b1) of a list of n candidates: an equal run.  (Chunks
+// of 32 dealt round-robin gave a warp up to twice another's candidates when a
+// list holds one or two chunks per warp, and the others waited at the barrier.)
+template <int G>
+__device__ __forceinline__ void share_of(int n, int w, int &b0, int &b1) {
+    const int per = (n + G - 1) / G;
+    b0 = G > 1 ? w * per : 0;
+    b1 = G > 1 ? min(n, b0 + per) : n;
+}
+
+// One warp's share of a work item: its run of the super cell's list is
+// filtered against the item box, 32 candidates at a time,
+// staged in pairs and evaluated against the lane's points.
 // Returns the lane's partial sums and pair counts; *cost gets the warp's
 // measured work.
 template <int G, int ADJ, int NT>
@@ -363,14 +373,13 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
             hi = box_max(hi, a.tile_hi[it.t0 + p]);
         }
     const uint32_t *lst = a.slist + (size_t)it.sup * a.scap;
-    const int L = min((int)a.scnt[it.sup], a.scap);
-    constexpr int kStride = 32 * G;
+    int b0, L;
+    share_of<G>(min((int)a.scnt[it.sup], a.scap), w, b0, L);
     int hp = 0, qp = 0, hf = 0, qf = 0;
     uint32_t nfull = 0, npart = 0;
     // software pipeline: records of the next chunk and indices of the one
     // after it are in flight while a chunk is filtered
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int b0 = 32 * w;
     uint32_t jc = b0 + lane < L ? lst[b0 + lane] : 0u;
     float4 c0 = zero4, c1 = zero4, c2 = zero4;
     if (b0 + lane < L) {
@@ -378,20 +387,20 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
         c1 = a.kfwd[3 * jc + 1];
         c2 = a.kfwd[3 * jc + 2];
     }
-    uint32_t jn = b0 + kStride + lane < L ? lst[b0 + kStride + lane] : 0u;
+    uint32_t jn = b0 + 32 + lane < L ? lst[b0 + 32 + lane] : 0u;
     int nchunks = 0;
     ntouch = 0;
-    for (int b = b0; b < L; b += kStride) {
+    for (int b = b0; b < L; b += 32) {
         const float4 k0 = c0, k1 = c1, k2 = c2;
         const uint32_t j = jc;
         const bool live = b + lane < L;
-        if (b + kStride + lane < L) {
+        if (b + 32 + lane < L) {
             c0 = a.kfwd[3 * jn];
             c1 = a.kfwd[3 * jn + 1];
             c2 = a.kfwd[3 * jn + 2];
         }
         jc = jn;
-        if (b + 2 * kStride + lane < L) jn = lst[b + 2 * kStride + lane];
+        if (b + 64 + lane < L) jn = lst[b + 64 + lane];
         ++nchunks;
         float near2, far2;
         box_near_far_d2(k0.x, k0.y, k0.z, lo, hi, near2, far2);
@@ -662,14 +671,14 @@ __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t *lst = a.slist + (size_t)it.sup * a.scap;
     const bool listed = ntouch <= tcap;
-    const int L = listed ? ntouch : min((int)a.scnt[it.sup], a.scap);
-    const int b0 = listed ? 0 : 32 * w, stride = listed ? 32 : 32 * G;
+    int b0 = 0, L = ntouch;
+    if (!listed) share_of<G>(min((int)a.scnt[it.sup], a.scap), w, b0, L);
     const float4 mid = make_float4(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z), 0.f);
     const float ex = hi.x - lo.x, ey = hi.y - lo.y, ez = hi.z - lo.z;
     const float hd = 0.5001f * sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
     const float qlim = form_limit(emax, nc);
     int head = 0, qn = 0, nk = 0;
-    for (int b = b0; b < L; b += stride) {
+    for (int b = b0; b < L; b += 32) {
         const bool live = b + lane < L;
         const uint32_t j = live ? (listed ? touch[b + lane] : lst[b + lane]) : 0u;
         bool hit = false;
