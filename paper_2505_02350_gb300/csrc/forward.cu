@@ -280,7 +280,17 @@ __device__ __forceinline__ void finish_item(const FwdArgs &a, uint32_t t, int nt
     if (lane > 0 && lane < ntl) a.part[t + lane] = FwdPart{0.f, 0.f, 0.f, 0u, 0ull};
 }
 
-// Eq. 3-18 filter and residual of one point; returns its loss contributions.
+// Eq. 3-18 filter of one point: whether it is in id_all, and its residual.
+__device__ __forceinline__ bool point_residual(const FwdArgs &a, bool valid, float t, float ps, float &e) {
+    const bool m0 = (a.tau1 < t) && (t < a.tau2);
+    const bool m1 = (t <= a.tau1) && (ps > a.tau1);
+    const bool m2 = (t >= a.tau2) && (ps < a.tau2);
+    const bool mk = valid && (m0 || m1 || m2);
+    e = mk ? __fsub_rn(ps, t) : 0.f;
+    return mk;
+}
+
+// The outputs of one point; returns its residual and loss contributions.
 __device__ __forceinline__ float point_out(const FwdArgs &a, int64_t i, bool valid, float t, float ps, uint32_t np,
                                            float &l2, float &mx, uint32_t &cnt, uint32_t &pairs) {
     l2 = 0.f;
@@ -288,11 +298,8 @@ __device__ __forceinline__ float point_out(const FwdArgs &a, int64_t i, bool val
     cnt = 0u;
     pairs = 0u;
     if (!valid) return 0.f;
-    const bool m0 = (a.tau1 < t) && (t < a.tau2);
-    const bool m1 = (t <= a.tau1) && (ps > a.tau1);
-    const bool m2 = (t >= a.tau2) && (ps < a.tau2);
-    const bool mk = m0 || m1 || m2;
-    const float e = mk ? __fsub_rn(ps, t) : 0.f;
+    float e;
+    const bool mk = point_residual(a, valid, t, ps, e);
     a.psi[i] = ps;
     a.err[i] = e;
     a.mask[i] = (uint8_t)mk;
@@ -863,50 +870,63 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     // slot 0 or 32
     //
     // Shared memory is kept small: the L1 cache that serves the kernel-record
-    // gathers gets what the blocks leave of the SM's unified 256 KB.  The
-    // rings are idle during the adjoint, so the nz points live in warp 0's
-    // first ring and each warp's adjoint queue in its second.
+    // gathers gets what the blocks leave of the SM's unified 256 KB.  A warp's
+    // rings are idle during the adjoint, so the nz points live in its first
+    // ring and its adjoint queue in the second.
     constexpr int NT = G > 1 ? 2 : kMostTiles;  // tiles of an item (the points of a lane)
     constexpr int GR = G > 1 ? G : 1;    // the cross-warp sums exist only for G > 1
     constexpr int RL = G > 1 ? 32 : 1;
     constexpr int kTouchW = G > 1 ? kTouch / 2 : kTouch;  // kernels remembered per warp
     __shared__ __align__(16) float ringP[G][(kQueue / 2) * kPairFloats];
     __shared__ __align__(16) float ringF[G][(kQueue / 2) * kPairFloats];
-    __shared__ float2 red_psi[GR][RL];
-    __shared__ uint2 red_n[GR][RL];
-    __shared__ uint32_t red_cost[G];
-    __shared__ uint4 s_rec;
-    // fused adjoint: the item's nz points (tile 0 at 0, tile 1 at 32), their
-    // counts and boxes, and the kernels each warp found reaching the item
-    __shared__ int s_nc[2];
-    __shared__ float4 s_box[2][2];
+    // what the warps of a block exchange, of the current and of the last item
+    __shared__ float2 red_psi[2][GR][RL];
+    __shared__ uint2 red_n[2][GR][RL];
+    __shared__ uint32_t red_cost[2][GR];
+    __shared__ uint4 s_rec[2];
+    // fused adjoint: the kernels each warp found reaching the item
     __shared__ uint32_t touch[ADJ ? G : 1][ADJ ? kTouchW : 1];
     // batch: the arguments of the current item's field
     __shared__ __align__(16) unsigned char s_args[BATCH ? sizeof(FwdArgs) : 16];
-    __shared__ uint32_t s_field;
+    __shared__ uint32_t s_field[2];
     static_assert(sizeof(NzPoints) <= sizeof(ringP[0]) && kQueue * 4 <= (int)sizeof(ringF[0]), "ring aliases");
-    NzPoints &nzs = *reinterpret_cast<NzPoints *>(ringP[0]);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    NzPoints &nzs = *reinterpret_cast<NzPoints *>(ringP[warp]);
     uint32_t *adjq = reinterpret_cast<uint32_t *>(ringF[warp]);
     if (threadIdx.x == 0) {
         if (BATCH) {
             uint32_t f;
-            s_rec = resolve_batch(b, atomicAdd(b.next, 1u), f);
-            s_field = f;
+            s_rec[0] = resolve_batch(b, atomicAdd(b.next, 1u), f);
+            s_field[0] = f;
         } else {
-            s_rec = resolve(a1, atomicAdd(a1.item_next, 1u));
+            s_rec[0] = resolve(a1, atomicAdd(a1.item_next, 1u));
         }
     }
     __syncthreads();
-    uint4 rec = s_rec;  // the item's record; x = ~0 when done
-    uint32_t field = BATCH ? s_field : 0u, loaded = ~0u;
+    uint4 rec = s_rec[0];  // the item's record; x = ~0 when done
+    uint32_t field = BATCH ? s_field[0] : 0u, loaded = ~0u;
     uint32_t mean = BATCH ? 0u : a1.sched[0];
     const FwdArgs &a = BATCH ? *reinterpret_cast<const FwdArgs *>(s_args) : a1;
+    // several warps: buffer of the current item, and the last item's record,
+    // whose cost is noted once its warps have met again
+    int par = 0;
+    uint4 done = make_uint4(~0u, 0u, 0u, 0u);
+    auto note_done = [&]() {
+        if (G > 1 && threadIdx.x == 0 && done.x != ~0u) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int q = 0; q < GR; ++q) c += red_cost[par ^ 1][q];
+            note_cost(a, mean, done, c);
+        }
+        done.x = ~0u;
+    };
     while (rec.x != ~0u) {
         if (BATCH && field != loaded) {
             // the block's threads copy the field's arguments (block-uniform
             // branch: every thread holds the same record and field)
             if (G == 1) __syncwarp(); else __syncthreads();
+            if (loaded != ~0u) note_done();  // with the arguments of its own field
+            if (G > 1) __syncthreads();
             const uint32_t *src = reinterpret_cast<const uint32_t *>(b.args + field);
             uint32_t *dst = reinterpret_cast<uint32_t *>(s_args);
             for (int k = threadIdx.x; k < (int)(sizeof(FwdArgs) / 4); k += blockDim.x) dst[k] = src[k];
@@ -922,15 +942,24 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
         f2 acc[NT];
         uint32_t n[NT], cost;
         int ntouch = 0;
+        // the targets, for the residuals after the sums: loaded early where
+        // registers allow (with one warp per item, or without the adjoint, that
+        // cost 1.6 % and 3 %)
+        constexpr bool kEarly = G > 1 && ADJ;
+        float tv[NT];
+        auto targets = [&]() {
+#pragma unroll
+            for (int p = 0; p < NT; ++p) tv[p] = lane + p * kTile < it.np ? a.t[it.i0 + lane + p * kTile] : 0.f;
+        };
+        if (kEarly) targets();
         forward_share<G, ADJ>(a, it, warp, ringP[warp], ringF[warp], lane, acc, n, cost, touch[ADJ ? warp : 0], kTouchW,
                               ntouch);
+        if (!kEarly) targets();
         uint4 rn = make_uint4(~0u, 0u, 0u, 0u);
         if (threadIdx.x == 0) rn = BATCH ? resolve_batch(b, knext, fnext) : resolve(a, knext);
         if constexpr (G == 1) {
             // one warp: finish the tiles directly
-            float tv[NT], ev[NT];
-#pragma unroll
-            for (int p = 0; p < NT; ++p) tv[p] = lane + p * kTile < it.np ? a.t[it.i0 + lane + p * kTile] : 0.f;
+            float ev[NT];
             ff l2 = {0.f, 0.f};
             float mx = 0.f;
             uint32_t cnt = 0u, pr = 0u, pb = 0u, ebits = 0u;
@@ -983,90 +1012,86 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             if (BATCH) field = __shfl_sync(0xffffffffu, fnext, 0);
             continue;
         } else {
-        {
-            float l0, h0, l1, h1;
-            f2_unpack(acc[0], l0, h0);
-            f2_unpack(acc[1], l1, h1);
-            red_psi[warp][lane] = make_float2(l0 + h0, l1 + h1);
-            red_n[warp][lane] = make_uint2(n[0], n[1]);
-            if (lane == 0) red_cost[warp] = cost;
-        }
-        __syncthreads();
-        // warp 0 finishes the first tile, warp 1 the second (if any)
-        if (warp < it.ntl) {
-            float ps = 0.f;
-            uint32_t np = 0;
-#pragma unroll
-            for (int q = 0; q < G; ++q) {
-                const float2 v = red_psi[q][lane];
-                const uint2 c = red_n[q][lane];
-                ps += warp ? v.y : v.x;
-                np += warp ? c.y : c.x;
+            // the only barrier of an item: the warps' sums, the next record and
+            // the last item's costs meet.  Every warp then forms the residuals
+            // of both tiles and its own nz points, so none waits for another's;
+            // warps 0 and 1 also write a tile each.  (With the nz points made by
+            // those two for all there were four barriers, a fifth of the warps'
+            // time for 64^3 + 32^3 points.)  A buffer is written again two
+            // items later, past the barrier that follows its last reader.
+            {
+                float l0, h0, l1, h1;
+                f2_unpack(acc[0], l0, h0);
+                f2_unpack(acc[1], l1, h1);
+                red_psi[par][warp][lane] = make_float2(l0 + h0, l1 + h1);
+                red_n[par][warp][lane] = make_uint2(n[0], n[1]);
             }
-            float l2, mx;
-            uint32_t cnt, pr;
-            const int64_t i = it.i0 + lane + warp * kTile;
-            const bool v = lane + warp * kTile < it.np;
-            const float e = point_out(a, i, v, v ? a.t[i] : 0.f, ps, np, l2, mx, cnt, pr);
-            finish_tile(a, it.t0 + warp, l2, mx, cnt, pr, lane);
-            if (ADJ) {
-                const float emax = __uint_as_float(redux_max_u32(__float_as_uint(fabsf(e))));
-                // adjoint pairs: every support pair of a point with E != 0
-                const uint32_t pb = redux_add(e != 0.f ? np : 0u);
-                if (lane == 0 && pb) atomicAdd(a.adj_pairs, (unsigned long long)pb);
+            if (threadIdx.x == 0) {
+                s_rec[par] = rn;
+                if (BATCH) s_field[par] = fnext;
+            }
+            __syncthreads();
+            note_done();
+            float ev[2];
+            uint32_t ebits = 0u, pb = 0u;
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                float ps = 0.f;
+                uint32_t np = 0;
+#pragma unroll
+                for (int q = 0; q < G; ++q) {
+                    const float2 v = red_psi[par][q][lane];
+                    const uint2 c = red_n[par][q][lane];
+                    ps += t ? v.y : v.x;
+                    np += t ? c.y : c.x;
+                }
+                const bool v = lane + t * kTile < it.np;
+                if (warp == t && t < it.ntl) {
+                    float l2, mx;
+                    uint32_t cnt, pr;
+                    ev[t] = point_out(a, it.i0 + lane + t * kTile, v, tv[t], ps, np, l2, mx, cnt, pr);
+                    finish_tile(a, it.t0 + t, l2, mx, cnt, pr, lane);
+                    // adjoint pairs: every support pair of a point with E != 0
+                    pb = ev[t] != 0.f ? np : 0u;
+                } else {
+                    point_residual(a, v, tv[t], ps, ev[t]);
+                }
+                ebits = max(ebits, __float_as_uint(fabsf(ev[t])));
+            }
+            if (ADJ) ebits = redux_max_u32(ebits);
+            if (ADJ && ebits != 0u) {
+                if (warp < 2) {
+                    pb = redux_add(pb);
+                    if (lane == 0 && pb) atomicAdd(a.adj_pairs, (unsigned long long)pb);
+                }
                 float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
                 float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
-                const int64_t iv = v ? i : it.i0;
-                const float x = a.x[iv], y = a.y[iv], z = a.z[iv];
-                const int nc = nz_tile(nzs, kTile * warp, e != 0.f, x, y, z, e, lane);
-                nz_grow(lo, hi, e != 0.f, x, y, z);
+                int nc = 0;
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int64_t i = it.i0 + (lane + t * kTile < it.np ? lane + t * kTile : 0);
+                    const float x = a.x[i], y = a.y[i], z = a.z[i];
+                    nz_grow(lo, hi, ev[t] != 0.f, x, y, z);
+                    nc += nz_tile(nzs, nc, ev[t] != 0.f, x, y, z, ev[t], lane);
+                }
                 nz_box(lo, hi);
                 __syncwarp();
-                if ((nc & 1) && lane == 0) nz_pad(nzs, kTile * warp + nc);
-                if (lane == 0) {
-                    s_nc[warp] = nc;
-                    lo.w = emax;
-                    s_box[warp][0] = lo;
-                    s_box[warp][1] = hi;
-                    if (warp == 0 && it.ntl < 2) s_nc[1] = 0;
-                }
+                if ((nc & 1) && lane == 0) nz_pad(nzs, nc);
+                __syncwarp();
+                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, (uint32_t)nc, nc, lo, hi, touch[ADJ ? warp : 0], ntouch,
+                                            kTouchW, __uint_as_float(ebits), adjq, lane, cost);
+                __syncwarp();
             }
-            if (warp == 0 && lane == 0) {
-                if (!ADJ) {
-                    uint32_t c = 0;
-#pragma unroll
-                    for (int q = 0; q < G; ++q) c += red_cost[q];
-                    note_cost(a, mean, rec, c);
-                }
-                s_rec = rn;
-                if (BATCH) s_field = fnext;
-            }
+            if (lane == 0) red_cost[par][warp] = cost;
+            done = rec;
+            rec = s_rec[par];
+            if (BATCH) field = s_field[par];
+            par ^= 1;
         }
-        if (ADJ) {
-            __syncthreads();
-            const int nc0 = s_nc[0], nc1 = s_nc[1];
-            if (nc0 + nc1 > 0) {
-                const float4 lo = nc1 ? (nc0 ? box_min(s_box[0][0], s_box[1][0]) : s_box[1][0]) : s_box[0][0];
-                const float4 hi = nc1 ? (nc0 ? box_max(s_box[0][1], s_box[1][1]) : s_box[1][1]) : s_box[0][1];
-                uint32_t c = 0;
-                const float emax = __uint_as_float(
-                    max(nc0 ? __float_as_uint(s_box[0][0].w) : 0u, nc1 ? __float_as_uint(s_box[1][0].w) : 0u));
-                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, (uint32_t)(nc0 | nc1 << 8), nc0 + nc1, lo, hi, touch[warp],
-                                            ntouch, kTouchW, emax, adjq, lane, c);
-                if (lane == 0) red_cost[warp] += c;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                uint32_t c = 0;
-#pragma unroll
-                for (int q = 0; q < G; ++q) c += red_cost[q];
-                note_cost(a, mean, rec, c);
-            }
-        }
+    }
+    if (G > 1) {
         __syncthreads();
-        rec = s_rec;
-        if (BATCH) field = s_field;
-        }
+        note_done();
     }
     // the last block out prepares the next launch: every block has made its
     // last claim and recorded its costs before it counts itself out
