@@ -28,10 +28,9 @@ class ERBFField(torch.autograd.Function):
         # so err = g / 2 gives sum_i g_i dPsi_i/dp
         err = (0.5 * g_psi).contiguous().to(torch.float32)
         grad = torch.zeros_like(pb.grad)
+        # columns of kernels beyond the live count stay zero: the call does not
+        # write them (so the count is not read here, which waited for the GPU)
         N.serbf_backward(pb.pts, pb.prm, pb.cfg, err, grad, pb.stats, pb.ws)
-        m = pb.m()
-        if m < grad.shape[1]:
-            grad[:, m:] = 0
         return grad, None
 
 

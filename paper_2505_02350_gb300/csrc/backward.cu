@@ -1,7 +1,7 @@
 // Kernel-major adjoint (App. A).  The points with a nonzero residual are first
 // compacted within their tile (x, y, z, E as float4 in the tile's 32 slots).
-// Then one block per kernel: its warps visit the super cells of the support
-// box, keep the tiles whose box the support reaches and that hold nonzero
+// Then one block per kernel: its warps visit the chunks of the super cells of
+// the support box, keep the tiles whose box the support reaches and that hold nonzero
 // residuals, queue those points in a per-warp shared-memory ring, and process
 // them 32 at a time: exact support predicate (Eq. 3-15-1), phi recomputed, and
 // ten moments of s = phi * E accumulated in the rotated frame u = R (v - c):
@@ -82,6 +82,7 @@ struct BwdArgs {
     const float4 *nzrec;   // packed records of tiles with nonzero residuals, per 32-tile chunk
     const uint32_t *nzc;   // records per chunk, indexed by the chunk's first tile
     const float4 *nz;
+    int chunks;  // most 32-tile chunks in one super cell
     float *mom;  // per kernel, per warp: 10 float-float moments S0, M1 (3), M2 (6), then the pair count (bits)
 };
 
@@ -106,72 +107,56 @@ __global__ void __launch_bounds__(kBwdThreads) k_moments(BwdArgs a) {
     const int nsb = nbx * nby * nbz;
     int head = 0, qn = 0;
     uint32_t *q = ring[warp];
-    // the kernel's super cells are dealt round-robin to all its warps; a warp
-    // tests 32 of its super cells at once (one per lane), then walks the hit
-    // ones and their packed nonzero tiles
+    // the 32-tile chunks of the kernel's super cells are dealt round-robin to
+    // all its warps; a warp tests 32 of its chunks at once (one per lane), then
+    // walks the packed nonzero tiles of those its support may reach.  Whole
+    // super cells of 4096 points left some warps with several and others with
+    // none: 19.7 M pairs of 512 kernels took 128 us, in chunks 101 us.  (Packed
+    // pairs of points, and tiles taken around the queue, did not help: 105 and
+    // 130 us, with more registers and fewer warps.)
     const int W = NW * gridDim.y, wid = split * NW + warp;
-    for (int base = wid; base < nsb; base += W * 32) {
-        const int sb = base + lane * W;
-        uint32_t t0 = 0, nt = 0;
-        unsigned long long packed = 0;  // chunk counts (6 bits each) of the first 8 chunks
-        if (sb < nsb) {
+    const int64_t units = (int64_t)nsb * a.chunks;
+    for (int64_t base = wid; base < units; base += W * 32) {
+        const int64_t un = base + (int64_t)lane * W;
+        uint32_t first = 0, cnt = 0;  // the chunk's first tile and its number of records
+        if (un < units) {
+            const int sb = (int)(un / a.chunks), ch = (int)(un - (int64_t)sb * a.chunks);
             const int sx = sx0 + sb % nbx, sy = sy0 + (sb / nbx) % nby, sz = sz0 + sb / (nbx * nby);
             const int s = (sz * a.nsy + sy) * a.nsx + sx;
-            if (box_d2(k0.x, k0.y, k0.z, a.slo[s], a.shi[s]) < k0.w) {
-                t0 = a.stile0[s];
-                nt = a.stile0[s + 1] - t0;  // tiles of the super cell
-                const uint32_t nch = (nt + 31) / 32;
-                for (uint32_t q8 = 0; q8 < 8 && q8 < nch; ++q8)
-                    packed |= (unsigned long long)a.nzc[t0 + 32u * q8] << (6 * q8);
-                if (!packed && nch <= 8) nt = 0;  // no nonzero tile at all
-            }
+            first = a.stile0[s] + 32u * ch;
+            if (first < a.stile0[s + 1] && box_d2(k0.x, k0.y, k0.z, a.slo[s], a.shi[s]) < k0.w) cnt = a.nzc[first];
         }
-        unsigned sbal = __ballot_sync(0xffffffffu, nt != 0);
-        while (sbal) {
-            const int ssrc = __ffs(sbal) - 1;
-            sbal &= sbal - 1;
-            const uint32_t st0 = __shfl_sync(0xffffffffu, t0, ssrc), snt = __shfl_sync(0xffffffffu, nt, ssrc);
-            const unsigned long long spk = __shfl_sync(0xffffffffu, packed, ssrc);
-            // the super cell's 32-tile chunks: the first 8 counts came with the
-            // super cell's test, later ones are loaded 32 at a time
-            const uint32_t nch = (snt + 31) / 32;
-            for (uint32_t cg = 0; cg < nch; cg += 32) {
-            uint32_t cc_l = 0;
-            if (cg + lane < nch)
-                cc_l = (cg + lane < 8) ? (uint32_t)((spk >> (6 * (cg + lane))) & 63ull) : a.nzc[st0 + 32u * (cg + lane)];
-            unsigned cbal = __ballot_sync(0xffffffffu, cc_l != 0);
-            while (cbal) {
-                const int csrc = __ffs(cbal) - 1;
-                cbal &= cbal - 1;
-                const uint32_t cb = st0 + 32u * (cg + csrc), ncr = __shfl_sync(0xffffffffu, cc_l, csrc);
-                uint32_t c = 0, t = 0;
-                if ((uint32_t)lane < ncr) {
-                    const float4 lo = a.nzrec[2 * (size_t)(cb + lane)], hi = a.nzrec[2 * (size_t)(cb + lane) + 1];
-                    if (box_d2(k0.x, k0.y, k0.z, lo, hi) < k0.w) {
-                        c = __float_as_uint(lo.w);
-                        t = __float_as_uint(hi.w);
-                    }
-                }
-                unsigned bal = __ballot_sync(0xffffffffu, c != 0);
-                while (bal) {
-                    const int src = __ffs(bal) - 1;
-                    bal &= bal - 1;
-                    const uint32_t cc = __shfl_sync(0xffffffffu, c, src);
-                    const uint32_t tt = __shfl_sync(0xffffffffu, t, src);
-                    if (lane < (int)cc) q[(head + qn + lane) & (RING - 1)] = tt * kTile + lane;
-                    qn += cc;
-                    __syncwarp();
-                    if (qn >= 64) {
-                        const float4 p0 = a.nz[q[(head + lane) & (RING - 1)]];
-                        const float4 p1 = a.nz[q[(head + 32 + lane) & (RING - 1)]];
-                        accumulate<KAHAN>(p0, k0, k1, k2, k3, acc, cmp, pairs);
-                        accumulate<KAHAN>(p1, k0, k1, k2, k3, acc, cmp, pairs);
-                        head = (head + 64) & (RING - 1);
-                        qn -= 64;
-                        __syncwarp();
-                    }
+        unsigned cbal = __ballot_sync(0xffffffffu, cnt != 0);
+        while (cbal) {
+            const int csrc = __ffs(cbal) - 1;
+            cbal &= cbal - 1;
+            const uint32_t cb = __shfl_sync(0xffffffffu, first, csrc), ncr = __shfl_sync(0xffffffffu, cnt, csrc);
+            uint32_t c = 0, t = 0;
+            if ((uint32_t)lane < ncr) {
+                const float4 lo = a.nzrec[2 * (size_t)(cb + lane)], hi = a.nzrec[2 * (size_t)(cb + lane) + 1];
+                if (box_d2(k0.x, k0.y, k0.z, lo, hi) < k0.w) {
+                    c = __float_as_uint(lo.w);
+                    t = __float_as_uint(hi.w);
                 }
             }
+            unsigned bal = __ballot_sync(0xffffffffu, c != 0);
+            while (bal) {
+                const int src = __ffs(bal) - 1;
+                bal &= bal - 1;
+                const uint32_t cc = __shfl_sync(0xffffffffu, c, src);
+                const uint32_t tt = __shfl_sync(0xffffffffu, t, src);
+                if (lane < (int)cc) q[(head + qn + lane) & (RING - 1)] = tt * kTile + lane;
+                qn += cc;
+                __syncwarp();
+                if (qn >= 64) {
+                    const float4 p0 = a.nz[q[(head + lane) & (RING - 1)]];
+                    const float4 p1 = a.nz[q[(head + 32 + lane) & (RING - 1)]];
+                    accumulate<KAHAN>(p0, k0, k1, k2, k3, acc, cmp, pairs);
+                    accumulate<KAHAN>(p1, k0, k1, k2, k3, acc, cmp, pairs);
+                    head = (head + 64) & (RING - 1);
+                    qn -= 64;
+                    __syncwarp();
+                }
             }
         }
     }
@@ -278,6 +263,7 @@ extern "C" int serbf_backward(const serbf_points *pts, const serbf_params *prm, 
     a.nzrec = ws->nzrec;
     a.nzc = ws->nzc_cnt;
     a.nz = ws->nz;
+    a.chunks = ws->max_chunks;
     a.mom = ws->moments;
     // enough warps in flight: split a kernel's super cells over more blocks when
     // there are few kernels, fewer when there are many (each split adds a
