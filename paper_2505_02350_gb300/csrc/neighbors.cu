@@ -55,9 +55,12 @@ __device__ __forceinline__ void prep_kernels(const float *p, int cap, int m, flo
     }
 }
 
+constexpr int64_t kOrderDirect = 64 * kOrderChunk;  // items up to which one launch makes the order
+
 // The forward's heavy-first order for its next launch: a stable sort of the
-// items by the cost class the last forward filed, descending, in two
-// launches on the workspace's side stream (next to the neighbour rebuild).
+// items by the cost class the last forward filed, descending, in one launch
+// (up to kOrderDirect items) or two on the workspace's side stream (next to
+// the neighbour rebuild).
 // k_class_count: block b counts the classes of items [b kOrderChunk,
 // (b + 1) kOrderChunk).  k_order_items: block b places the same items; a
 // class starts after all heavier classes and after this class in earlier
@@ -86,6 +89,7 @@ __global__ void __launch_bounds__(kOrderChunk) k_class_count(const uint8_t *item
     class_count_body(item_class, nitems, hist, blockIdx.x);
 }
 
+// hist == nullptr: the block counts the classes of all items itself.
 __device__ __forceinline__ void order_items_body(const uint8_t *item_class, const uint32_t *hist,
                                                  const uint4 *item_rec, uint4 *order_rec, int64_t nitems, int bx) {
     constexpr int NW = kOrderChunk / 32;
@@ -94,8 +98,32 @@ __device__ __forceinline__ void order_items_body(const uint8_t *item_class, cons
     __shared__ uint32_t s_wcnt[NW][kCostClasses];  // per warp: class counts, then offsets
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nchunks = (int)((nitems + kOrderChunk - 1) / kOrderChunk), b = bx;
-    // class totals and this class's count in earlier chunks: warp c handles class c
-    if (warp < kCostClasses) {
+    if (!hist) {
+        if (threadIdx.x < kCostClasses) s_base[threadIdx.x] = s_tot[threadIdx.x] = 0u;
+        __syncthreads();
+        // four items at a time; eight 8-bit counters a thread (kOrderDirect
+        // items are 64 per thread)
+        unsigned long long tot = 0ull, before = 0ull;
+        for (int64_t i = 4 * (int64_t)threadIdx.x; i < nitems; i += 4 * kOrderChunk) {
+            const uint32_t w = *reinterpret_cast<const uint32_t *>(item_class + i);
+            unsigned long long c = 0ull;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i + k < nitems) c += 1ull << (((w >> (8 * k)) & 7u) * 8);
+            tot += c;
+            if (i < (int64_t)b * kOrderChunk) before += c;
+        }
+#pragma unroll
+        for (int c = 0; c < kCostClasses; ++c) {
+            const uint32_t t = __reduce_add_sync(0xffffffffu, (uint32_t)(tot >> (8 * c)) & 255u);
+            const uint32_t f = __reduce_add_sync(0xffffffffu, (uint32_t)(before >> (8 * c)) & 255u);
+            if (lane == 0 && t) {
+                atomicAdd(&s_tot[c], t);
+                atomicAdd(&s_base[c], f);
+            }
+        }
+    } else if (warp < kCostClasses) {
+        // class totals and this class's count in earlier chunks: warp c handles class c
         uint32_t tot = 0, before = 0;
         for (int q = lane; q < nchunks; q += 32) {
             const uint32_t v = hist[(size_t)q * kCostClasses + warp];
@@ -744,8 +772,12 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
         if (cudaEventRecord(ws->ev_fork, s) != cudaSuccess) return SERBF_ECUDA;
         if (cudaStreamWaitEvent(ws->aux, ws->ev_fork, 0) != cudaSuccess) return SERBF_ECUDA;
         const unsigned nchunks = (unsigned)((items.n + kOrderChunk - 1) / kOrderChunk);
-        k_class_count<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, items.n, ws->class_hist);
-        k_order_items<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, ws->class_hist, items.rec, items.order, items.n);
+        // few items: every block counts all classes itself, one launch less on
+        // the way to the forward
+        const bool direct = items.n <= kOrderDirect;
+        if (!direct) k_class_count<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, items.n, ws->class_hist);
+        k_order_items<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, direct ? nullptr : ws->class_hist, items.rec,
+                                                            items.order, items.n);
         SERBF_CHECK_LAUNCH();
         if (cudaEventRecord(ws->ev_join, ws->aux) != cudaSuccess) return SERBF_ECUDA;
     }
