@@ -15,7 +15,7 @@
 //
 // One block walking point by point took 100 ms for 23 k interior points and
 // 6457 centres (64^3, 15 us a centre, nearly all of it barriers and dependent
-// loads); ten rounds take under 1 ms.
+// loads); ten rounds take 0.9 ms, two thirds of it in k_settle's one block.
 #include <math.h>
 
 #include "common.cuh"
@@ -69,7 +69,7 @@ static_assert(kBatch * 16 <= 256 * (kDirectBlocks + 1) * 4, "the fresh centres f
 
 struct WalkArgs {
     Walk *w;
-    const float4 *pts;
+    float4 *pts;            // interior points in order; settled places take the centres
     const uint32_t *order;  // binned indices of the interior points, |S| descending
     uint8_t *removed;       // per sorted position
     uint32_t *centres;      // binned indices of the centres, in selection order
@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kBatch) k_settle(WalkArgs a) {
     if (left) {
         if (before + o < (uint32_t)a.cap) a.centres[before + o] = a.order[s_pos[tid]];
         a.fresh[o] = p;
+        a.pts[before + o] = p;  // at or before this point's own place, which is settled
     }
     if (tid == 0) {
         a.w->next = s_next;
@@ -154,50 +155,68 @@ __global__ void __launch_bounds__(kBatch) k_settle(WalkArgs a) {
     }
 }
 
-// The points from the next position on that a new centre covers are removed.
+// The points from the next position on that a new centre covers are removed:
+// blocks (x, y) test their points against the y-th kCoverPart of the new
+// centres (all of them by one thread were a chain of up to 1024 tests, 26 us
+// a round).
+constexpr int kCoverPart = 128;
 __global__ void __launch_bounds__(256) k_cover(WalkArgs a) {
     pdl_wait();
     pdl_trigger();
-    __shared__ float4 c[256];
-    const uint32_t nin = a.w->count, k = a.w->fresh, next = a.w->next;
+    __shared__ float4 c[kCoverPart];
+    const uint32_t nin = a.w->count, fresh = a.w->fresh, next = a.w->next, first = blockIdx.y * kCoverPart;
+    if (first >= fresh) return;
+    const int k = (int)min((uint32_t)kCoverPart, fresh - first);
+    if (threadIdx.x < k) c[threadIdx.x] = a.fresh[first + threadIdx.x];
+    __syncthreads();
     for (uint64_t q0 = (uint64_t)next + blockIdx.x * 256ull; q0 < nin; q0 += gridDim.x * 256ull) {
         const uint64_t q = q0 + threadIdx.x;
         bool here = q < nin && !a.removed[q];
         const float4 p = here ? a.pts[q] : make_float4(0.f, 0.f, 0.f, 0.f);
         bool gone = false;
-        for (uint32_t c0 = 0; c0 < k; c0 += 256) {
-            __syncthreads();
-            if (c0 + threadIdx.x < k) c[threadIdx.x] = a.fresh[c0 + threadIdx.x];
-            __syncthreads();
-            const int m = (int)min(256u, k - c0);
-            if (here && !gone)
-                for (int i = 0; i < m && !gone; ++i) gone = covered(p, c[i]);
-        }
+        if (here)
+            for (int i = 0; i < k && !gone; ++i) gone = covered(p, c[i]);
         if (gone) a.removed[q] = 1;
     }
 }
 
-// Eq. 3-12 for the selected centres (a warp per centre): dhat = distance to
+// Eq. 3-12 for the selected centres (a warp per kNearest centres, which share
+// the coordinates that it reads): dhat = distance to
 // the nearest other centre (a single centre: twice its radius), then
 // d = 2 sqrt(-ln(gamma / w^2)) / dhat on all axes, angles 0, w = t.
+constexpr int kNearest = 4;
 __global__ void k_init_params(const float *x, const float *y, const float *z, const float *t, const float *S,
-                              const uint32_t *centres, const uint32_t *ncentres, int32_t cap, float gamma, float *p,
-                              int32_t *m_dev) {
+                              const uint32_t *centres, const float4 *at, const uint32_t *ncentres, int32_t cap,
+                              float gamma, float *p, int32_t *m_dev) {
     const int M = (int)min(*ncentres, (uint32_t)cap);
-    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (j == 0 && lane == 0) *m_dev = M;
-    if (j >= M) return;
+    const int j0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kNearest, lane = threadIdx.x & 31;
+    if (j0 == 0 && lane == 0) *m_dev = M;
+    if (j0 >= M) return;
+    float4 c[kNearest];
+    float near[kNearest];
+#pragma unroll
+    for (int k = 0; k < kNearest; ++k) {
+        c[k] = at[min(j0 + k, M - 1)];
+        near[k] = INFINITY;
+    }
+    for (int i = lane; i < M; i += 32) {
+        const float4 q = at[i];
+#pragma unroll
+        for (int k = 0; k < kNearest; ++k) {
+            const float dx = q.x - c[k].x, dy = q.y - c[k].y, dz = q.z - c[k].z;
+            const float d2 = dx * dx + dy * dy + dz * dz;
+            if (i != j0 + k) near[k] = fminf(near[k], d2);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kNearest; ++k) near[k] = -warp_max(-near[k]);
+    const int j = j0 + lane;
+    if (lane >= kNearest || j >= M) return;
+    float best = near[0];
+#pragma unroll
+    for (int k = 1; k < kNearest; ++k) best = lane == k ? near[k] : best;
     const uint32_t cj = centres[j];
     const float px = x[cj], py = y[cj], pz = z[cj];
-    float best = INFINITY;
-    for (int i = lane; i < M; i += 32) {
-        if (i == j) continue;
-        const uint32_t ci = centres[i];
-        const float dx = x[ci] - px, dy = y[ci] - py, dz = z[ci] - pz;
-        best = fminf(best, dx * dx + dy * dy + dz * dz);
-    }
-    best = -warp_max(-best);
-    if (lane != 0) return;
     const float dhat = M > 1 ? sqrtf(best) : 2.f * fabsf(S[cj]);
     const float w = t[cj];
     const float d = 2.f * sqrtf(-logf(gamma / (w * w))) / dhat;
@@ -245,15 +264,15 @@ extern "C" int serbf_init_kernels(const serbf_points *pts, const float *S_raw, d
             // ends: every round settles at least one point
             for (int q = 0; q < kRounds; ++q) {
                 launch_pdl(k_settle, dim3(1), dim3(kBatch), 0, s, a);
-                launch_pdl(k_cover, dim3((unsigned)(cover < most ? cover : most)), dim3(256), 0, s, a);
+                launch_pdl(k_cover, dim3((unsigned)(cover < most ? cover : most), kBatch / kCoverPart), dim3(256), 0, s, a);
             }
             SERBF_CHECK_LAUNCH();
             if (cudaMemcpyAsync(&now, w, sizeof(Walk), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SERBF_ECUDA;
             if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
         } while (now.next < now.count);
         found = now.centres;
-        k_init_params<<<(unsigned)((prm->cap + 7) / 8), 256, 0, s>>>(pts->x, pts->y, pts->z, pts->t, S_raw, vt, &w->centres,
-                                                                     prm->cap, (float)gamma, prm->p, prm->m);
+        k_init_params<<<(unsigned)((prm->cap + 8 * kNearest - 1) / (8 * kNearest)), 256, 0, s>>>(
+            pts->x, pts->y, pts->z, pts->t, S_raw, vt, ws->nz, &w->centres, prm->cap, (float)gamma, prm->p, prm->m);
     } else {
         if (cudaMemsetAsync(prm->m, 0, sizeof(int32_t), s) != cudaSuccess) return SERBF_ECUDA;
     }
