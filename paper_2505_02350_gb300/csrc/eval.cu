@@ -132,20 +132,52 @@ __device__ __forceinline__ long long block_iscan_i64(long long v, long long *tmp
     return v;
 }
 
-// The tile sums of element values get(i), i < n, by one block per tile.
+// The tile sums of element values get(i), i < n, by one block per tile: a
+// thread's values of all rounds first, their warp scans, then one scan of the
+// rounds' and warps' totals (two barriers a tile).
 template <typename F>
 __device__ __forceinline__ void scan_tile(int64_t n, int64_t *a, F get) {
-    __shared__ long long tmp[32];
+    constexpr int NW = kScanThreads / 32, N = NW * kScanPer;
+    static_assert(N % 32 == 0, "whole warps of totals");
+    __shared__ long long tot[N];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t base = blockIdx.x * (int64_t)kScanTile;
     if (blockIdx.x == 0 && threadIdx.x == 0) a[0] = 0;
-    long long carry = 0;
-#pragma unroll 1
+    long long v[kScanPer];
+#pragma unroll
     for (int r = 0; r < kScanPer; ++r) {
         const int64_t i = base + r * kScanThreads + threadIdx.x;
-        long long total;
-        const long long v = block_iscan_i64(i < n ? get(i) : 0ll, tmp, &total);
-        if (i < n) a[i + 1] = carry + v;
-        carry += total;
+        v[r] = i < n ? get(i) : 0ll;
+    }
+#pragma unroll
+    for (int r = 0; r < kScanPer; ++r) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long t = __shfl_up_sync(0xffffffffu, v[r], o);
+            if (lane >= o) v[r] += t;
+        }
+        if (lane == 31) tot[r * NW + warp] = v[r];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        long long carry = 0;
+        for (int q = 0; q < N; q += 32) {
+            const long long own = tot[q + lane];
+            long long inc = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            tot[q + lane] = carry + inc - own;
+            carry += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kScanPer; ++r) {
+        const int64_t i = base + r * kScanThreads + threadIdx.x;
+        if (i < n) a[i + 1] = tot[r * NW + warp] + v[r];
     }
 }
 
@@ -180,24 +212,41 @@ __global__ void __launch_bounds__(kScanThreads) k_mt_count(const float *f, Grid3
     });
 }
 
-__global__ void __launch_bounds__(256) k_mt_write(const float *f, Grid3 g, float iso, int64_t ncubes,
-                                                  const int64_t *off, float *tri) {
-    const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c >= ncubes) return;
-    const Cube q = cube_at(f, g, c);
-    const int in = inside(q, iso);
-    if (in == 0 || in == 255) return;
-    float *t = tri + 9 * tile_prefix(off, c);
-#pragma unroll 1
-    for (int k = 0; k < 6; ++k) {
-        const int m = tet_mask(in, k), nin = __popc(m);
+// A block first lists its crossed cubes (about one in thirty of a surface's
+// grid), then a thread takes one tetrahedron of one listed cube, so that warps
+// are full of them; cubes taken where they lie left a few lanes of each warp
+// working (61 us for 2.1 M cubes, now 31).
+constexpr int kMtThreads = 256;
+__global__ void __launch_bounds__(kMtThreads) k_mt_write(const float *f, Grid3 g, float iso, int64_t ncubes,
+                                                         const int64_t *off, float *tri) {
+    __shared__ uint16_t s_cube[kMtThreads];
+    __shared__ uint8_t s_in[kMtThreads];
+    __shared__ uint32_t tmp[33];
+    const int64_t base = blockIdx.x * (int64_t)kMtThreads, mine = base + threadIdx.x;
+    int in = 0;
+    if (mine < ncubes) in = inside(cube_at(f, g, mine), iso);
+    const bool crossed = in != 0 && in != 255;
+    uint32_t n;
+    const uint32_t at = block_exscan(crossed, tmp, &n);
+    if (crossed) {
+        s_cube[at] = (uint16_t)threadIdx.x;
+        s_in[at] = (uint8_t)in;
+    }
+    __syncthreads();
+    for (uint32_t w = threadIdx.x; w < 6 * n; w += kMtThreads) {
+        const uint32_t a = w / 6, k = w - 6 * a;
+        const int all = s_in[a], m = tet_mask(all, k), nin = __popc(m);
         if (nin == 0 || nin == 4) continue;
+        const int64_t c = base + s_cube[a];
+        int64_t o = tile_prefix(off, c);
+        for (uint32_t b = 0; b < k; ++b) o += tris_of(tet_mask(all, b));
+        float *t = tri + 9 * o;
+        const Cube q = cube_at(f, g, c);
         const int *v = c_tets[k];
         if (nin != 2) {
             const int l = __ffs(nin == 1 ? m : ~m & 15) - 1;  // the lone vertex
 #pragma unroll
             for (int e = 0; e < 3; ++e) edge_point(q, g, v[l], v[e + (e >= l)], iso, t + 3 * e);
-            t += 9;
         } else {
             const int A = __ffs(m) - 1, B = 31 - __clz(m), C = __ffs(~m & 15) - 1, D = 31 - __clz(~m & 15);
             float ac[3], ad[3], bd[3], bc[3];
@@ -206,15 +255,14 @@ __global__ void __launch_bounds__(256) k_mt_write(const float *f, Grid3 g, float
             edge_point(q, g, v[B], v[D], iso, bd);
             edge_point(q, g, v[B], v[C], iso, bc);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                t[a] = ac[a];
-                t[3 + a] = ad[a];
-                t[6 + a] = bd[a];
-                t[9 + a] = ac[a];
-                t[12 + a] = bd[a];
-                t[15 + a] = bc[a];
+            for (int a3 = 0; a3 < 3; ++a3) {
+                t[a3] = ac[a3];
+                t[3 + a3] = ad[a3];
+                t[6 + a3] = bd[a3];
+                t[9 + a3] = ac[a3];
+                t[12 + a3] = bd[a3];
+                t[15 + a3] = bc[a3];
             }
-            t += 18;
         }
     }
 }
@@ -278,7 +326,7 @@ __global__ void k_sample(const float *tri, int64_t ntri, const int64_t *cum, con
 // node of the implied octree is a contiguous range of cells and of points; a
 // query descends nearest child first and leaves out nodes whose (rounded down)
 // distance is above the best.  All pairs took 10.5 ms for two sets of 10^5
-// points.  Smaller sets are streamed through shared memory.
+// points, this 0.25 ms with the grids' making.  Smaller sets are streamed through shared memory.
 constexpr int kNnThreads = 256;
 constexpr int64_t kNnMin = 1024;
 constexpr int kNnMaxLevels = 8;
@@ -485,10 +533,73 @@ __device__ __forceinline__ void nn_search(const NnSet &s, const NnFrame &f, floa
     }
 }
 
+// What a direction (points of P to set Q) needs: P's own grid, when it has
+// one, gives the order in which its points are taken.
+struct NnDir {
+    NnSet P, Q;
+    const float *nP, *nQ;
+    float *best;     // per point of P: squared distance to the nearest of Q
+    uint32_t *bi;    // and its index
+    double *part;    // three doubles per block of k_nn_sums
+};
+struct NnDirs {
+    NnDir d[2];
+};
+
+// Nearest points of both directions (blockIdx.y).  Points are taken in the
+// order of their own grid, so the lanes of a warp walk about the same nodes (in
+// the sampling order, 200 us a direction for 10^5 points each; now 155 for both).
+__global__ void __launch_bounds__(kNnThreads) k_nearest(NnDirs a) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float sq[kNnThreads * 3];
+    const NnDir &d = a.d[blockIdx.y];
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q - threadIdx.x >= d.P.n) return;
+    const bool live = q < d.P.n;
+    const int64_t i = live ? (d.P.levels >= 0 ? (int64_t)d.P.idx[q] : q) : 0;
+    const float px = d.P.p[3 * i], py = d.P.p[3 * i + 1], pz = d.P.p[3 * i + 2];
+    float best = INFINITY;
+    int64_t bi = 0;
+    if (d.Q.levels >= 0) {
+        if (live) nn_search(d.Q, nn_frame(d.Q), px, py, pz, best, bi);
+    } else {
+        for (int64_t j0 = 0; j0 < d.Q.n; j0 += kNnThreads) {
+            __syncthreads();
+            const int cnt = (int)min((int64_t)kNnThreads, d.Q.n - j0);
+            for (int k = threadIdx.x; k < 3 * cnt; k += kNnThreads) sq[k] = d.Q.p[3 * j0 + k];
+            __syncthreads();
+            for (int k = 0; k < cnt; ++k) {
+                const float d2 = nn_d2(px, py, pz, sq + 3 * k);
+                if (d2 < best) {
+                    best = d2;
+                    bi = j0 + k;
+                }
+            }
+        }
+    }
+    if (live) {
+        d.best[i] = best;
+        d.bi[i] = (uint32_t)bi;
+    }
+}
+
 // Largest distance, sum of distances and sum of |n_P . n_Q| of a block's
 // points, in a fixed order.
-__device__ __forceinline__ void nn_partial(double d, double c, double *out) {
+__global__ void __launch_bounds__(kNnThreads) k_nn_sums(NnDirs a) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double sm[3][32];
+    const NnDir &D = a.d[blockIdx.y];
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i - threadIdx.x >= D.P.n) return;
+    double d = 0.0, c = 0.0;
+    if (i < D.P.n) {
+        const float *p = D.nP + 3 * i, *q = D.nQ + 3 * (int64_t)D.bi[i];
+        d = __dsqrt_rn((double)D.best[i]);
+        c = fabs(__dadd_rn(__dadd_rn(__dmul_rn((double)p[0], (double)q[0]), __dmul_rn((double)p[1], (double)q[1])),
+                           __dmul_rn((double)p[2], (double)q[2])));
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double m = d;
     for (int o = 16; o > 0; o >>= 1) {
@@ -508,47 +619,10 @@ __device__ __forceinline__ void nn_partial(double d, double c, double *out) {
         d += sm[1][w];
         c += sm[2][w];
     }
+    double *out = D.part + 3 * (int64_t)blockIdx.x;
     out[0] = m;
     out[1] = d;
     out[2] = c;
-}
-
-// part: three doubles per block.
-__global__ void __launch_bounds__(kNnThreads) k_nearest(const float *P, const float *nP, int64_t np, const NnSet Q,
-                                                        const float *nQ, double *part) {
-    pdl_wait();
-    pdl_trigger();
-    __shared__ float sq[kNnThreads * 3];
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool live = i < np;
-    const float px = live ? P[3 * i] : 0.f, py = live ? P[3 * i + 1] : 0.f, pz = live ? P[3 * i + 2] : 0.f;
-    float best = INFINITY;
-    int64_t bi = 0;
-    if (Q.levels >= 0) {
-        if (live) nn_search(Q, nn_frame(Q), px, py, pz, best, bi);
-    } else {
-        for (int64_t j0 = 0; j0 < Q.n; j0 += kNnThreads) {
-            __syncthreads();
-            const int cnt = (int)min((int64_t)kNnThreads, Q.n - j0);
-            for (int k = threadIdx.x; k < 3 * cnt; k += kNnThreads) sq[k] = Q.p[3 * j0 + k];
-            __syncthreads();
-            for (int k = 0; k < cnt; ++k) {
-                const float d2 = nn_d2(px, py, pz, sq + 3 * k);
-                if (d2 < best) {
-                    best = d2;
-                    bi = j0 + k;
-                }
-            }
-        }
-    }
-    double dist = 0.0, cosv = 0.0;
-    if (live) {
-        dist = __dsqrt_rn((double)best);
-        cosv = fabs(__dadd_rn(__dadd_rn(__dmul_rn((double)nP[3 * i], (double)nQ[3 * bi]),
-                                        __dmul_rn((double)nP[3 * i + 1], (double)nQ[3 * bi + 1])),
-                              __dmul_rn((double)nP[3 * i + 2], (double)nQ[3 * bi + 2])));
-    }
-    nn_partial(dist, cosv, part + 3 * (int64_t)blockIdx.x);
 }
 
 // One block per direction: the blocks' partials into red[3 x direction ..].
@@ -636,7 +710,7 @@ extern "C" int serbf_marching_tets(const float *f, const int32_t dims[3], const 
     if (cudaStreamSynchronize(s) != cudaSuccess) return SERBF_ECUDA;
     *ntri = n;
     if (n > cap) return SERBF_ECAPACITY;
-    k_mt_write<<<(unsigned)((ncubes + 255) / 256), 256, 0, s>>>(f, g, iso, ncubes, scratch, tri);
+    k_mt_write<<<(unsigned)((ncubes + kMtThreads - 1) / kMtThreads), kMtThreads, 0, s>>>(f, g, iso, ncubes, scratch, tri);
     SERBF_CHECK_LAUNCH();
     return cudaStreamSynchronize(s) == cudaSuccess ? SERBF_OK : SERBF_ECUDA;
 }
@@ -664,20 +738,23 @@ extern "C" int serbf_surface_metrics(const float *A, const float *nA, int64_t na
     SERBF_TRACE();
     if (!A || !nA || !B || !nB || na < 1 || nb < 1 || !out || !scratch) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    // scratch (16 bytes per point and 48): the six results last; the blocks'
-    // partials (a set of one block writes its result in place), then per grid
-    // its box, cells and indices -- at most 24 / 256 + 2 + 4 bytes per point
-    double *red = scratch + 2 * (na + nb), *next = scratch;
-    const float *pts[2] = {A, B}, *nrm[2] = {nA, nB};
-    const int64_t n[2] = {na, nb};
+    // scratch (16 bytes per point and 48): the six results last; from the start
+    // 8 bytes per point for the nearest points, the blocks' partials (a set of
+    // one block writes its result in place), then per grid its box, cells and
+    // indices -- at most 8 + 24 / 256 + 2 + 4 bytes per point and 32
+    double *red = scratch + 2 * (na + nb), *next = scratch + na + nb;
+    float *best = reinterpret_cast<float *>(scratch);
+    NnDirs dirs{};
     NnParts parts{};
     parts.red = red;
+    const float *pts[2] = {A, B}, *nrm[2] = {nA, nB};
+    const int64_t n[2] = {na, nb};
+    NnSets sets{};
     for (int d = 0; d < 2; ++d) {
         parts.n[d] = (n[d] + kNnThreads - 1) / kNnThreads;
         parts.part[d] = parts.n[d] > 1 ? next : red + 3 * d;
         if (parts.n[d] > 1) next += 3 * parts.n[d];
     }
-    NnSets sets{};
     uint32_t *word = reinterpret_cast<uint32_t *>(next);
     bool grids = false;
     for (int d = 0; d < 2; ++d) {
@@ -694,17 +771,23 @@ extern "C" int serbf_surface_metrics(const float *A, const float *nA, int64_t na
         word = q.idx + n[d];
         grids = true;
     }
+    for (int d = 0; d < 2; ++d) {
+        dirs.d[d] = NnDir{sets.s[d], sets.s[1 - d], nrm[d], nrm[1 - d], best,
+                          reinterpret_cast<uint32_t *>(best + n[d]), const_cast<double *>(parts.part[d])};
+        best += 2 * n[d];
+    }
+    const int64_t most = na > nb ? na : nb;
     if (grids) {
-        const dim3 grid((unsigned)blocks_for(na > nb ? na : nb), 2);
+        const dim3 grid((unsigned)blocks_for(most), 2);
         launch_pdl(k_nn_clear, grid, dim3(256), 0, s, sets);
         launch_pdl(k_nn_box, grid, dim3(256), 0, s, sets);
         launch_pdl(k_nn_cells<false>, grid, dim3(256), 0, s, sets);
         launch_pdl(k_nn_scan, dim3(2), dim3(1024), 0, s, sets);
         launch_pdl(k_nn_cells<true>, grid, dim3(256), 0, s, sets);
     }
-    for (int d = 0; d < 2; ++d)
-        launch_pdl(k_nearest, dim3((unsigned)parts.n[d]), dim3(kNnThreads), 0, s, pts[d], nrm[d], n[d], sets.s[1 - d],
-                   nrm[1 - d], const_cast<double *>(parts.part[d]));
+    const dim3 each((unsigned)((most + kNnThreads - 1) / kNnThreads), 2);
+    launch_pdl(k_nearest, each, dim3(kNnThreads), 0, s, dirs);
+    launch_pdl(k_nn_sums, each, dim3(kNnThreads), 0, s, dirs);
     launch_pdl(k_metric_sums, dim3(2), dim3(1024), 0, s, parts);
     SERBF_CHECK_LAUNCH();
     double r[6];
