@@ -106,6 +106,7 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
         const serbf_field &F = fields[f];
         if (!F.cfg || !F.ws || F.ws->magic != kMagic || !F.ws->binned || F.cfg->kahan != kahan) return SERBF_EINVAL;
         items2 += F.ws->items[0].n;
+        F.ws->unmeasured = 0;  // the batched epochs measure
         sm = F.ws->sm_count;
     }
     const int G = forward_warps(items2, sm, fwd_warps);

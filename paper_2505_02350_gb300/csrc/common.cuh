@@ -104,6 +104,7 @@ struct serbf_workspace {
     float4 *tile_lo, *tile_hi;
     ItemSet items[2];
     uint32_t *class_hist;   // order chunks x kCostClasses
+    int32_t unmeasured;     // no forward has filed classes since the binning (its order stands)
     float4 *sup_lo, *sup_hi;
     // per-kernel records
     float4 *kfwd;  // 3 per kernel
@@ -224,12 +225,29 @@ __device__ __forceinline__ int cell_axis(float v, float o, float h, int n) {
     return (int)f;
 }
 
+// cell_axis with a reciprocal of h: the product decides unless it lies so
+// close to an integer that the rounded quotient might be on the other side.
+__device__ __forceinline__ int cell_axis_by(float v, float o, float h, float inv, int n) {
+    const float q = __fmul_rn(__fsub_rn(v, o), inv), f = floorf(q), r = q - f, tol = 1e-6f * fmaxf(fabsf(q), 1.f);
+    if (!(r > tol && r < 1.f - tol)) return cell_axis(v, o, h, n);
+    if (!(f >= 0.f)) return 0;
+    if (f >= (float)(n - 1)) return n - 1;
+    return (int)f;
+}
+
 // Super-major cell key: super cell id * sf^3 + cell id inside the super cell.
 __device__ __forceinline__ uint32_t cell_key(int kx, int ky, int kz, int sf, int nsx, int nsy) {
     const int sx = kx / sf, sy = ky / sf, sz = kz / sf;
     const int lx = kx - sx * sf, ly = ky - sy * sf, lz = kz - sz * sf;
     const uint32_t sup = ((uint32_t)sz * (uint32_t)nsy + (uint32_t)sy) * (uint32_t)nsx + (uint32_t)sx;
     return sup * (uint32_t)(sf * sf * sf) + (uint32_t)((lz * sf + ly) * sf + lx);
+}
+
+// cell_key for super cells of 2^lg cells per edge.
+__device__ __forceinline__ uint32_t cell_key_pow2(int kx, int ky, int kz, int lg, int nsx, int nsy) {
+    const int m = (1 << lg) - 1;
+    const uint32_t sup = ((uint32_t)(kz >> lg) * (uint32_t)nsy + (uint32_t)(ky >> lg)) * (uint32_t)nsx + (uint32_t)(kx >> lg);
+    return (sup << (3 * lg)) + (uint32_t)((((kz & m) << lg) + (ky & m) << lg) + (kx & m));
 }
 
 // Float-float ("double-float") accumulator: hi + lo carries about 48 bits.
@@ -336,6 +354,19 @@ __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// Minimum and maximum of a warp in one instruction (redux.sync, sm_100
+// family); they select one of the inputs, so the order does not matter.
+__device__ __forceinline__ float redux_min(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float redux_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 __device__ __forceinline__ float warp_max(float v) {

@@ -211,17 +211,6 @@ __device__ __forceinline__ uint32_t redux_max_u32(uint32_t v) {
     asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
     return r;
 }
-__device__ __forceinline__ float redux_min(float v) {
-    float r;
-    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ float redux_max(float v) {
-    float r;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-
 // Partial of a group of tiles: the loss sum in double (the global loss
 // reduction runs in FP64; a tile's own sum of 32 squares is float-float).
 struct FwdGPart {
@@ -1364,6 +1353,7 @@ int forward_impl(const serbf_points *pts, const serbf_params *prm, const serbf_c
     cudaStream_t s = (cudaStream_t)stream;
     int rc = SERBF_OK;
     if (ws->ntiles > 0) {
+        ws->unmeasured = 0;
         const int64_t ni = a.nitems;
         const int mode = adj ? (cfg->kahan ? 2 : 1) : 0;
         switch (G * 4 + mode) {

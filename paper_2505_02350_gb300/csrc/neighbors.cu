@@ -765,9 +765,21 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
     if (kmajor && (!kmajor->rowptr || (kmajor->cap > 0 && !kmajor->col))) return SERBF_EINVAL;
     if (pmajor && (!pmajor->rowptr || (pmajor->cap > 0 && !pmajor->col))) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    // fork: the item order for the next forward overlaps the rebuild
+    // fork: the item order for the next forward overlaps the rebuild.  Nothing
+    // to order when no forward has measured since the binning, whose order is
+    // there already -- except under capture, where the graph will be replayed
+    // after forwards that do measure.
     const ItemSet &items = items_of(ws, forward_warps(ws->items[0].n, ws->sm_count, cfg->fwd_warps));
-    const bool fork = items.n > 0 && ws->aux;
+    bool measured = !ws->unmeasured;
+    if (!measured) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+            cudaGetLastError();  // another stream's capture forbids the question on the default stream
+            measured = true;
+        }
+        measured |= capture != cudaStreamCaptureStatusNone;
+    }
+    const bool fork = items.n > 0 && ws->aux && measured;
     if (fork) {
         if (cudaEventRecord(ws->ev_fork, s) != cudaSuccess) return SERBF_ECUDA;
         if (cudaStreamWaitEvent(ws->aux, ws->ev_fork, 0) != cudaSuccess) return SERBF_ECUDA;
