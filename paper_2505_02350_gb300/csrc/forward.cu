@@ -844,7 +844,8 @@ __device__ __forceinline__ void sched_finish_batch(const FwdBatch &b, int lane) 
     }
 }
 
-// Persistent blocks take work items, heaviest first, from a global counter.
+// Persistent blocks take work items, heaviest first: block b the b-th, then
+// from a global counter (claims past the grid's first items).
 // The G warps of a block share an item (its candidate list split by 32-entry
 // chunks); their partial sums are combined in warp order, so Psi does not
 // depend on timing.  G = 1 when there are enough items to balance the warps,
@@ -885,10 +886,10 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     if (threadIdx.x == 0) {
         if (BATCH) {
             uint32_t f;
-            s_rec[0] = resolve_batch(b, atomicAdd(b.next, 1u), f);
+            s_rec[0] = resolve_batch(b, blockIdx.x, f);
             s_field[0] = f;
         } else {
-            s_rec[0] = resolve(a1, atomicAdd(a1.item_next, 1u));
+            s_rec[0] = resolve(a1, blockIdx.x);
         }
     }
     __syncthreads();
@@ -927,7 +928,7 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
         // the next claim is made now, its record is fetched after the sums
         // and used at the end, so neither round trip is on the item's path
         uint32_t knext = 0, fnext = 0;
-        if (threadIdx.x == 0) knext = atomicAdd(BATCH ? b.next : a.item_next, 1u);
+        if (threadIdx.x == 0) knext = gridDim.x + atomicAdd(BATCH ? b.next : a.item_next, 1u);
         f2 acc[NT];
         uint32_t n[NT], cost;
         int ntouch = 0;
