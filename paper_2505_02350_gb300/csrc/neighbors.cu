@@ -554,7 +554,11 @@ __global__ void __launch_bounds__(256) k_pmajor(const float *x, const float *y, 
     const float4 lo = tlo[t], hi = thi[t];
     const int L = min((int)scnt[s], scap);
     const uint32_t *lst = slist + (size_t)s * scap;
+    // a row's entries are written in aligned groups of four: single stores to
+    // 32 rows at once took a pass of the store unit each
     uint32_t *row = FILL && valid ? col + rowptr[i] : nullptr;
+    const uint32_t phase = (uint32_t)(reinterpret_cast<uintptr_t>(row) >> 2) & 3u;
+    uint32_t e0 = 0, e1 = 0, e2 = 0;  // the last three entries
     uint32_t n = 0;
     for (int b = 0; b < L; b += 32) {
         const bool live = b + lane < L;
@@ -568,10 +572,27 @@ __global__ void __launch_bounds__(256) k_pmajor(const float *x, const float *y, 
             const float cz = __shfl_sync(0xffffffffu, k.z, q), r2 = __shfl_sync(0xffffffffu, k.w, q);
             const uint32_t jq = __shfl_sync(0xffffffffu, j, q);
             if (in_support(px, py, pz, cx, cy, cz, r2)) {
-                if (FILL) row[n] = jq;
+                if (FILL && ((n + phase) & 3u) == 3u) {
+                    if (n >= 3u) {
+                        *reinterpret_cast<uint4 *>(row + n - 3) = make_uint4(e0, e1, e2, jq);
+                    } else {  // the row begins inside the group
+                        row[n] = jq;
+                        if (n > 0) row[n - 1] = e2;
+                        if (n > 1) row[n - 2] = e1;
+                    }
+                }
+                e0 = e1;
+                e1 = e2;
+                e2 = jq;
                 ++n;
             }
         }
+    }
+    if (FILL) {  // what the last group lacks
+        const uint32_t rest = min(n, (n + phase) & 3u);
+        if (rest > 0) row[n - 1] = e2;
+        if (rest > 1) row[n - 2] = e1;
+        if (rest > 2) row[n - 3] = e0;
     }
     if (!FILL && valid) rowptr[i] = n;
 }
@@ -587,7 +608,7 @@ constexpr int kRowParts = 32;
 static_assert(kRowParts == 32 && kRowParts + 4 <= kBwdWarpsPerKernel * 22, "a lane per share; the shares' counts fit the standalone adjoint's moments");
 
 template <bool FILL>
-__global__ void __launch_bounds__(256) k_kmajor(const float *x, const float *y, const float *z, const float4 *kfwd,
+__global__ void __launch_bounds__(256, 4) k_kmajor(const float *x, const float *y, const float *z, const float4 *kfwd,
                                                 const int32_t *m_dev, serbf_grid g, int sf, int nsx, int nsy,
                                                 const float4 *slo, const float4 *shi, const uint32_t *stile0,
                                                 const uint32_t *tile_start, const float4 *tlo, const float4 *thi,
@@ -605,6 +626,7 @@ __global__ void __launch_bounds__(256) k_kmajor(const float *x, const float *y, 
     const int64_t all = (int64_t)nx * ny * nz;
     const int64_t q0 = all * share / kRowParts, q1 = all * (share + 1) / kRowParts;
     uint32_t *out = FILL ? col + rowptr[j] + part[w] : nullptr;
+    const unsigned lt = (1u << lane) - 1u;
     uint32_t count = 0;
     // 32 super cells at a time, one per lane, then 32 tiles of a reached one
     for (int64_t qb = q0; qb < q1; qb += 32) {
@@ -634,13 +656,23 @@ __global__ void __launch_bounds__(256) k_kmajor(const float *x, const float *y, 
                 }
                 unsigned bal = __ballot_sync(0xffffffffu, hit);
                 while (bal) {
-                    const int ts = __ffs(bal) - 1;
+                    // two tiles at a time: their loads overlap
+                    const int ta = __ffs(bal) - 1;
                     bal &= bal - 1;
-                    const uint32_t i = __shfl_sync(0xffffffffu, start, ts) + lane;
-                    const bool in = i < end && in_support(x[i], y[i], z[i], k.x, k.y, k.z, k.w);
-                    const unsigned m = __ballot_sync(0xffffffffu, in);
-                    if (FILL && in) out[count + __popc(m & ((1u << lane) - 1u))] = i;
+                    const int tz = bal ? __ffs(bal) - 1 : ta;
+                    const bool two = bal != 0;
+                    bal &= bal - 1;
+                    const uint32_t i = __shfl_sync(0xffffffffu, start, ta) + lane, i2 = __shfl_sync(0xffffffffu, start, tz) + lane;
+                    const bool v = i < end, v2 = two && i2 < end;
+                    const float xa = v ? x[i] : 0.f, ya = v ? y[i] : 0.f, za = v ? z[i] : 0.f;
+                    const float xb = v2 ? x[i2] : 0.f, yb = v2 ? y[i2] : 0.f, zb = v2 ? z[i2] : 0.f;
+                    const bool in = v && in_support(xa, ya, za, k.x, k.y, k.z, k.w);
+                    const bool in2 = v2 && in_support(xb, yb, zb, k.x, k.y, k.z, k.w);
+                    const unsigned m = __ballot_sync(0xffffffffu, in), m2 = __ballot_sync(0xffffffffu, in2);
+                    if (FILL && in) out[count + __popc(m & lt)] = i;
                     count += __popc(m);
+                    if (FILL && in2) out[count + __popc(m2 & lt)] = i2;
+                    count += __popc(m2);
                 }
             }
         }
