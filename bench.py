@@ -38,14 +38,10 @@ ADJ_INSTR_PER_PAIR = 32  # minimum FP32-pipe instructions of one adjoint pair (r
 # kernel plus its finishing kernel, from one ncu capture per workload, warp
 # split and super-cell size, valid only for the library version it was taken
 # with (any other version, workload, split or size reports null)
-_TRAFFIC_036 = {
-    ("c4", 1, 4): 170_680_000 + 64_060_000 + 9_920_000,
-    ("c3", 2, 2): 39_480_000 + 258_560 + 2_310_000,
+TRAFFIC_BYTES = {
+    ("serbf 0.4.0 (sm_103a)", "c4", 1, 2): 183_976_448 + 61_820_416 + 9_995_264,
+    ("serbf 0.4.0 (sm_103a)", "c3", 2, 2): 39_483_904 + 312_576 + 2_309_120,
 }
-# 0.3.7 changes only the neighbour rebuild (a third list level), not the two
-# kernels captured
-TRAFFIC_BYTES = {(v,) + k: b for v in ("serbf 0.3.6 (sm_103a)", "serbf 0.3.7 (sm_103a)") for k, b in _TRAFFIC_036.items()}
-TRAFFIC_BYTES[("serbf 0.3.7 (sm_103a)", "c4", 1, 2)] = 187_060_000 + 64_840_000 + 9_990_000
 DEFAULT_STEPS = {"c1": 3000, "c2": 3000, "c3": 500, "c4": 200, "c5": 2000}
 WORKLOADS = {
     "c1": ("sphere |x|-0.5 on 32^3, M=64 isotropic", None),
@@ -456,7 +452,7 @@ def run_batched(args, ws, rank, local):
                    "autotune_ms": {str(k): round(v, 4) for k, v in tune.items()},
                    "batched": "serbf_epoch_batched in one CUDA graph per epoch: one persistent forward + adjoint "
                               "launch over every field's work items, one launch per other stage",
-                   "loop": "each field's epoch graph (11 launches) in turn",
+                   "loop": "each field's epoch graph (10 launches) in turn",
                    "target": "each field's RMSE after the loop's %d epochs (Algorithm 3 to M^e)" % E,
                    "check_every": chunk, "l2_flush": "256 MiB buffer written before each timed run"},
         "loop_s": t_loop, "speedup_vs_loop": t_loop / t_batch, "epochs_to_target": done,
