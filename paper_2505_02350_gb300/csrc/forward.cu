@@ -883,23 +883,26 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     NzPoints &nzs = *reinterpret_cast<NzPoints *>(ringP[warp]);
     uint32_t *adjq = reinterpret_cast<uint32_t *>(ringF[warp]);
+    // the first record lies in the slot that the first item does not write: a
+    // warp may still have to read it when thread 0 stores the second one
+    constexpr int kFirstSlot = 1;
     if (threadIdx.x == 0) {
         if (BATCH) {
             uint32_t f;
-            s_rec[0] = resolve_batch(b, blockIdx.x, f);
-            s_field[0] = f;
+            s_rec[kFirstSlot] = resolve_batch(b, blockIdx.x, f);
+            s_field[kFirstSlot] = f;
         } else {
-            s_rec[0] = resolve(a1, blockIdx.x);
+            s_rec[kFirstSlot] = resolve(a1, blockIdx.x);
         }
     }
     __syncthreads();
-    uint4 rec = s_rec[0];  // the item's record; x = ~0 when done
-    uint32_t field = BATCH ? s_field[0] : 0u, loaded = ~0u;
+    uint4 rec = s_rec[kFirstSlot];  // the item's record; x = ~0 when done
+    uint32_t field = BATCH ? s_field[kFirstSlot] : 0u, loaded = ~0u;
     uint32_t mean = BATCH ? 0u : a1.sched[0];
     const FwdArgs &a = BATCH ? *reinterpret_cast<const FwdArgs *>(s_args) : a1;
     // several warps: buffer of the current item, and the last item's record,
     // whose cost is noted once its warps have met again
-    int par = 0;
+    int par = kFirstSlot ^ 1;
     uint4 done = make_uint4(~0u, 0u, 0u, 0u);
     auto note_done = [&]() {
         if (G > 1 && threadIdx.x == 0 && done.x != ~0u) {
@@ -1008,7 +1011,8 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
             // warps 0 and 1 also write a tile each.  (With the nz points made by
             // those two for all there were four barriers, a fifth of the warps'
             // time for 64^3 + 32^3 points.)  A buffer is written again two
-            // items later, past the barrier that follows its last reader.
+            // items later, past the barrier that follows its last reader; the
+            // record of the first item lies in the buffer of the second one.
             {
                 float l0, h0, l1, h1;
                 f2_unpack(acc[0], l0, h0);
