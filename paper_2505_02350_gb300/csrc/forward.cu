@@ -29,6 +29,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "form_bound.cuh"
 
 using namespace serbf;
 
@@ -621,41 +622,14 @@ __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *
     }
 }
 
-// Lower bound of a kernel's quadratic form (log2 units) over a box with
-// centre b and half diagonal hd, less ceil(log2(max(1, r2))): by the triangle
-// inequality sqrt(q) falls by at most sqrt(largest eigenvalue of Q) hd on the
-// way from the centre, and k2.w holds that root.  The float error of q, here
-// and in the pair loop, is a few units of 2^-24 of the largest eigenvalue
-// times |Delta|^2, and |Delta|^2 < r2 for a support pair: eps covers both many
-// times over.  Not finite in, NaN out (which culls nothing).
-__device__ __forceinline__ float form_floor(float4 k0, float4 k1, float4 k2, float4 b, float hd) {
-    const float dx = b.x - k0.x, dy = b.y - k0.y, dz = b.z - k0.z;
-    const float ra = fmaf(k2.y, dz, fmaf(k2.x, dy, k1.x * dx)), rb = fmaf(k2.z, dz, k1.y * dy);
-    const float q = fmaf(k1.z, dz * dz, fmaf(dy, rb, dx * ra));
-    const float eps = 1.6e-5f * k2.w * k2.w * k0.w;
-    const float s = fmaf(-1.0001f * k2.w, hd, sqrtf(q - eps));
-    const float lg = fmaxf((float)((int)(__float_as_uint(k0.w) >> 23) - 126), 0.f);
-    return s > 0.f ? fmaf(s, s, -eps) - lg : 0.f * s;
-}
-
-// Power of two above which a kernel's form makes all its moments over the
-// item's cnt residual points round to zero: |moment| <= cnt max|E| 2^-q
-// max(1, r2) (phi <= 2^-q, and |Delta| <= sqrt(r2) in the support) is below
-// 2^-38 for q - log2(max(1, r2)) > this.  Infinite when a residual is not
-// finite (emax is the largest of the residuals' absolute bits, where a NaN
-// lies above everything).
-__device__ __forceinline__ float form_limit(float emax, int cnt) {
-    const int e = (int)(__float_as_uint(emax) >> 23);  // emax < 2^(e - 126)
-    return e >= 255 ? INFINITY : (float)(38 + (e - 126) + (32 - __clz(cnt)));
-}
-
 // One warp's share of an item's adjoint: the kernels this warp found
 // reaching the item box (or, if it found more than tcap, its candidate
 // chunks of the super cell's list again), filtered against the nz box.  A
 // kernel whose form is so large over that box that every moment would be
-// converted to a fixed-point zero is left out as well: the accumulators hold
-// the same bits without it (supports are balls of the longest axis, so about a
-// quarter of the support pairs of kernels with axes of 1 : 4 lie there).  The
+// converted to a fixed-point zero is left out as well: it would add nothing
+// (supports are balls of the longest axis, so about a quarter of the support
+// pairs of kernels with axes of 1 : 4 lie there; the kernels that stay may form
+// a shorter last batch, which other lanes share, and round otherwise).  The
 // test stands here and not in the forward's scan, where every candidate would
 // pay for it: an epoch of 9.4 M points and 16384 kernels took 2560 us without
 // it, 2462 us with it here, 2533 us with it there.
