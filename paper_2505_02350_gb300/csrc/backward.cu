@@ -26,11 +26,13 @@ static_assert(kBwdWarpsPerKernel == 32, "the epilogue reduces one partial per la
 
 namespace {
 
-// One block per (32-tile chunk, super cell), one warp per tile: compact the
+// One block per (super cell, chunk row), one warp per tile: compact the
 // tile's nonzero-residual points into its 32 slots (x, y, z, E), then warp 0
 // packs the chunk's tiles that hold any as two float4 records -- (box lo,
 // count) and (box hi, tile id) -- at the chunk's own record slots, so the
-// adjoint reads a candidate tile's test data in one round trip.
+// adjoint reads a candidate tile's test data in one round trip.  The super
+// cells lie along the grid's x: y holds 65535 at most, and a field may have
+// more of them.
 __global__ void __launch_bounds__(1024) k_nz_compact(const float *x, const float *y, const float *z, const float *err,
                                                      const uint32_t *stile0, const uint32_t *tile_start,
                                                      const uint32_t *cell_start, int cps, const float4 *tlo,
@@ -38,36 +40,39 @@ __global__ void __launch_bounds__(1024) k_nz_compact(const float *x, const float
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t cnt[32];
-    const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t t0 = stile0[s], t1 = stile0[s + 1];
-    const uint32_t cb = t0 + blockIdx.x * 32u;
-    if (cb >= t1) return;
-    const uint32_t t = cb + warp;
-    uint32_t c = 0;
-    if (t < t1) {
-        const uint32_t pe = cell_start[(int64_t)(s + 1) * cps];
-        const uint32_t i = tile_start[t] + lane;
-        const float e = i < pe ? err[i] : 0.f;
-        const bool v = e != 0.f;
-        const unsigned bal = __ballot_sync(0xffffffffu, v);
-        if (v) nz[(size_t)t * kTile + __popc(bal & ((1u << lane) - 1u))] = make_float4(x[i], y[i], z[i], e);
-        c = __popc(bal);
+    const unsigned lt = (1u << lane) - 1u;
+    for (uint32_t cb = t0 + blockIdx.y * 32u; cb < t1; cb += gridDim.y * 32u) {
+        const uint32_t t = cb + warp;
+        uint32_t c = 0;
+        if (t < t1) {
+            const uint32_t pe = cell_start[(int64_t)(s + 1) * cps];
+            const uint32_t i = tile_start[t] + lane;
+            const float e = i < pe ? err[i] : 0.f;
+            const bool v = e != 0.f;
+            const unsigned bal = __ballot_sync(0xffffffffu, v);
+            if (v) nz[(size_t)t * kTile + __popc(bal & lt)] = make_float4(x[i], y[i], z[i], e);
+            c = __popc(bal);
+        }
+        if (lane == 0) cnt[warp] = c;
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t tt = cb + lane;
+            const uint32_t cl = cnt[lane];
+            const unsigned bal = __ballot_sync(0xffffffffu, cl != 0);
+            if (cl) {
+                const uint32_t o = cb + __popc(bal & lt);
+                float4 lo = tlo[tt], hi = thi[tt];
+                lo.w = __uint_as_float(cl);
+                hi.w = __uint_as_float(tt);
+                rec[2 * (size_t)o] = lo;
+                rec[2 * (size_t)o + 1] = hi;
+            }
+            if (lane == 0) ccnt[cb] = __popc(bal);
+        }
+        __syncthreads();
     }
-    if (lane == 0) cnt[warp] = c;
-    __syncthreads();
-    if (warp != 0) return;
-    const uint32_t tt = cb + lane;
-    const uint32_t cl = cnt[lane];
-    const unsigned bal = __ballot_sync(0xffffffffu, cl != 0);
-    if (cl) {
-        const uint32_t o = cb + __popc(bal & ((1u << lane) - 1u));
-        float4 lo = tlo[tt], hi = thi[tt];
-        lo.w = __uint_as_float(cl);
-        hi.w = __uint_as_float(tt);
-        rec[2 * (size_t)o] = lo;
-        rec[2 * (size_t)o + 1] = hi;
-    }
-    if (lane == 0) ccnt[cb] = __popc(bal);
 }
 
 struct BwdArgs {
@@ -244,7 +249,7 @@ extern "C" int serbf_backward(const serbf_points *pts, const serbf_params *prm, 
     const int64_t nt = ws->ntiles;
     const int cps = ws->sf * ws->sf * ws->sf;
     if (nt > 0)
-        launch_pdl(k_nz_compact, dim3((unsigned)ws->max_chunks, (unsigned)ws->nsuper), dim3(1024), 0, s,
+        launch_pdl(k_nz_compact, dim3((unsigned)ws->nsuper, (unsigned)(ws->max_chunks < 65535 ? ws->max_chunks : 65535)), dim3(1024), 0, s,
             pts->x, pts->y, pts->z, err, ws->super_tile0, ws->tile_start, ws->cell_start, cps, ws->tile_lo,
             ws->tile_hi, ws->nz, ws->nzrec, ws->nzc_cnt);
     BwdArgs a;
