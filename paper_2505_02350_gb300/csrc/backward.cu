@@ -18,6 +18,7 @@
 // kBwdSplit blocks: no global atomics.
 #include <math.h>
 
+#include "chunk_rows.cuh"
 #include "common.cuh"
 
 using namespace serbf;
@@ -75,6 +76,11 @@ __global__ void __launch_bounds__(1024) k_nz_compact(const float *x, const float
     }
 }
 
+// As many rows as a kernel's warps look at in so many passes of their lanes are
+// taken whatever the average super cell holds (bounded by its chunk_rows alone,
+// the uneven sets there took 402 and 838 us).
+constexpr int kRowPasses = 8;
+
 struct BwdArgs {
     const float4 *kbwd;
     const int32_t *m;
@@ -87,7 +93,7 @@ struct BwdArgs {
     const float4 *nzrec;   // packed records of tiles with nonzero residuals, per 32-tile chunk
     const uint32_t *nzc;   // records per chunk, indexed by the chunk's first tile
     const float4 *nz;
-    int chunks;  // most 32-tile chunks in one super cell
+    int rows, chunks;  // rows of 32-tile chunks per super cell (at least), and the most chunks of one
     float *mom;  // per kernel, per warp: 10 float-float moments S0, M1 (3), M2 (6), then the pair count (bits)
 };
 
@@ -113,56 +119,70 @@ __global__ void __launch_bounds__(kBwdThreads) k_moments(BwdArgs a) {
     int head = 0, qn = 0;
     uint32_t *q = ring[warp];
     // the 32-tile chunks of the kernel's super cells are dealt round-robin to
-    // all its warps; a warp tests 32 of its chunks at once (one per lane), then
-    // walks the packed nonzero tiles of those its support may reach.  Whole
-    // super cells of 4096 points left some warps with several and others with
-    // none: 19.7 M pairs of 512 kernels took 128 us, in chunks 101 us.  (Packed
-    // pairs of points, and tiles taken around the queue, did not help: 105 and
-    // 130 us, with more registers and fewer warps.)
+    // all its warps, in rows: row r of a super cell is its chunks r, r + rows,
+    // ... (one chunk a row unless the points are very uneven, see chunk_rows).
+    // A super cell's rows lie side by side, turned by one for every W rows
+    // before it: where the rows divide the warps, some warps would get the full
+    // chunks and others the remainders.  A warp tests 32 of its rows at once
+    // (one per lane), then walks the packed nonzero tiles of the chunks its
+    // support may reach.
+    // Whole super cells left some warps with several and others with none: 64^3
+    // points and 512 kernels 89 us, in chunks 66; 100 000 scattered points (43
+    // tiles a super cell) 53.5, in unturned rows 57, turned 49.  (Packed pairs of
+    // points, and tiles taken around the queue, did not help: 4 and 29 % slower,
+    // with more registers and fewer warps.)
     const int W = NW * gridDim.y, wid = split * NW + warp;
-    const int64_t units = (int64_t)nsb * a.chunks;
+    const int rows = min(a.chunks, max(a.rows, kRowPasses * 32 * W / nsb));
+    const int64_t units = (int64_t)nsb * rows;
     for (int64_t base = wid; base < units; base += W * 32) {
         const int64_t un = base + (int64_t)lane * W;
-        uint32_t first = 0, cnt = 0;  // the chunk's first tile and its number of records
+        uint32_t first = 0, end = 0;  // the row's next chunk (its first tile) and the super cell's end
         if (un < units) {
-            const int sb = (int)(un / a.chunks), ch = (int)(un - (int64_t)sb * a.chunks);
+            const int sb = (int)(un / rows);
+            const int64_t before = (int64_t)sb * rows;
+            const int row = (int)((un - before + before / W) % rows);
             const int sx = sx0 + sb % nbx, sy = sy0 + (sb / nbx) % nby, sz = sz0 + sb / (nbx * nby);
             const int s = (sz * a.nsy + sy) * a.nsx + sx;
-            first = a.stile0[s] + 32u * ch;
-            if (first < a.stile0[s + 1] && box_d2(k0.x, k0.y, k0.z, a.slo[s], a.shi[s]) < k0.w) cnt = a.nzc[first];
+            first = a.stile0[s] + 32u * row;
+            end = a.stile0[s + 1];
+            if (first < end && !(box_d2(k0.x, k0.y, k0.z, a.slo[s], a.shi[s]) < k0.w)) end = first;
         }
-        unsigned cbal = __ballot_sync(0xffffffffu, cnt != 0);
-        while (cbal) {
-            const int csrc = __ffs(cbal) - 1;
-            cbal &= cbal - 1;
-            const uint32_t cb = __shfl_sync(0xffffffffu, first, csrc), ncr = __shfl_sync(0xffffffffu, cnt, csrc);
-            uint32_t c = 0, t = 0;
-            if ((uint32_t)lane < ncr) {
-                const float4 lo = a.nzrec[2 * (size_t)(cb + lane)], hi = a.nzrec[2 * (size_t)(cb + lane) + 1];
-                if (box_d2(k0.x, k0.y, k0.z, lo, hi) < k0.w) {
-                    c = __float_as_uint(lo.w);
-                    t = __float_as_uint(hi.w);
+        while (__any_sync(0xffffffffu, first < end)) {
+            const uint32_t cnt = first < end ? a.nzc[first] : 0u;
+            unsigned cbal = __ballot_sync(0xffffffffu, cnt != 0);
+            while (cbal) {
+                const int csrc = __ffs(cbal) - 1;
+                cbal &= cbal - 1;
+                const uint32_t cb = __shfl_sync(0xffffffffu, first, csrc), ncr = __shfl_sync(0xffffffffu, cnt, csrc);
+                uint32_t c = 0, t = 0;
+                if ((uint32_t)lane < ncr) {
+                    const float4 lo = a.nzrec[2 * (size_t)(cb + lane)], hi = a.nzrec[2 * (size_t)(cb + lane) + 1];
+                    if (box_d2(k0.x, k0.y, k0.z, lo, hi) < k0.w) {
+                        c = __float_as_uint(lo.w);
+                        t = __float_as_uint(hi.w);
+                    }
                 }
-            }
-            unsigned bal = __ballot_sync(0xffffffffu, c != 0);
-            while (bal) {
-                const int src = __ffs(bal) - 1;
-                bal &= bal - 1;
-                const uint32_t cc = __shfl_sync(0xffffffffu, c, src);
-                const uint32_t tt = __shfl_sync(0xffffffffu, t, src);
-                if (lane < (int)cc) q[(head + qn + lane) & (RING - 1)] = tt * kTile + lane;
-                qn += cc;
-                __syncwarp();
-                if (qn >= 64) {
-                    const float4 p0 = a.nz[q[(head + lane) & (RING - 1)]];
-                    const float4 p1 = a.nz[q[(head + 32 + lane) & (RING - 1)]];
-                    accumulate<KAHAN>(p0, k0, k1, k2, k3, acc, cmp, pairs);
-                    accumulate<KAHAN>(p1, k0, k1, k2, k3, acc, cmp, pairs);
-                    head = (head + 64) & (RING - 1);
-                    qn -= 64;
+                unsigned bal = __ballot_sync(0xffffffffu, c != 0);
+                while (bal) {
+                    const int src = __ffs(bal) - 1;
+                    bal &= bal - 1;
+                    const uint32_t cc = __shfl_sync(0xffffffffu, c, src);
+                    const uint32_t tt = __shfl_sync(0xffffffffu, t, src);
+                    if (lane < (int)cc) q[(head + qn + lane) & (RING - 1)] = tt * kTile + lane;
+                    qn += cc;
                     __syncwarp();
+                    if (qn >= 64) {
+                        const float4 p0 = a.nz[q[(head + lane) & (RING - 1)]];
+                        const float4 p1 = a.nz[q[(head + 32 + lane) & (RING - 1)]];
+                        accumulate<KAHAN>(p0, k0, k1, k2, k3, acc, cmp, pairs);
+                        accumulate<KAHAN>(p1, k0, k1, k2, k3, acc, cmp, pairs);
+                        head = (head + 64) & (RING - 1);
+                        qn -= 64;
+                        __syncwarp();
+                    }
                 }
             }
+            first += 32u * (uint32_t)rows;
         }
     }
     if (lane < qn) accumulate<KAHAN>(a.nz[q[(head + lane) & (RING - 1)]], k0, k1, k2, k3, acc, cmp, pairs);
@@ -247,9 +267,10 @@ extern "C" int serbf_backward(const serbf_points *pts, const serbf_params *prm, 
     if (!grad || !stats || (pts->n > 0 && (!err || !pts->x || !pts->y || !pts->z))) return SERBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t nt = ws->ntiles;
+    const int rows = chunk_rows(nt, ws->nsuper, ws->max_chunks);
     const int cps = ws->sf * ws->sf * ws->sf;
     if (nt > 0)
-        launch_pdl(k_nz_compact, dim3((unsigned)ws->nsuper, (unsigned)(ws->max_chunks < 65535 ? ws->max_chunks : 65535)), dim3(1024), 0, s,
+        launch_pdl(k_nz_compact, dim3((unsigned)ws->nsuper, (unsigned)(rows < 65535 ? rows : 65535)), dim3(1024), 0, s,
             pts->x, pts->y, pts->z, err, ws->super_tile0, ws->tile_start, ws->cell_start, cps, ws->tile_lo,
             ws->tile_hi, ws->nz, ws->nzrec, ws->nzc_cnt);
     BwdArgs a;
@@ -268,6 +289,7 @@ extern "C" int serbf_backward(const serbf_points *pts, const serbf_params *prm, 
     a.nzrec = ws->nzrec;
     a.nzc = ws->nzc_cnt;
     a.nz = ws->nz;
+    a.rows = rows;
     a.chunks = ws->max_chunks;
     a.mom = ws->moments;
     // enough warps in flight: split a kernel's super cells over more blocks when
