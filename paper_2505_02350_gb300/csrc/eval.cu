@@ -331,6 +331,13 @@ constexpr int kNnThreads = 256;
 constexpr int64_t kNnMin = 1024;
 constexpr int kNnMaxLevels = 8;
 constexpr int kNnLeaf = 16;  // nodes of so few points are not split further
+// A set with more than 1 / kNnDense of its points in one cell is streamed as
+// well: a far point stretches the box until a cluster lies in a few cells, and
+// its queries would walk them point by point through the index.  Two sets of
+// 10^5 points, each with one point at a hundred times the others' extent: 18.0 ms
+// by cells, 8.8 streamed (all pairs at any time: 10.8 before the grid).  At ten
+// times the extent (densest cell below 1 / 8) cells take 1.5 ms.
+constexpr int64_t kNnDense = 8;
 
 __device__ __forceinline__ float nn_d2(float px, float py, float pz, const float *q) {
     const float dx = __fsub_rn(px, q[0]), dy = __fsub_rn(py, q[1]), dz = __fsub_rn(pz, q[2]);
@@ -338,14 +345,14 @@ __device__ __forceinline__ float nn_d2(float px, float py, float pz, const float
 }
 
 // One set and its grid.  box: ordered keys of the least and the largest finite
-// coordinate per axis.
+// coordinate per axis, then the most points in one cell.
 struct NnSet {
     const float *p;
     int64_t n;
     int levels;     // < 0: no grid
     uint32_t *end;  // per cell, after k_nn_fill: one past its last point
     uint32_t *idx;  // point indices by cell
-    int *box;       // 6
+    int *box;       // 7
 };
 
 struct NnFrame {
@@ -403,7 +410,8 @@ __global__ void k_nn_clear(NnSets a) {
     const int64_t cells = (int64_t)1 << (3 * s.levels);
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < cells; c += (int64_t)gridDim.x * blockDim.x)
         s.end[c] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x < 6) s.box[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (int)0x80000000;
+    if (blockIdx.x == 0 && threadIdx.x < 7)
+        s.box[threadIdx.x] = threadIdx.x < 3 ? 0x7fffffff : (threadIdx.x < 6 ? (int)0x80000000 : 0);
 }
 
 __global__ void __launch_bounds__(256) k_nn_box(NnSets a) {
@@ -456,7 +464,7 @@ __global__ void __launch_bounds__(1024) k_nn_scan(NnSets a) {
     const NnSet &s = a.s[blockIdx.x];
     if (s.levels < 0) return;
     const int64_t cells = (int64_t)1 << (3 * s.levels);
-    uint32_t carry = 0;
+    uint32_t carry = 0, most = 0;
     for (int64_t c0 = 0; c0 < cells; c0 += 4096) {
         const int64_t c = c0 + 4 * threadIdx.x;
         uint32_t v[4], sum = 0;
@@ -464,6 +472,7 @@ __global__ void __launch_bounds__(1024) k_nn_scan(NnSets a) {
         for (int k = 0; k < 4; ++k) {
             v[k] = c + k < cells ? s.end[c + k] : 0u;
             sum += v[k];
+            most = max(most, v[k]);
         }
         uint32_t total, o = block_exscan(sum, tmp, &total) + carry;
 #pragma unroll
@@ -473,6 +482,8 @@ __global__ void __launch_bounds__(1024) k_nn_scan(NnSets a) {
         }
         carry += total;
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s.box[6], (int)most);
 }
 
 // Best point of the grid of Q for p, from (best, bi).
@@ -561,7 +572,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nearest(NnDirs a) {
     const float px = d.P.p[3 * i], py = d.P.p[3 * i + 1], pz = d.P.p[3 * i + 2];
     float best = INFINITY;
     int64_t bi = 0;
-    if (d.Q.levels >= 0) {
+    if (d.Q.levels >= 0 && kNnDense * d.Q.box[6] <= d.Q.n) {
         if (live) nn_search(d.Q, nn_frame(d.Q), px, py, pz, best, bi);
     } else {
         for (int64_t j0 = 0; j0 < d.Q.n; j0 += kNnThreads) {
