@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "order_rule.cuh"
 
 using namespace serbf;
 
@@ -55,14 +56,14 @@ __device__ __forceinline__ void prep_kernels(const float *p, int cap, int m, flo
     }
 }
 
-// One launch makes the order up to so many points, and items (the counters
-// below hold 255 per thread).
-constexpr int64_t kOrderDirectPoints = 1 << 22, kOrderDirect = 128 * kOrderChunk;
+// One launch makes the order of so many items (the counters below hold 255 per
+// thread of a block).
+static_assert(kOrderDirectItems <= 128 * kOrderChunk, "items per thread of the one-launch order");
 
 // The forward's heavy-first order for its next launch: a stable sort of the
 // items by the cost class the last forward filed, descending, in one launch
-// (up to 4.2 M points) or two on the workspace's side stream (next to the
-// neighbour rebuild).
+// or two (order_direct) on the workspace's side stream (next to the neighbour
+// rebuild).
 // k_class_count: block b counts the classes of items [b kOrderChunk,
 // (b + 1) kOrderChunk).  k_order_items: block b places the same items; a
 // class starts after all heavier classes and after this class in earlier
@@ -103,8 +104,8 @@ __device__ __forceinline__ void order_items_body(const uint8_t *item_class, cons
     if (!hist) {
         if (threadIdx.x < kCostClasses) s_base[threadIdx.x] = s_tot[threadIdx.x] = 0u;
         __syncthreads();
-        // four items at a time; eight 8-bit counters a thread (kOrderDirect
-        // items are 128 per thread)
+        // four items at a time; eight 8-bit counters a thread (kOrderDirectItems
+        // are 128 per thread)
         unsigned long long tot = 0ull, before = 0ull;
         for (int64_t i = 4 * (int64_t)threadIdx.x; i < nitems; i += 4 * kOrderChunk) {
             const uint32_t w = *reinterpret_cast<const uint32_t *>(item_class + i);
@@ -820,7 +821,7 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
         const unsigned nchunks = (unsigned)((items.n + kOrderChunk - 1) / kOrderChunk);
         // few items: every block counts all classes itself, one launch less on
         // the way to the forward
-        const bool direct = ws->npoints <= kOrderDirectPoints && items.n <= kOrderDirect;
+        const bool direct = order_direct(ws->npoints, ws->nsuper);
         if (!direct) k_class_count<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, items.n, ws->class_hist);
         k_order_items<<<nchunks, kOrderChunk, 0, ws->aux>>>(items.cls, direct ? nullptr : ws->class_hist, items.rec,
                                                             items.order, items.n);

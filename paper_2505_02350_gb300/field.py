@@ -217,8 +217,9 @@ class Problem:
 
     def launches_per_epoch(self):
         """Kernel launches of one fused full-batch epoch: item order (side
-        stream; 1 up to 2^22 points, else 2), rebuild (1; 2 when the library builds the candidate lists
-        in two levels: cfg.rebuild_levels >= 2, or 0 with super cells x
+        stream; 1 up to 2^16 items, counted as one per 64 points and one per
+        super cell that may hold points, else 2), rebuild (1; 2 when the library
+        builds the candidate lists in two levels: cfg.rebuild_levels >= 2, or 0 with super cells x
         kernel capacity >= 2^25 on a grid whose blocks of 2 x 2 x 2 super
         cells fit the workspace; 3 in three levels: cfg.rebuild_levels == 3,
         or 0 with those blocks x capacity >= 2^25 as well), forward + finish
@@ -231,7 +232,8 @@ class Problem:
         lv = self.cfg.rebuild_levels
         two = (lv >= 2 or (lv == 0 and nsuper * self.cap >= 1 << 25)) and ncoarse <= nsuper // 4 + 16
         three = two and (lv == 3 or (lv == 0 and ncoarse * self.cap >= 1 << 25)) and ntop <= nsuper
-        return 9 + (1 if self.n <= 1 << 22 else 2) + (1 if two else 0) + (1 if three else 0)
+        direct = self.n // 64 + min(nsuper, self.n) <= 1 << 16
+        return 9 + (1 if direct else 2) + (1 if two else 0) + (1 if three else 0)
 
     def epoch(self):
         """One Algorithm 3 epoch with the full batch: no host synchronisation."""
