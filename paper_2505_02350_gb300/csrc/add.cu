@@ -404,14 +404,15 @@ __device__ void append_kept(const AppendArgs &a, const uint32_t *sel_idx, const 
         a.st->m_added = added;
         a.st->adam_t = 0;
         a.st->do_add = 0;
-        info[0] = 0;
+        // info[0] stays: blocks of this launch may still have to read it, and the
+        // next addition's first launch sets it
     }
 }
 
 // Warps over the selected points (grid-stride): reject a point if an id_all
 // point within the radius has a larger |E| (distance in float, same operation
-// order as the support test, <= r2).  One block per SM, so a step without an
-// addition retires few blocks.  The last block appends the survivors.
+// order as the support test, <= r2).  Few blocks per SM, so that a step without
+// an addition retires few.  The last block appends the survivors.
 __device__ __forceinline__ void add_localmax_body(const AddArgs &A, int bx, int nbx) {
     const AppendArgs &ap = A.ap;
     const uint32_t *sel_idx = A.lo;  // the sorted selection's indices
@@ -446,24 +447,104 @@ __global__ void __launch_bounds__(kLmThreads) k_add_localmax(AddArgs A) {
     add_localmax_body(A, blockIdx.x, gridDim.x);
 }
 
-// Batches of fields: field blockIdx.y.
-__global__ void __launch_bounds__(kHistThreads) k_add_hist_batch(const AddArgs *aa) {
+// Batches of fields.  Most epochs add nothing, so a launch has about a single
+// field's blocks; they are shared out among the fields whose addition is due, a
+// block to each and the others by their points.
+constexpr int kMaxDue = 1024;  // fields of a batch
+
+struct Share {
+    int field;    // -1: nothing is due
+    int bx, nbx;  // this block's place among the field's blocks
+};
+
+// This block's share, for the fields for which due(field) holds; needs at least
+// as many blocks as fields.  Every block comes to the same division: due fields
+// in order, the j-th from block j + (blocks - due fields) points before it /
+// points of all.
+template <typename Due>
+__device__ __forceinline__ Share due_share(const AddArgs *aa, int nfields, Due due) {
+    constexpr int kPer = 8;  // fields per thread at most (blocks of 128 threads or more)
+    __shared__ long long s_points[32];
+    __shared__ int s_count[32];
+    __shared__ Share s_share;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int per = (nfields + (int)blockDim.x - 1) / (int)blockDim.x, f0 = (int)threadIdx.x * per;
+    long long points = 0;
+    int count = 0;
+    uint32_t mine = 0;
+    for (int k = 0; k < per && k < kPer; ++k)
+        if (f0 + k < nfields && due(f0 + k)) {
+            mine |= 1u << k;
+            points += aa[f0 + k].n;
+            ++count;
+        }
+    if (!__syncthreads_or(count)) return Share{-1, 0, 1};
+    // exclusive sums over the threads (fields in order), and the totals
+    long long ip = points;
+    int ic = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long p = __shfl_up_sync(0xffffffffu, ip, o);
+        const int c = __shfl_up_sync(0xffffffffu, ic, o);
+        if (lane >= o) {
+            ip += p;
+            ic += c;
+        }
+    }
+    if (lane == 31) {
+        s_points[warp] = ip;
+        s_count[warp] = ic;
+    }
+    __syncthreads();
+    long long before = ip - points, all = 0;
+    int at = ic - count, ndue = 0;
+    for (int w = 0; w < nw; ++w) {
+        if (w < warp) {
+            before += s_points[w];
+            at += s_count[w];
+        }
+        all += s_points[w];
+        ndue += s_count[w];
+    }
+    const long long extra = (long long)gridDim.x - ndue;
+    for (int k = 0; k < per && k < kPer; ++k) {
+        if (!((mine >> k) & 1u)) continue;
+        const long long n = aa[f0 + k].n, div = all > 0 ? all : 1;
+        const int b0 = at + (int)(extra * before / div);
+        const int b1 = at + 1 == ndue ? (int)gridDim.x : at + 1 + (int)(extra * (before + n) / div);
+        if (b0 <= (int)blockIdx.x && (int)blockIdx.x < b1) s_share = Share{f0 + k, (int)blockIdx.x - b0, b1 - b0};
+        before += n;
+        ++at;
+    }
+    __syncthreads();
+    return s_share;
+}
+static_assert(kMaxDue <= 8 * kLmThreads && kMaxDue <= 8 * kHistThreads && kMaxDue <= 8 * kGatherThreads, "fields per thread");
+
+__global__ void __launch_bounds__(kHistThreads) k_add_hist_batch(const AddArgs *aa, int nfields) {
     pdl_wait();
     pdl_trigger();
-    add_hist_body(aa[blockIdx.y], blockIdx.x, gridDim.x);
+    const Share h = due_share(aa, nfields, [&](int f) {
+        const bool go = aa[f].force || aa[f].ap.st->do_add;
+        if (!go && blockIdx.x == 0) aa[f].info[0] = 0;
+        return go;
+    });
+    if (h.field >= 0) add_hist_body(aa[h.field], h.bx, h.nbx);
 }
 
-__global__ void __launch_bounds__(kGatherThreads) k_add_gather_batch(const AddArgs *aa) {
+__global__ void __launch_bounds__(kGatherThreads) k_add_gather_batch(const AddArgs *aa, int nfields) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem[];
-    add_gather_body(aa[blockIdx.y], blockIdx.x, gridDim.x, smem);
+    const Share h = due_share(aa, nfields, [&](int f) { return aa[f].info[0] != 0; });
+    if (h.field >= 0) add_gather_body(aa[h.field], h.bx, h.nbx, smem);
 }
 
-__global__ void __launch_bounds__(kLmThreads) k_add_localmax_batch(const AddArgs *aa) {
+__global__ void __launch_bounds__(kLmThreads) k_add_localmax_batch(const AddArgs *aa, int nfields) {
     pdl_wait();
     pdl_trigger();
-    add_localmax_body(aa[blockIdx.y], blockIdx.x, gridDim.x);
+    const Share h = due_share(aa, nfields, [&](int f) { return aa[f].info[0] != 0; });
+    if (h.field >= 0) add_localmax_body(aa[h.field], h.bx, h.nbx);
 }
 
 int gather_smem() {
@@ -543,13 +624,15 @@ int batch_add_launch(const void *args, int nfields, int sm_count, cudaStream_t s
     if (gather_attr()) return SERBF_ECUDA;
     const AddArgs *aa = static_cast<const AddArgs *>(args);
     const unsigned nsm = (unsigned)(sm_count > 0 ? sm_count : 1);
-    // as many blocks in all as a single field takes, at least 8 per field: most
-    // epochs add nothing, and retiring a single field's blocks for each of 16
-    // fields took 37 us
-    const unsigned per = nsm / (unsigned)nfields > 8 ? nsm / (unsigned)nfields : 8;
-    launch_pdl(k_add_hist_batch, dim3(2 * per, (unsigned)nfields), dim3(kHistThreads), 0, s, aa);
-    launch_pdl(k_add_gather_batch, dim3(per, (unsigned)nfields), dim3(kGatherThreads), (size_t)gather_smem(), s, aa);
-    launch_pdl(k_add_localmax_batch, dim3(per, (unsigned)nfields), dim3(kLmThreads), 0, s, aa);
+    // 16 fields (5.2 M points, four of 884 736 points), an epoch of 549 us when
+    // nothing is due: one large field due +273 us, all +482 (four blocks per SM in
+    // the last launch +543).  With a single field's blocks for each +250 and +455,
+    // but 37 on every epoch; with 18, 9 and 9 blocks a field +376 and +2290: the
+    // local-maximum test wants every warp there is.
+    const auto blocks = [&](unsigned per_sm) { return dim3(per_sm * nsm > (unsigned)nfields ? per_sm * nsm : (unsigned)nfields); };
+    launch_pdl(k_add_hist_batch, blocks(2), dim3(kHistThreads), 0, s, aa, nfields);
+    launch_pdl(k_add_gather_batch, blocks(1), dim3(kGatherThreads), (size_t)gather_smem(), s, aa, nfields);
+    launch_pdl(k_add_localmax_batch, blocks(8), dim3(kLmThreads), 0, s, aa, nfields);
     SERBF_CHECK_LAUNCH();
     return SERBF_OK;
 }
