@@ -203,7 +203,13 @@ class Problem:
         times = {}
         for g in (1, 2, 4, 8):
             self.cfg.fwd_warps = g
-            fn()  # files the work costs for this configuration's order
+            # the order that an epoch of a fit runs in: one call gives the mean
+            # cost of this configuration's items, the next files them by it, the
+            # rebuild sorts (in natural order one warp per item took 436 us on the
+            # 128^3 workload instead of 305, and lost by that)
+            fn()
+            fn()
+            self.build_neighbors()
             torch.cuda.synchronize(self.dev)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()
