@@ -37,19 +37,17 @@ namespace {
 
 struct FwdArgs {
     const float *x, *y, *z, *t;
-    const uint32_t *tile_super, *tile_start, *cell_start, *stile0;
     const float4 *tile_lo, *tile_hi;
     const uint32_t *slist, *scnt;
     const float4 *kfwd;
-    const float4 *kbwd;      // adjoint records (c, r2), rows of R with log2(e) d_k^2
     const uint4 *order_rec;  // item records, heaviest class first (stable)
     uint8_t *item_class;     // cost class of each item, for the next order
     uint32_t *sched;         // mean cost of the last launch
     unsigned long long *sched_total;
     unsigned long long *adj_fix;    // fixed-point moments (fused adjoint)
     unsigned long long *adj_pairs;  // adjoint pair count (fused adjoint)
-    int64_t ntiles, nitems;
-    int scap, cps;
+    int64_t nitems;
+    int scap;
     float tau1, tau2;  // tau1 rounded down, tau2 rounded up to float: exact double decisions
     float *psi, *err;
     uint8_t *mask;
@@ -148,9 +146,9 @@ __device__ __forceinline__ void box_near_far_d2(float cx, float cy, float cz, fl
     far2 = support_d2(fminf(ax, bx), fminf(ay, by), fminf(az, bz));
 }
 
-// npairs staged kernel pairs from pair index pb against the lane's two
-// points.  NP: the lane's points that take part, of NT (an item of a sparse
-// super cell may have fewer tiles).  PARTIAL: the support only partly covers the item box, so each
+// npairs staged kernel pairs from pair index pb against the lane's points.
+// NP: those that take part, of NT (an item of a sparse super cell may have
+// fewer tiles).  PARTIAL: the support only partly covers the item box, so each
 // pair takes the exact Eq. 3-15-1 predicate (the operations of support_d2,
 // packed: fma(dz, dz, fma(dy, dy, fl(dx dx))) < r2).
 template <bool PARTIAL, int UNROLL, int NP, int NT>
@@ -457,9 +455,9 @@ __device__ __forceinline__ void forward_share(const FwdArgs &a, const ItemInfo &
 }
 
 // ---------------------------------------------------------------- fused adjoint
-// After an item's residuals are known, its points with E != 0 (at most 64,
-// in shared memory as x, y, z, E arrays: tile 0 from 0, tile 1 from 32, each
-// padded to an even count) are taken against the kernels that reached the
+// After an item's residuals are known, its points with E != 0 (at most 128 with
+// one warp per item, 64 with several; in shared memory in point order, padded to
+// an even count) are taken against the kernels that reached the
 // item box in the forward filter, kept if their support reaches the box of
 // those points: lanes are kernels, each lane loops over the points two at a
 // time (packed f32x2) and accumulates the ten moments of its kernel in the
@@ -515,15 +513,14 @@ __device__ __forceinline__ void f2_kadd(f2 &s, f2 &c, f2 v) {
 }
 
 // A batch of cnt <= 32 kernels from queue slot head: all nz points of the
-// item against each kernel (segs: 8 bits for each run of points, runs from
-// slots 0, 32, ...).  A short batch spreads each kernel over
+// item (nc) against each kernel.  A short batch spreads each kernel over
 // L = 2, 4 or 8 neighbouring lanes (cnt <= 16, 8, 4) that take every L-th
 // point pair; their moments are combined with xor shuffles within the group
 // (a fixed order for a given cnt) before the atomics, so short batches do
 // not leave most lanes idle.  KAHAN: compensated per-lane sums.
 template <bool KAHAN>
 __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *q, int head, int cnt,
-                                              const NzPoints &nz, uint32_t segs, int lane) {
+                                              const NzPoints &nz, int nc, int lane) {
     const int sh = cnt > 16 ? 0 : (cnt > 8 ? 1 : (cnt > 4 ? 2 : 3));
     const int L = 1 << sh, kl = lane >> sh, sub = lane & (L - 1);
     const bool act = kl < cnt;  // whole groups of L lanes are inactive together
@@ -537,56 +534,53 @@ __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *
     for (int r = 0; r < 10; ++r) acc[r] = 0ull;
 #pragma unroll
     for (int r = 0; r < (KAHAN ? 10 : 1); ++r) cmp[r] = 0ull;
-#pragma unroll 1
-    for (int base = 0; segs != 0u; base += kTile, segs >>= 8) {
-        const int cntp = act ? (int)((segs & 255u) + 1u) >> 1 : 0;
+    const int cntp = act ? (nc + 1) >> 1 : 0;
 #pragma unroll 4
-        for (int pp = sub; pp < cntp; pp += L) {
-            const int i = base + 2 * pp;
-            const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(&nz.v[i]);
-            const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(&nz.v[i + 1]);
-            const f2 px = wa.x, py = wa.y, pz = wb.x, pe = wb.y;
-            const f2 dx = f2_sub(px, cx), dy = f2_sub(py, cy), dz = f2_sub(pz, cz);
-            const f2 zz = f2_mul(dz, dz);
-            // q = Delta^T Q Delta (log2 units), the forward's operation order
-            const f2 ra = f2_fma(q13, dz, f2_fma(q12, dy, f2_mul(q11, dx)));
-            const f2 rb = f2_fma(q23, dz, f2_mul(q22, dy));
-            const f2 qv = f2_fma(q33, zz, f2_fma(dy, rb, f2_mul(dx, ra)));
-            float q0, q1;
-            f2_unpack(qv, q0, q1);
-            float e0 = ex2_approx(-q0), e1 = ex2_approx(-q1);
-            // Eq. 3-15-1, the operations of support_d2, packed
-            const f2 d2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
-            float d0, d1;
-            f2_unpack(d2, d0, d1);
-            const bool i0 = d0 < k0.w, i1 = d1 < k0.w;
-            e0 = i0 ? e0 : 0.f;
-            e1 = i1 ? e1 : 0.f;
-            const f2 sv = f2_mul(f2_pack(e0, e1), pe);
-            const f2 sx = f2_mul(sv, dx), sy = f2_mul(sv, dy), sz = f2_mul(sv, dz);
-            if (KAHAN) {
-                f2_kadd(acc[0], cmp[0], sv);
-                f2_kadd(acc[1], cmp[1], sx);
-                f2_kadd(acc[2], cmp[2], sy);
-                f2_kadd(acc[3], cmp[3], sz);
-                f2_kadd(acc[4], cmp[4], f2_mul(sx, dx));
-                f2_kadd(acc[5], cmp[5], f2_mul(sx, dy));
-                f2_kadd(acc[6], cmp[6], f2_mul(sx, dz));
-                f2_kadd(acc[7], cmp[7], f2_mul(sy, dy));
-                f2_kadd(acc[8], cmp[8], f2_mul(sy, dz));
-                f2_kadd(acc[9], cmp[9], f2_mul(sz, dz));
-            } else {
-                acc[0] = f2_add(acc[0], sv);
-                acc[1] = f2_add(acc[1], sx);
-                acc[2] = f2_add(acc[2], sy);
-                acc[3] = f2_add(acc[3], sz);
-                acc[4] = f2_fma(sx, dx, acc[4]);
-                acc[5] = f2_fma(sx, dy, acc[5]);
-                acc[6] = f2_fma(sx, dz, acc[6]);
-                acc[7] = f2_fma(sy, dy, acc[7]);
-                acc[8] = f2_fma(sy, dz, acc[8]);
-                acc[9] = f2_fma(sz, dz, acc[9]);
-            }
+    for (int pp = sub; pp < cntp; pp += L) {
+        const int i = 2 * pp;
+        const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(&nz.v[i]);
+        const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(&nz.v[i + 1]);
+        const f2 px = wa.x, py = wa.y, pz = wb.x, pe = wb.y;
+        const f2 dx = f2_sub(px, cx), dy = f2_sub(py, cy), dz = f2_sub(pz, cz);
+        const f2 zz = f2_mul(dz, dz);
+        // q = Delta^T Q Delta (log2 units), the forward's operation order
+        const f2 ra = f2_fma(q13, dz, f2_fma(q12, dy, f2_mul(q11, dx)));
+        const f2 rb = f2_fma(q23, dz, f2_mul(q22, dy));
+        const f2 qv = f2_fma(q33, zz, f2_fma(dy, rb, f2_mul(dx, ra)));
+        float q0, q1;
+        f2_unpack(qv, q0, q1);
+        float e0 = ex2_approx(-q0), e1 = ex2_approx(-q1);
+        // Eq. 3-15-1, the operations of support_d2, packed
+        const f2 d2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+        float d0, d1;
+        f2_unpack(d2, d0, d1);
+        const bool i0 = d0 < k0.w, i1 = d1 < k0.w;
+        e0 = i0 ? e0 : 0.f;
+        e1 = i1 ? e1 : 0.f;
+        const f2 sv = f2_mul(f2_pack(e0, e1), pe);
+        const f2 sx = f2_mul(sv, dx), sy = f2_mul(sv, dy), sz = f2_mul(sv, dz);
+        if (KAHAN) {
+            f2_kadd(acc[0], cmp[0], sv);
+            f2_kadd(acc[1], cmp[1], sx);
+            f2_kadd(acc[2], cmp[2], sy);
+            f2_kadd(acc[3], cmp[3], sz);
+            f2_kadd(acc[4], cmp[4], f2_mul(sx, dx));
+            f2_kadd(acc[5], cmp[5], f2_mul(sx, dy));
+            f2_kadd(acc[6], cmp[6], f2_mul(sx, dz));
+            f2_kadd(acc[7], cmp[7], f2_mul(sy, dy));
+            f2_kadd(acc[8], cmp[8], f2_mul(sy, dz));
+            f2_kadd(acc[9], cmp[9], f2_mul(sz, dz));
+        } else {
+            acc[0] = f2_add(acc[0], sv);
+            acc[1] = f2_add(acc[1], sx);
+            acc[2] = f2_add(acc[2], sy);
+            acc[3] = f2_add(acc[3], sz);
+            acc[4] = f2_fma(sx, dx, acc[4]);
+            acc[5] = f2_fma(sx, dy, acc[5]);
+            acc[6] = f2_fma(sx, dz, acc[6]);
+            acc[7] = f2_fma(sy, dy, acc[7]);
+            acc[8] = f2_fma(sy, dz, acc[8]);
+            acc[9] = f2_fma(sz, dz, acc[9]);
         }
     }
     float v[10];
@@ -635,9 +629,8 @@ __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *
 // it, 2462 us with it here, 2533 us with it there.
 template <int G, bool KAHAN>
 __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &it, int w, const NzPoints &nz,
-                                              uint32_t segs, int nc, float4 lo, float4 hi, const uint32_t *touch,
-                                              int ntouch, int tcap, float emax, uint32_t *q, int lane,
-                                              uint32_t &cost) {
+                                              int nc, float4 lo, float4 hi, const uint32_t *touch, int ntouch, int tcap,
+                                              float emax, uint32_t *q, int lane, uint32_t &cost) {
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t *lst = a.slist + (size_t)it.sup * a.scap;
     const bool listed = ntouch <= tcap;
@@ -662,13 +655,13 @@ __device__ __forceinline__ void adjoint_share(const FwdArgs &a, const ItemInfo &
         nk += __popc(bal);
         __syncwarp();
         if (qn >= 32) {
-            adjoint_batch<KAHAN>(a, q, head, 32, nz, segs, lane);
+            adjoint_batch<KAHAN>(a, q, head, 32, nz, nc, lane);
             head = (head + 32) & (kQueue - 1);
             qn -= 32;
             __syncwarp();
         }
     }
-    if (qn > 0) adjoint_batch<KAHAN>(a, q, head, qn, nz, segs, lane);
+    if (qn > 0) adjoint_batch<KAHAN>(a, q, head, qn, nz, nc, lane);
     __syncwarp();
     cost += (uint32_t)(nk * nc) / 4u + 32u;
 }
@@ -820,10 +813,10 @@ __device__ __forceinline__ void sched_finish_batch(const FwdBatch &b, int lane) 
 
 // Persistent blocks take work items, heaviest first: block b the b-th, then
 // from a global counter (claims past the grid's first items).
-// The G warps of a block share an item (its candidate list split by 32-entry
-// chunks); their partial sums are combined in warp order, so Psi does not
-// depend on timing.  G = 1 when there are enough items to balance the warps,
-// 2 or 4 for small problems.
+// The G warps of a block share an item (equal runs of its candidate list);
+// their partial sums are combined in warp order, so Psi does not depend on
+// timing.  G = 1 when there are enough items to balance the warps, 2 or 4 for
+// small problems.
 // ADJ: 0 forward only, 1 with the fused adjoint, 2 with the fused adjoint
 // and compensated (Kahan) per-item moment sums.
 // BATCH: the items of a batch of fields (b); otherwise of one field (a1).
@@ -967,7 +960,7 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
                 __syncwarp();
                 if ((nc & 1) && lane == 0) nz_pad(nzs, nc);
                 __syncwarp();
-                adjoint_share<1, (ADJ > 1)>(a, it, 0, nzs, (uint32_t)nc, nc, lo, hi, touch[0], ntouch, kTouchW,
+                adjoint_share<1, (ADJ > 1)>(a, it, 0, nzs, nc, lo, hi, touch[0], ntouch, kTouchW,
                                             __uint_as_float(ebits), adjq, lane, cost);
                 __syncwarp();
             }
@@ -1046,7 +1039,7 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
                 __syncwarp();
                 if ((nc & 1) && lane == 0) nz_pad(nzs, nc);
                 __syncwarp();
-                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, (uint32_t)nc, nc, lo, hi, touch[ADJ ? warp : 0], ntouch,
+                adjoint_share<G, (ADJ > 1)>(a, it, warp, nzs, nc, lo, hi, touch[ADJ ? warp : 0], ntouch,
                                             kTouchW, __uint_as_float(ebits), adjq, lane, cost);
                 __syncwarp();
             }
@@ -1262,27 +1255,20 @@ bool make_args(const serbf_points *pts, const serbf_params *prm, const serbf_con
     a.y = pts->y;
     a.z = pts->z;
     a.t = pts->t;
-    a.tile_super = ws->tile_super;
-    a.stile0 = ws->super_tile0;
     const ItemSet &items = items_of(ws, G);
     a.order_rec = items.order;
     a.item_class = items.cls;
     a.sched = items.sched;
     a.sched_total = items.total;
     a.nitems = items.n;
-    a.tile_start = ws->tile_start;
-    a.cell_start = ws->cell_start;
     a.tile_lo = ws->tile_lo;
     a.tile_hi = ws->tile_hi;
     a.slist = ws->sup_list;
     a.scnt = ws->sup_cnt;
     a.kfwd = ws->kfwd;
-    a.kbwd = ws->kbwd;
     a.adj_fix = ws->adj_fix;
     a.adj_pairs = ws->adj_pairs;
-    a.ntiles = ws->ntiles;
     a.scap = ws->sz.super_cap;
-    a.cps = ws->sf * ws->sf * ws->sf;
     // float thresholds that give the same decisions as comparing in double:
     // t <= tau1 iff t <= (largest float <= tau1), t >= tau2 iff t >= (smallest float >= tau2)
     a.tau1 = (float)cfg->tau1;
