@@ -304,8 +304,9 @@ int serbf_marching_tets(const float *f, const int32_t dims[3], const float origi
 int serbf_sample_surface(const float *tri, int64_t ntri, const double *u, int64_t ns, float *pts, float *nrm,
                          int64_t *scratch, void *stream);
 
-/* Sec. 4 metrics between two sampled surfaces (point-to-point, nearest
- * point by brute force, ties to the lowest index): out (host) = {HD, CD, CS}
+/* Sec. 4 metrics between two sampled surfaces (point-to-point, nearest point
+ * as comparing all pairs gives it, ties to the lowest index; large sets are
+ * searched through a grid of cells): out (host) = {HD, CD, CS}
  * with HD = max(max_a d(a, B), max_b d(b, A)), CD = mean_a d(a, B) / 2 +
  * mean_b d(b, A) / 2, CS = the same means of |n . n_nearest|.  scratch:
  * 2 (na + nb) + 6 doubles (device).  SYNCHRONISES. */

@@ -19,8 +19,9 @@
 // halve that rest per point and widen the item box (a few more pairs outside
 // the support); with one warp per item that gains (9.4 M points 2118 -> 2070 us,
 // 16 fields 844 -> 704 us for the fused call), with several it does not (64^3 +
-// 32^3 points 59 -> 72 us with four), so they keep two.  The tiles follow from
-// the warps alone, so a field in a batch gets the bits it gets by itself.
+// 32^3 points 60 -> 64 us with four, 128^3 292 -> 318 with two), so they keep two.
+// The tiles follow from the warps alone, so a field in a batch gets the bits it
+// gets by itself.
 //
 // Persistent blocks take items heaviest first (order from the costs measured
 // by the previous launch) to keep the tail short; the warps of a block split
@@ -534,7 +535,10 @@ __device__ __forceinline__ void adjoint_batch(const FwdArgs &a, const uint32_t *
     for (int r = 0; r < 10; ++r) acc[r] = 0ull;
 #pragma unroll
     for (int r = 0; r < (KAHAN ? 10 : 1); ++r) cmp[r] = 0ull;
-    const int cntp = act ? (nc + 1) >> 1 : 0;
+    // nc <= 128: with its range in sight the loop counts in fewer instructions
+    // (9.4 M points 2066 -> 2046 us an epoch)
+    static_assert(kNz < 256, "residual points of an item");
+    const int cntp = act ? (int)(((uint32_t)nc & 255u) + 1u) >> 1 : 0;
 #pragma unroll 4
     for (int pp = sub; pp < cntp; pp += L) {
         const int i = 2 * pp;
@@ -1372,11 +1376,15 @@ namespace serbf {
 // (an item in the middle of the kernels whose points all carry residuals costs
 // five times the mean and more), so a launch with few items per warp waits for
 // its heaviest ones; more warps per item shorten that tail and cost issue slots
-// for barriers and short batches.  Measured crossings on a 152-SM part, fused
-// call in us with 1 / 2 / 4 warps: 8.0 k items (80^3) 149 / 106 / 93, 14.6 k
-// (97^3, compensated) 251 / 181 / 172, 20.8 k (110^3) 243 / 194 / 226, 32.8 k
-// (128^3) 318 / 292 / 364, 147 k (9.4 M points) 2118 / 2280 / 2801; 8 warps were
-// within 3 % of 4 below 2 k items and slower above.
+// for barriers and short batches.  Measured on a 152-SM part with the items that
+// each takes (four tiles with one warp, two with several), items2 and the fused
+// call in us with 1 / 2 / 4 warps: 0.5 k (32^3) 36 / 35 / 35, 4.6 k (64^3 + 32^3)
+// 104 / 66 / 65, 14.3 k (97^3) 163 / 148 / 159 (compensated 233 / 196 / 198), 27 k
+// (120^3) 275 / 251 / 297, 33 k (128^3) 337 / 309 / 365, 43 k (140^3) 384 / 385 /
+// 458, 53 k (150^3) 467 / 476 / 568, 64 k 548 / 574 / 688, 125 k 963 / 1062 / 1270,
+// 147 k (9.4 M points of a band) 1671 / 1817 / 2109; a batch of 16 fields, 82 k in
+// all, 552 / 718 / 979 an epoch.  8 warps are within 8 % of 4 up to 0.5 k items and
+// slower above.
 int forward_warps(int64_t items2, int sm_count, int fixed) {
     if (fixed == 1 || fixed == 2 || fixed == 4 || fixed == 8) return fixed;
     const int64_t resident = 20 * (int64_t)sm_count;  // warps in flight

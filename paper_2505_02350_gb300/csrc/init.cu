@@ -26,7 +26,9 @@ namespace {
 
 constexpr int kBatch = 1024;      // points settled per round, one per thread
 constexpr int kRounds = 8;        // rounds between two looks at the state
-constexpr uint32_t kSparse = 384; // new centres in a round after which the next one looks for conflicts first
+// New centres in a round after which the next one looks for conflicts first
+// (40^3 / 64^3 / 80^3 points: 410 / 890 / 1107 us, never looking 826 / 2122 / 3150).
+constexpr uint32_t kSparse = 384;
 
 // Where the walk stands (device; ws->counters + 8).
 struct Walk {

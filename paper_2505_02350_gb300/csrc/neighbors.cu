@@ -716,9 +716,6 @@ bool rebuild_three_level(int levels, int64_t ncoarse, int cap) {
 }  // namespace
 
 namespace serbf {
-}  // namespace serbf
-
-namespace serbf {
 
 size_t rebuild_args_size() { return sizeof(RebuildArgs); }
 
