@@ -224,48 +224,58 @@ __global__ void __launch_bounds__(256) k_cells(const uint32_t *keys, int64_t n, 
 // One block: tiles and forward work items (both sets) of every super cell,
 // numbered in super-cell order; out = {tiles, items of set 0, of set 1, most
 // tiles in one super cell}.  Also clears the forward's scheduling state (no
-// mean cost yet: the first forward files every item in the same class).
+// mean cost yet: the first forward files every item in the same class).  The
+// block's passes over the super cells bound it, one barrier each and the next
+// pass's loads ahead (three scans of three barriers each took 163 us for 97 336).
 __global__ void __launch_bounds__(1024) k_supers(const uint32_t *cell_start, int nsuper, int cps, uint32_t *stile,
                                                  ItemSet two, ItemSet four, uint32_t *out, uint32_t *arrived) {
     pdl_wait();
     pdl_trigger();
-    __shared__ uint32_t tmp[33];
+    __shared__ uint32_t s_sum[2][3][32];  // per warp: tiles and items of either set
     __shared__ uint32_t s_max;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_max = 0u;
     if (threadIdx.x < 4) two.sched[threadIdx.x] = four.sched[threadIdx.x] = 0u;
     if (threadIdx.x < 2) two.total[threadIdx.x] = four.total[threadIdx.x] = 0ull;
-    __syncthreads();
-    uint32_t t0 = 0, i0 = 0, q0 = 0, mx = 0;
-    for (int s0 = 0; s0 < nsuper; s0 += blockDim.x) {
+    auto tiles_of = [&](int s) {
+        if (s >= nsuper) return 0u;
+        return (cell_start[(int64_t)(s + 1) * cps] - cell_start[(int64_t)s * cps] + kTile - 1) / kTile;
+    };
+    uint32_t base[3] = {0u, 0u, 0u}, mx = 0, next = tiles_of(threadIdx.x);
+    int buf = 0;
+    for (int s0 = 0; s0 < nsuper; s0 += blockDim.x, buf ^= 1) {
         const int s = s0 + threadIdx.x;
-        uint32_t nt = 0;
-        if (s < nsuper) {
-            const uint32_t b = cell_start[(int64_t)s * cps], e = cell_start[(int64_t)(s + 1) * cps];
-            nt = (e - b + kTile - 1) / kTile;
-        }
+        const uint32_t nt = next, v[3] = {nt, (nt + 1) / 2, (nt + kMostTiles - 1) / kMostTiles};
+        next = tiles_of(s + blockDim.x);
         mx = max(mx, nt);
-        uint32_t ts, is, qs;
-        const uint32_t to = block_exscan(nt, tmp, &ts), io = block_exscan((nt + 1) / 2, tmp, &is);
-        const uint32_t qo = block_exscan((nt + kMostTiles - 1) / kMostTiles, tmp, &qs);
-        if (s < nsuper) {
-            stile[s] = t0 + to;
-            two.super0[s] = i0 + io;
-            four.super0[s] = q0 + qo;
+        uint32_t inc[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            inc[k] = warp_iscan(v[k]);
+            if (lane == 31) s_sum[buf][k][warp] = inc[k];
         }
-        t0 += ts;
-        i0 += is;
-        q0 += qs;
+        __syncthreads();  // the other buffer is written next: one barrier a pass
+        uint32_t at[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t own = s_sum[buf][k][lane], to = warp_iscan(own);
+            at[k] = base[k] + __shfl_sync(0xffffffffu, to - own, warp) + inc[k] - v[k];
+            base[k] += __shfl_sync(0xffffffffu, to, 31);
+        }
+        if (s < nsuper) {
+            stile[s] = at[0];
+            two.super0[s] = at[1];
+            four.super0[s] = at[2];
+        }
     }
+    __syncthreads();
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_max, mx);
     __syncthreads();
     if (threadIdx.x == 0) {
-        stile[nsuper] = t0;
-        two.super0[nsuper] = i0;
-        four.super0[nsuper] = q0;
-        out[0] = t0;
-        out[1] = i0;
-        out[2] = q0;
+        stile[nsuper] = out[0] = base[0];
+        two.super0[nsuper] = out[1] = base[1];
+        four.super0[nsuper] = out[2] = base[2];
         out[3] = s_max;
         *arrived = 0u;
     }
@@ -292,11 +302,16 @@ __device__ __forceinline__ void grow(float4 &lo, float4 &hi, float4 a, float4 b)
 }
 
 constexpr int kTilesThreads = 512;
+constexpr int kTilesWarps = kTilesThreads / 32;
+// Points per super cell up to which k_tiles takes many super cells a block: a
+// block each costs a barrier, a fence and a counter, whatever it holds.  Whole
+// binning, us, a block each / sixteen a block: 6000 points in 68 921 super cells
+// 495 / 229, 300 000 in 97 336 965 / 352 (150 000 of them in one 908 / 478), 16,
+// 32, 64 and 128 points in each of 27 000 386 / 209, 391 / 218, 460 / 293, 593 /
+// 473, of 1000 105 / 97, 110 / 103, 129 / 118, 132 / 139.
+constexpr int64_t kSparsePoints = 64;
+constexpr uint32_t kAloneTiles = 4;  // a warp of the sparse form takes so many tiles by itself
 
-// One block per super cell, a warp per tile: the tile's start and bounding
-// box, the work items (the first forward takes them in this order), the
-// super cell's box (empty: +inf / -inf).  The last block unites the super
-// cells' boxes (the box of every binned point).
 __device__ __forceinline__ void put_item(const ItemSet &set, int s, uint32_t t, uint32_t k, uint32_t ps, uint32_t left,
                                          uint32_t tiles) {
     if (k % tiles) return;
@@ -307,19 +322,13 @@ __device__ __forceinline__ void put_item(const ItemSet &set, int s, uint32_t t, 
     set.cls[it] = 3;  // one class for all until a forward has measured them
 }
 
-__global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    constexpr int NW = kTilesThreads / 32;
-    __shared__ float4 wlo[NW], whi[NW];
-    __shared__ bool s_last;
-    const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Tiles first, first + step, ... of super cell s, a warp at a time: their
+// starts, boxes and work items; grows the box lo .. hi by theirs.
+__device__ __forceinline__ void super_tiles(const TilesArgs &a, int s, uint32_t first, uint32_t step, int lane, float4 &lo,
+                                            float4 &hi) {
     const uint32_t t0 = a.stile0[s], t1 = a.stile0[s + 1];
     const uint32_t p0 = a.cell_start[(int64_t)s * a.cps], pe = a.cell_start[(int64_t)(s + 1) * a.cps];
-    const float4 none_lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
-    const float4 none_hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
-    float4 lo = none_lo, hi = none_hi;
-    for (uint32_t t = t0 + warp; t < t1; t += NW) {
+    for (uint32_t t = t0 + first; t < t1; t += step) {
         const uint32_t ps = p0 + (t - t0) * kTile, i = ps + lane;
         const bool v = i < pe;
         float4 tl, th;
@@ -334,15 +343,61 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
             put_item(a.four, s, t, t - t0, ps, pe - ps, (uint32_t)kMostTiles);
         }
     }
-    if (lane == 0) {
-        wlo[warp] = lo;
-        whi[warp] = hi;
+}
+
+// One block per super cell, a warp per tile: the tile's start and bounding
+// box, the work items (the first forward takes them in this order), the
+// super cell's box (empty: +inf / -inf).  The last block unites the super
+// cells' boxes (the box of every binned point).
+// SPARSE: a block takes kTilesWarps super cells, a warp each, and all its warps
+// together those of more than kAloneTiles tiles.
+template <bool SPARSE>
+__global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    constexpr int NW = kTilesWarps;
+    __shared__ float4 wlo[NW], whi[NW];
+    __shared__ bool s_many[NW];
+    __shared__ bool s_last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s0 = SPARSE ? blockIdx.x * NW : blockIdx.x, ns = SPARSE ? min(NW, a.nsuper - s0) : 1;
+    const float4 none_lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    const float4 none_hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+    float4 lo = none_lo, hi = none_hi;
+    if (SPARSE) {
+        bool many = false;
+        if (warp < ns) {
+            const int s = s0 + warp;
+            many = a.stile0[s + 1] - a.stile0[s] > kAloneTiles;
+            if (!many) {
+                super_tiles(a, s, 0u, 1u, lane, lo, hi);
+                if (lane == 0) {
+                    a.slo[s] = lo;
+                    a.shi[s] = hi;
+                }
+            }
+        }
+        if (lane == 0) s_many[warp] = many;
+        __syncthreads();
     }
-    __syncthreads();
+    for (int c = 0; c < ns; ++c) {
+        if (SPARSE && !s_many[c]) continue;
+        lo = none_lo;
+        hi = none_hi;
+        super_tiles(a, s0 + c, (uint32_t)warp, (uint32_t)NW, lane, lo, hi);
+        if (lane == 0) {
+            wlo[warp] = lo;
+            whi[warp] = hi;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < NW; ++w) grow(lo, hi, wlo[w], whi[w]);
+            a.slo[s0 + c] = lo;
+            a.shi[s0 + c] = hi;
+        }
+        if (SPARSE) __syncthreads();
+    }
     if (threadIdx.x == 0) {
-        for (int w = 1; w < NW; ++w) grow(lo, hi, wlo[w], whi[w]);
-        a.slo[s] = lo;
-        a.shi[s] = hi;
         __threadfence();
         s_last = atomicAdd(a.arrived, 1u) == gridDim.x - 1;
     }
@@ -480,7 +535,9 @@ extern "C" int serbf_bin_points(const float *x, const float *y, const float *z, 
     uint32_t *out = ws->counters + 12;
     launch_pdl(k_supers, dim3(1), dim3(1024), 0, s, ws->cell_start, (int)nsuper, cps, ws->super_tile0, ws->items[0],
                ws->items[1], out, ws->counters);
-    launch_pdl(k_tiles, dim3((unsigned)nsuper), dim3(kTilesThreads), 0, s,
+    const bool sparse = n <= kSparsePoints * nsuper;
+    launch_pdl(sparse ? k_tiles<true> : k_tiles<false>, dim3((unsigned)(sparse ? (nsuper + kTilesWarps - 1) / kTilesWarps : nsuper)),
+               dim3(kTilesThreads), 0, s,
                TilesArgs{ws->cell_start, ws->super_tile0, (int)nsuper, cps, ws->tile_super, ws->tile_start, ws->items[0],
                          ws->items[1], xb, yb, zb, ws->tile_lo, ws->tile_hi, ws->sup_lo, ws->sup_hi, ws->field_box,
                          ws->counters});
