@@ -1069,10 +1069,13 @@ __device__ __forceinline__ void forward_loop(const FwdArgs &a1, const FwdBatch &
 
 // Resident warps per SM (the register budget): 16 with one warp per item (four
 // points per lane: 126 registers; 20 warps spill 80 bytes and took 2158 us
-// instead of 2085 for 9.4 M points) and with four, 20 for the fused variant
-// with two, 24 with eight and for the forward alone with two or four; measured
-// on the 128^3 and 256^3 fields, other bounds were slower.
-#define SERBF_FWD_BOUNDS(G, ADJ) __launch_bounds__(G * 32, (G == 1 ? 16 : (G == 8 ? 24 : (ADJ ? (G == 4 ? 16 : 20) : 24))) / G)
+// instead of 2085 for 9.4 M points), with four, and with two and compensated
+// sums (20 spill 116 bytes: 64^3 + 32^3 points 75 us, now 68, 97^3 214 and 193,
+// 128^3 374 and 345); 20 for the fused variant with two, 24 with eight (16 spill
+// nothing and took 450 us instead of 430 on 128^3) and for the forward alone with
+// two or four; measured on the 128^3 and 256^3 fields, other bounds were slower.
+#define SERBF_FWD_BOUNDS(G, ADJ) \
+    __launch_bounds__(G * 32, (G == 1 ? 16 : (G == 8 ? 24 : (ADJ ? (G == 4 || ADJ == 2 ? 16 : 20) : 24))) / G)
 
 template <int G, int ADJ>
 __global__ void SERBF_FWD_BOUNDS(G, ADJ) k_forward(FwdArgs a) {
