@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "warps_rule.cuh"
 
 namespace serbf {
 size_t fwd_args_size();
@@ -101,15 +102,15 @@ int serbf_batch_init(serbf_batch *b, const serbf_field *fields, int32_t nfields,
     int64_t total = 0, fin_blocks = 1, chunks = 0;
     int lvl1 = 1, parents = 0, step_nb = 1, sm = 0;
     const int kahan = fields[0].cfg ? fields[0].cfg->kahan : 0;
-    int64_t items2 = 0;
+    int64_t items4 = 0;
     for (int f = 0; f < nfields; ++f) {
         const serbf_field &F = fields[f];
         if (!F.cfg || !F.ws || F.ws->magic != kMagic || !F.ws->binned || F.cfg->kahan != kahan) return SERBF_EINVAL;
-        items2 += F.ws->items[0].n;
+        items4 += F.ws->items[1].n;
         F.ws->unmeasured = 0;  // the batched epochs measure
         sm = F.ws->sm_count;
     }
-    const int G = forward_warps(items2, sm, fwd_warps);
+    const int G = forward_warps(items4, sm, fwd_warps);
     for (int f = 0; f < nfields; ++f) {
         const serbf_field &F = fields[f];
         serbf_params prm = F.prm;

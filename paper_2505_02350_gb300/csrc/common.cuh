@@ -560,9 +560,7 @@ __device__ __forceinline__ KBox kernel_box(float cx, float cy, float cz, float r
 
 // ---------------------------------------------------------------- cross-unit launchers
 namespace serbf {
-// Warps per forward work item for a field (or batch) of items2 items of two
-// tiles, unless fixed (1, 2, 4 or 8) says so; and the item set they take.
-int forward_warps(int64_t items2, int sm_count, int fixed);
+// The item set that so many warps per item take.
 inline const ItemSet &items_of(const serbf_workspace *ws, int warps) { return ws->items[warps == 1 ? 1 : 0]; }
 constexpr int kScanTile = 4096;  // elements of a tile of launch_exscan_i64
 // Exclusive scan in place, a[n] = total; tiles: n / kScanTile + 1 words of scratch.

@@ -31,6 +31,7 @@
 
 #include "common.cuh"
 #include "form_bound.cuh"
+#include "warps_rule.cuh"
 
 using namespace serbf;
 
@@ -1319,7 +1320,7 @@ int forward_impl(const serbf_points *pts, const serbf_params *prm, const serbf_c
     FinishArgs f;
     int64_t nb = 1;
     if (!cfg || !ws || ws->magic != kMagic) return SERBF_EINVAL;
-    const int G = forward_warps(ws->items[0].n, ws->sm_count, cfg->fwd_warps);
+    const int G = forward_warps(ws->items[1].n, ws->sm_count, cfg->fwd_warps);
     if (!make_args(pts, prm, cfg, psi, err, mask, grad, stats, ws, G, a, f, nb)) return SERBF_EINVAL;
     const bool adj = grad != nullptr;
     cudaStream_t s = (cudaStream_t)stream;
@@ -1374,25 +1375,6 @@ int launch_forward_batch(const FwdBatch &b, int64_t nitems, int sm_count, cudaSt
 }  // namespace
 
 namespace serbf {
-
-// Warps per item, unless the configuration fixes it.  Items differ in cost
-// (an item in the middle of the kernels whose points all carry residuals costs
-// five times the mean and more), so a launch with few items per warp waits for
-// its heaviest ones; more warps per item shorten that tail and cost issue slots
-// for barriers and short batches.  Measured on a 152-SM part with the items that
-// each takes (four tiles with one warp, two with several), items2 and the fused
-// call in us with 1 / 2 / 4 warps: 0.5 k (32^3) 36 / 35 / 35, 4.6 k (64^3 + 32^3)
-// 104 / 66 / 65, 14.3 k (97^3) 163 / 148 / 159 (compensated 233 / 196 / 198), 27 k
-// (120^3) 275 / 251 / 297, 33 k (128^3) 337 / 309 / 365, 43 k (140^3) 384 / 385 /
-// 458, 53 k (150^3) 467 / 476 / 568, 64 k 548 / 574 / 688, 125 k 963 / 1062 / 1270,
-// 147 k (9.4 M points of a band) 1671 / 1817 / 2109; a batch of 16 fields, 82 k in
-// all, 552 / 718 / 979 an epoch.  8 warps are within 8 % of 4 up to 0.5 k items and
-// slower above.
-int forward_warps(int64_t items2, int sm_count, int fixed) {
-    if (fixed == 1 || fixed == 2 || fixed == 4 || fixed == 8) return fixed;
-    const int64_t resident = 20 * (int64_t)sm_count;  // warps in flight
-    return items2 >= 16 * resident ? 1 : (items2 >= 6 * resident ? 2 : 4);
-}
 
 size_t fwd_args_size() { return sizeof(FwdArgs); }
 size_t finish_args_size() { return sizeof(FinishArgs); }

@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "order_rule.cuh"
+#include "warps_rule.cuh"
 
 using namespace serbf;
 
@@ -801,7 +802,7 @@ extern "C" int serbf_build_neighbors(const serbf_points *pts, const serbf_params
     // to order when no forward has measured since the binning, whose order is
     // there already -- except under capture, where the graph will be replayed
     // after forwards that do measure.
-    const ItemSet &items = items_of(ws, forward_warps(ws->items[0].n, ws->sm_count, cfg->fwd_warps));
+    const ItemSet &items = items_of(ws, forward_warps(ws->items[1].n, ws->sm_count, cfg->fwd_warps));
     bool measured = !ws->unmeasured;
     if (!measured) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
