@@ -39,8 +39,8 @@ ADJ_INSTR_PER_PAIR = 32  # minimum FP32-pipe instructions of one adjoint pair (r
 # split and super-cell size, valid only for the library version it was taken
 # with (any other version, workload, split or size reports null)
 TRAFFIC_BYTES = {
-    ("serbf 0.4.0 (sm_103a)", "c4", 1, 2): 183_976_448 + 61_820_416 + 9_995_264,
-    ("serbf 0.4.0 (sm_103a)", "c3", 2, 2): 39_483_904 + 312_576 + 2_309_120,
+    ("serbf 0.4.2 (sm_103a)", "c4", 1, 2): 184_003_840 + 61_719_808 + 9_995_264,
+    ("serbf 0.4.2 (sm_103a)", "c3", 2, 2): 39_480_832 + 305_664 + 2_310_144,
 }
 DEFAULT_STEPS = {"c1": 3000, "c2": 3000, "c3": 500, "c4": 200, "c5": 2000}
 WORKLOADS = {

@@ -240,7 +240,7 @@ int launch_exscan_i64(int64_t *a, int64_t n, int64_t *tiles, cudaStream_t s) {
 
 extern "C" {
 
-const char *serbf_version(void) { return "serbf 0.4.1 (sm_103a)"; }
+const char *serbf_version(void) { return "serbf 0.4.2 (sm_103a)"; }
 
 const char *serbf_status_string(int code) {
     switch (code) {
