@@ -306,10 +306,12 @@ constexpr int kTilesWarps = kTilesThreads / 32;
 // Points per super cell up to which k_tiles takes many super cells a block: a
 // block each costs a barrier, a fence and a counter, whatever it holds.  Whole
 // binning, us, a block each / sixteen a block: 6000 points in 68 921 super cells
-// 495 / 229, 300 000 in 97 336 965 / 352 (150 000 of them in one 908 / 478), 16,
+// 495 / 219, 300 000 in 97 336 965 / 344 (150 000 of them in one 908 / 463), 16,
 // 32, 64 and 128 points in each of 27 000 386 / 209, 391 / 218, 460 / 293, 593 /
-// 473, of 1000 105 / 97, 110 / 103, 129 / 118, 132 / 139.
+// 473, of 1000 105 / 97, 110 / 103, 129 / 118, 132 / 139.  While a block each fits
+// the chip at once (512 super cells, those of a thin band: 93 / 101) it is taken.
 constexpr int64_t kSparsePoints = 64;
+constexpr int64_t kWaveBlocks = 2048 / kTilesThreads;  // blocks of k_tiles on an SM
 constexpr uint32_t kAloneTiles = 4;  // a warp of the sparse form takes so many tiles by itself
 
 __device__ __forceinline__ void put_item(const ItemSet &set, int s, uint32_t t, uint32_t k, uint32_t ps, uint32_t left,
@@ -360,14 +362,16 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
     __shared__ bool s_many[NW];
     __shared__ bool s_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s0 = SPARSE ? blockIdx.x * NW : blockIdx.x, ns = SPARSE ? min(NW, a.nsuper - s0) : 1;
+    // a block's super cells lie a grid apart, as dense ones lie side by side (a
+    // thin band in 512 of them: 118 us with neighbours in a block, 108 so)
+    const int s0 = blockIdx.x, ds = (int)gridDim.x, ns = SPARSE ? min(NW, (a.nsuper - s0 + ds - 1) / ds) : 1;
     const float4 none_lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
     const float4 none_hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
     float4 lo = none_lo, hi = none_hi;
     if (SPARSE) {
         bool many = false;
         if (warp < ns) {
-            const int s = s0 + warp;
+            const int s = s0 + warp * ds;
             many = a.stile0[s + 1] - a.stile0[s] > kAloneTiles;
             if (!many) {
                 super_tiles(a, s, 0u, 1u, lane, lo, hi);
@@ -384,7 +388,7 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
         if (SPARSE && !s_many[c]) continue;
         lo = none_lo;
         hi = none_hi;
-        super_tiles(a, s0 + c, (uint32_t)warp, (uint32_t)NW, lane, lo, hi);
+        super_tiles(a, s0 + c * ds, (uint32_t)warp, (uint32_t)NW, lane, lo, hi);
         if (lane == 0) {
             wlo[warp] = lo;
             whi[warp] = hi;
@@ -392,8 +396,8 @@ __global__ void __launch_bounds__(kTilesThreads) k_tiles(TilesArgs a) {
         __syncthreads();
         if (threadIdx.x == 0) {
             for (int w = 1; w < NW; ++w) grow(lo, hi, wlo[w], whi[w]);
-            a.slo[s0 + c] = lo;
-            a.shi[s0 + c] = hi;
+            a.slo[s0 + c * ds] = lo;
+            a.shi[s0 + c * ds] = hi;
         }
         if (SPARSE) __syncthreads();
     }
@@ -535,7 +539,7 @@ extern "C" int serbf_bin_points(const float *x, const float *y, const float *z, 
     uint32_t *out = ws->counters + 12;
     launch_pdl(k_supers, dim3(1), dim3(1024), 0, s, ws->cell_start, (int)nsuper, cps, ws->super_tile0, ws->items[0],
                ws->items[1], out, ws->counters);
-    const bool sparse = n <= kSparsePoints * nsuper;
+    const bool sparse = n <= kSparsePoints * nsuper && nsuper > kWaveBlocks * (int64_t)ws->sm_count;
     launch_pdl(sparse ? k_tiles<true> : k_tiles<false>, dim3((unsigned)(sparse ? (nsuper + kTilesWarps - 1) / kTilesWarps : nsuper)),
                dim3(kTilesThreads), 0, s,
                TilesArgs{ws->cell_start, ws->super_tile0, (int)nsuper, cps, ws->tile_super, ws->tile_start, ws->items[0],

@@ -10,9 +10,11 @@ from gpu_util import torch_cuda
 
 pytestmark = pytest.mark.gpu
 
-# supers per axis at super factor 1: 1331 = 83 x 16 + 3 super cells, and 8
+# supers per axis at super factor 1: 1331 = 83 x 16 + 3 super cells, 8, and 512 and
+# 729 to either side of the number that is on the chip at once
 @pytest.mark.parametrize("cells,n,dense", [(11, 64 * 1331, 0), (11, 64 * 1331 + 1, 0), (11, 3000, 128), (11, 3000, 129),
-                                           (11, 6000, 5000), (2, 64 * 8, 0), (2, 40, 0), (11, 1, 0)])
+                                           (11, 6000, 5000), (8, 4000, 2000), (9, 4000, 2000), (9, 64 * 729, 0),
+                                           (2, 64 * 8, 0), (2, 40, 0), (11, 1, 0)])
 def test_sparse_super_cells(orc, cells, n, dense):
     torch = torch_cuda()
     from paper_2505_02350_gb300 import _native as N, build, field
